@@ -384,7 +384,7 @@ def work(case):
 def _omega(z):
     """The solution of w + log w = z."""
     zc = z.clamp_min(-600.0)
-    w = torch.where(zc < -1, torch.exp(zc.clamp_max(0)), torch.where(zc > 3, zc - torch.log(zc.clamp_min(1)), 1 + (zc - 1) / 2))
+    w = torch.where(zc < -1, torch.exp(zc.clamp_max(0)), torch.where(zc > 3, zc - torch.log(zc.clamp_min(1)), 1 + (zc - 1) / 2 + (zc - 1) ** 2 / 16))
     w = torch.where(zc < -1, w * torch.exp(-w), w)
     for _ in range(8):
         w = w * (1 + zc - torch.log(w)) / (1 + w)
