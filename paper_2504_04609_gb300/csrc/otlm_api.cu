@@ -520,6 +520,9 @@ int otlm_tune_ragged(otlm_handle h, int batch, const int* n, const int* k, const
     }
     return good && cudaEventElapsedTime(ms_out, e0, e1) == cudaSuccess;
   };
+  // a later choice has to be faster by more than two timings of one choice differ, so that equal
+  // choices (the rows per thread of problems whose applies run by block expansions) do not alternate
+  constexpr float TUNE_MARGIN = 0.92f;
   float best_total = 1e30f;
   int best_v = h->rg_variant;
   unsigned char best_rows[otlm::RAGGED_BUCKETS] = {};
@@ -540,7 +543,7 @@ int otlm_tune_ragged(otlm_handle h, int batch, const int* n, const int* k, const
         h->rg_rows[b] = (unsigned char)l;
         float ms = 0.f;
         ok = time_bucket(v, by_bucket[b], &ms);
-        if (ok && ms < best_b) {
+        if (ok && ms < TUNE_MARGIN * best_b) {
           best_b = ms;
           best_l = l;
         }
@@ -548,7 +551,7 @@ int otlm_tune_ragged(otlm_handle h, int batch, const int* n, const int* k, const
       rows[b] = (unsigned char)best_l;
       total += best_b;
     }
-    if (ok && total < best_total) {
+    if (ok && total < TUNE_MARGIN * best_total) {
       best_total = total;
       best_v = v;
       std::memcpy(best_rows, rows, sizeof(rows));

@@ -6,15 +6,22 @@
 // decreasing n_p^2, i.e. largest work first), so the 256x spread in work per problem balances
 // across the SMs without any host round trip.
 //
-// The kernel apply inside a CTA: thread t owns R consecutive rows (R even, a compile-time
+// The kernel apply inside a CTA: block expansions (expansion.cuh) wherever the problem's grid
+// qualifies, which is decided per problem in the kernel from the grid itself.  Other grids (unsorted,
+// or with fewer than 32 bins per 1.47 kernel widths) are summed term by term: thread t owns R consecutive rows (R even, a compile-time
 // constant picked from n_p); with its own centre c_t (the middle of its rows) the exponent
 // in_j - m_i - (xt_i - xt_j)^2 becomes FFMA(2 di, dj, h_j) - q_i with h_j = in_j - dj^2 formed
 // once per column and q_i = m_i + di^2 once per row; rows are processed in packed pairs
 // (fma/add.f32x2).  Shift: the previous sums (later iterations), the diagonal term (first
 // iteration), or an exact max pass when any sum leaves [2^-60, 2^60].
+//
+// 800 problems, n 256..4096, k 8..128, eps 2e-3..5e-2, 20 iterations: 45.4 ms with every apply term by
+// term and row-at-a-time dictionary passes (exponent unit and load latency), 6.6 ms with expansions
+// and passes that keep 16 loads of D in flight per warp.  What is left is D: 0.6 MB per problem, read
+// twice per iteration, mostly from DRAM.
 #pragma once
 
-#include "kernels.cuh"
+#include "expansion.cuh"
 
 namespace otlm {
 
@@ -57,7 +64,11 @@ template <int NT>
 struct RaggedSmem {
   // offsets (floats) into dynamic shared memory for a problem of n_max bins, k_max atoms
   static __host__ __device__ size_t floats(int n_max, int k_max) {
-    return 6 * (size_t)n_max + 2 * (size_t)k_max + (NT / 32) * (size_t)k_max + 64;
+    return state(n_max, k_max) + ex_scratch_floats(EX_NB * EX_NB);
+  }
+  // everything but the expansion's scratch, rounded up to 16 bytes
+  static __host__ __device__ size_t state(int n_max, int k_max) {
+    return (6 * (size_t)n_max + 2 * (size_t)k_max + (NT / 32) * (size_t)k_max + 64 + 3) / 4 * 4;
   }
 };
 
@@ -179,6 +190,125 @@ __device__ void ragged_apply(const float* xt, const float* in, float* out, int n
 
 __device__ __forceinline__ float block_sum_f(float v, float* red) { return block_sum<float>(v, red); }
 
+// The same apply by block expansions (expansion.cuh), for grids that qualify.  Out of line: one copy
+// serves the source and target applies of every rows-per-thread variant.
+template <int NT>
+__device__ __noinline__ void ragged_apply_ex(const float* xt, const float* in, float* out, int n, ExPlan pl, float* scr,
+                                             float* ratio) {
+  using P = Prec<float>;
+  ex_apply<NT>(in, xt, n, pl, 0, pl.nb, scr, [&](int i, float base, float sum, float di2) {
+    if (ratio) ratio[i] = sum > 0.f ? sum * P::exp2((base - out[i]) - di2) : 0.f;
+    out[i] = sum > 0.f ? base + (P::log2(sum) - di2) : P::ninf();
+  });
+  __syncthreads();
+}
+
+// The two dictionary passes of an iteration.  D [n][k] is read from L2 or HBM twice per iteration
+// and is what an iteration waits for, so a warp keeps U rows x KQ loads of 32 columns in flight
+// (U KQ = 16); lanes are columns, warps take rows.
+//   ragged_dtr: red_k[warp][j] = sum over the warp's rows of D_ij r_i
+//   ragged_dw : row_done(i, sum_j D_ij w_j), once per row by one lane; U rows are summed over the
+//               lanes by one transposing butterfly
+template <int NT, int KQ>
+__device__ __forceinline__ void ragged_dtr(const float* D, const float* r, int n, int k, int k_max, float* red_k) {
+  constexpr int NW = NT / 32, U = KQ >= 8 ? 2 : (KQ >= 4 ? 4 : 8);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float acc[KQ];
+#pragma unroll
+  for (int q = 0; q < KQ; ++q) acc[q] = 0.f;
+  for (int i0 = warp * U; i0 < n; i0 += NW * U) {
+    float d[U][KQ];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int q = 0; q < KQ; ++q) {
+        const int j = lane + 32 * q;
+        d[u][q] = (i0 + u < n && j < k) ? D[(size_t)(i0 + u) * k + j] : 0.f;
+      }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const float ri = i0 + u < n ? r[i0 + u] : 0.f;
+#pragma unroll
+      for (int q = 0; q < KQ; ++q) acc[q] = fmaf(d[u][q], ri, acc[q]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < KQ; ++q)
+    if (lane + 32 * q < k) red_k[warp * k_max + lane + 32 * q] = acc[q];
+}
+template <int NT, int KQ, class F>
+__device__ __forceinline__ void ragged_dw(const float* D, const float* W, int n, int k, F row_done) {
+  constexpr int NW = NT / 32, U = KQ >= 8 ? 2 : (KQ >= 4 ? 4 : 8);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float w[KQ];
+#pragma unroll
+  for (int q = 0; q < KQ; ++q) w[q] = lane + 32 * q < k ? W[lane + 32 * q] : 0.f;
+  for (int i0 = warp * U; i0 < n; i0 += NW * U) {
+    float s[U];
+    {
+      float d[U][KQ];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int q = 0; q < KQ; ++q) {
+          const int j = lane + 32 * q;
+          d[u][q] = (i0 + u < n && j < k) ? D[(size_t)(i0 + u) * k + j] : 0.f;
+        }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        s[u] = 0.f;
+#pragma unroll
+        for (int q = 0; q < KQ; ++q) s[u] = fmaf(d[u][q], w[q], s[u]);
+      }
+    }
+    // transpose while the values outnumber one: lanes with bit o set keep the upper half
+#pragma unroll
+    for (int o = 16, c = U; o > 0; o >>= 1) {
+      if (c > 1) {
+        c >>= 1;
+#pragma unroll
+        for (int u = 0; u < c; ++u) {
+          const bool up = lane & o;
+          const float keep = up ? s[u + c] : s[u], give = up ? s[u] : s[u + c];
+          s[u] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+      } else {
+        s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+      }
+    }
+    // lane l holds the total of row i0 + (the top log2 U bits of l)
+    const int i = i0 + lane / (32 / U);
+    if (lane % (32 / U) == 0 && i < n) row_done(i, s[0]);
+  }
+}
+
+// D^T r by columns per lane, and S = D w with F2 = log2 S - LA2 (F2 not null) and the thread's share
+// of the mass.  Out of line: shared by every rows-per-thread variant.
+template <int NT>
+__device__ __noinline__ void ragged_dtr_any(const float* D, const float* r, int n, int k, int k_max, float* red_k) {
+  if (k <= 32) ragged_dtr<NT, 1>(D, r, n, k, k_max, red_k);
+  else if (k <= 64) ragged_dtr<NT, 2>(D, r, n, k, k_max, red_k);
+  else if (k <= 128) ragged_dtr<NT, 4>(D, r, n, k, k_max, red_k);
+  else ragged_dtr<NT, 8>(D, r, n, k, k_max, red_k);
+}
+template <int NT>
+__device__ __noinline__ float ragged_dw_any(const float* D, const float* W, const float* LA2, float* S, float* F2, int n,
+                                            int k) {
+  using P = Prec<float>;
+  float mass = 0.f;
+  auto row_done = [&](int i, float s) {
+    if (s < P::tiny()) s = 0.f;
+    S[i] = s;
+    if (F2) F2[i] = s > 0.f ? P::log2(s) - LA2[i] : P::ninf();
+    mass += s;
+  };
+  if (k <= 32) ragged_dw<NT, 1>(D, W, n, k, row_done);
+  else if (k <= 64) ragged_dw<NT, 2>(D, W, n, k, row_done);
+  else if (k <= 128) ragged_dw<NT, 4>(D, W, n, k, row_done);
+  else ragged_dw<NT, 8>(D, W, n, k, row_done);
+  return mass;
+}
+
 template <int NT, int R>
 __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
   using P = Prec<float>;
@@ -191,7 +321,7 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
   const bool valid = n >= 2 && n <= A.n_max && k >= 1 && k <= A.k_max && (n + NT - 1) / NT <= R && on >= 0 &&
                      on + n <= A.tot_n && oD >= 0 && oD + (long long)n * k <= A.tot_D && ok >= 0 &&
                      ok + k <= A.tot_k &&
-                     6 * (long long)A.n_max + 2 * A.k_max + (NT / 32) * A.k_max + 64 <= A.smem_floats;
+                     (long long)RaggedSmem<NT>::floats(A.n_max, A.k_max) <= A.smem_floats;
   if (!__syncthreads_and(valid)) {
     if (threadIdx.x == 0) {
       A.iters[p] = 0;
@@ -211,6 +341,8 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
   float* xcol = W + A.k_max;
   float* red_k = xcol + A.k_max;  // [NT/32][k_max]
   float* red = red_k + (NT / 32) * A.k_max;  // 32 floats + scalars
+  float* scr = sm + RaggedSmem<NT>::state(A.n_max, A.k_max);  // the expansion's scratch
+  __shared__ ExPlan plan_s;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int NW = NT / 32;
 
@@ -220,14 +352,17 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
     G2[i] = A.g_in ? A.g_in[on + i] / eps_ln2 : 0.f;
   }
   for (int j = tid; j < k; j += NT) W[j] = A.w[ok + j];
-  // column sums x_j: warps over rows, lanes over columns
-  for (int j0 = 0; j0 < k; j0 += 32) {
-    float part = 0.f;
-    const int j = j0 + lane;
-    if (j < k)
-      for (int i = warp; i < n; i += NW) part += D[(size_t)i * k + j];
-    if (j < k) red_k[warp * A.k_max + j] = part;
+  __syncthreads();
+  const bool sorted = ex_sorted(xt, n);
+  if (warp == 0) {
+    const ExPlan pl = ex_plan_warp(xt, n, sorted);
+    if (lane == 0) plan_s = pl;
   }
+  // column sums x_j (F2 holds ones until the first iteration)
+  for (int i = tid; i < n; i += NT) F2[i] = 1.f;
+  __syncthreads();
+  const ExPlan plan = plan_s;
+  ragged_dtr_any<NT>(D, F2, n, k, A.k_max, red_k);
   __syncthreads();
   for (int j = tid; j < k; j += NT) {
     float s = 0.f;
@@ -236,23 +371,11 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
   }
   __syncthreads();
 
-  // S = D w (warp per row, lanes over atoms), mass
+  // S = D w, F2 = log2 S - LA2 (when asked for) and the mass
   auto source_step = [&](bool write_f2) -> float {
-    float mass = 0.f;
-    for (int i = warp; i < n; i += NW) {
-      float s = 0.f;
-      for (int j = lane; j < k; j += 32) s = fmaf(D[(size_t)i * k + j], W[j], s);
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (s < P::tiny()) s = 0.f;
-      if (lane == 0) {
-        S[i] = s;
-        if (write_f2) F2[i] = s > 0.f ? P::log2(s) - LA2[i] : P::ninf();
-      }
-      mass += s;  // identical in every lane
-    }
+    const float mass = ragged_dw_any<NT>(D, W, LA2, S, write_f2 ? F2 : nullptr, n, k);
     __syncthreads();
-    float tot = lane == 0 ? mass : 0.f;
-    return block_sum_f(tot, red);
+    return block_sum_f(mass, red);
   };
   float mass = source_step(false);
 
@@ -261,7 +384,8 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
   int st = ST_MAX_ITER;
   for (;; ++it) {
     // source apply; F2 doubles as the ratio buffer a_new / a_old
-    ragged_apply<NT, R>(xt, G2, LA2, n, it > 0, F2);
+    if (plan.nb) ragged_apply_ex<NT>(xt, G2, LA2, n, plan, scr, it > 0 ? F2 : nullptr);
+    else ragged_apply<NT, R>(xt, G2, LA2, n, it > 0, F2);
     if (it > 0) {
       float part = 0.f;
       for (int i = tid; i < n; i += NT)
@@ -275,28 +399,25 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
     // MM step: nu_j = log w_j + (ln2 / x_j) sum_i D_ij (LA2_i - log2 S_i), then S = D w; mm_steps
     // times with the same LA2, the last one also writing F2
     for (int m = 0; m < A.mm_steps; ++m) {
-      for (int j0 = 0; j0 < k; j0 += 32) {
-        const int j = j0 + lane;
-        float part = 0.f;
-        if (j < k)
-          for (int i = warp; i < n; i += NW) {
-            const float s = S[i];
-            if (s > 0.f) part = fmaf(D[(size_t)i * k + j], LA2[i] - P::log2(s), part);
-          }
-        if (j < k) red_k[warp * A.k_max + j] = part;
-      }
+      for (int i = tid; i < n; i += NT) F2[i] = S[i] > 0.f ? LA2[i] - P::log2(S[i]) : 0.f;  // the log ratios
+      __syncthreads();
+      ragged_dtr_any<NT>(D, F2, n, k, A.k_max, red_k);
       __syncthreads();
       for (int j = tid; j < k; j += NT) {
         float sum = 0.f;
         for (int w8 = 0; w8 < NW; ++w8) sum += red_k[w8 * A.k_max + j];
         const float xj = xcol[j];
-        const float nu = P::log(W[j]) + sum * float(kLn2) / xj;
+        const float dl = sum * float(kLn2) / xj;
+        const float nu = P::log(W[j]) + dl;
         const float shift = (A.penalty == PEN_L1 || A.penalty == PEN_ELASTIC) ? A.alpha / (eps * xj) : 0.f;
         float wn;
         if (A.penalty == PEN_L2SQ || A.penalty == PEN_ELASTIC) {
           const float c = (A.penalty == PEN_ELASTIC ? A.beta : A.alpha) / (eps * xj);
           wn = wright_omega<float>(P::log(c) + nu - shift) / c;
-        } else wn = P::exp(nu - shift);
+        } else {
+          // w e^(dl - shift): no rounding of log w, whose size is that of the weights' whole range
+          wn = fabsf(dl - shift) < 60.f ? W[j] * P::exp(dl - shift) : P::exp(nu - shift);
+        }
         W[j] = wn;
       }
       __syncthreads();
@@ -304,7 +425,8 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
       if (m + 1 == A.mm_steps) mass = m_mass;
     }
     // target apply and the datafit step (Table 1) in log2 units
-    ragged_apply<NT, R>(xt, F2, LB2, n, it > 0, nullptr);
+    if (plan.nb) ragged_apply_ex<NT>(xt, F2, LB2, n, plan, scr, nullptr);
+    else ragged_apply<NT, R>(xt, F2, LB2, n, it > 0, nullptr);
     const float kl_coef = A.lam / (eps + A.lam), tv_bound = A.lam / eps_ln2, loe = A.lam / eps;
     const float lloe = logf(A.lam / eps);
     for (int j = tid; j < n; j += NT) {
