@@ -1,0 +1,542 @@
+// Batched kernel applies by block expansions (expansion.cuh) for a batch sharing one squared-distance
+// grid, with the iteration's row work fused in: one CTA reads a problem's row once, applies K and
+// finishes the rows it computed.
+//
+//   source apply (EXA_SOURCE): in = G2;  out = LA2, the source-marginal violation and the stopping
+//     decision of the previous iteration (stop_decision), and on tensor-core handles the MM log
+//     ratios r = LA2 - log2 S as the TF32 hi/lo operand of D^T r
+//   target apply (EXA_TARGET): in = F2 = log2 S - LA2 (formed on the fly);  out = LB2, the datafit
+//     step G2 (Table 1) and, on tensor-core handles, the mass sum S
+//
+// The row is staged in shared memory (n <= EXA_MAX_N).  Small batches split a problem's row blocks
+// over `parts` CTAs (grid.y), each forming the moments of its own row blocks from the whole row; the
+// last CTA of a problem to finish adds the violation's partial sums in a fixed order and decides.
+// A grid that does not qualify for expansions (ExPlan.nb = 0, known on the device only) is summed
+// term by term here too.
+#pragma once
+
+#include "expansion.cuh"
+
+namespace otlm {
+
+
+inline size_t exa_smem_bytes(int n, int warps) {
+  return 4 * ((size_t)(n + 3) / 4 * 4 + ex_scratch_floats(warps));
+}
+
+static __global__ void __launch_bounds__(1024) ex_plan_kernel(const float* xt, int n, ExPlan* plan) {
+  const bool sorted = ex_sorted(xt, n);
+  if (threadIdx.x < 32) {
+    const ExPlan pl = ex_plan_warp(xt, n, sorted);
+    if (threadIdx.x == 0) *plan = pl;
+  }
+}
+
+// Rows [i0, i1) term by term, four rows per warp at a time, lanes over the columns.  Shift: the
+// previous sum `old` where there is one; rows whose sum leaves [2^-60, 2^60] are redone around their
+// largest term.  row(...) as in ex_apply, with the shift in place of the integer base.
+template <int T, class Load, class Row>
+__device__ __forceinline__ void ex_direct(const float* in_s, const float* xt, int n, int i0, int i1, const float* old,
+                                          Load load, Row row) {
+  using P = Prec<float>;
+  constexpr int Q = 4;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int r0 = i0 + warp * Q; r0 < i1; r0 += T * Q) {
+    float xi[Q], m[Q], sum[Q];
+    bool ok = old != nullptr;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int i = min(r0 + q, i1 - 1);
+      xi[q] = xt[i];
+      m[q] = old ? old[i] : 0.f;
+      ok &= isfinite(m[q]);
+    }
+    auto sweep = [&] {
+#pragma unroll
+      for (int q = 0; q < Q; ++q) sum[q] = 0.f;
+      for (int j = lane; j < n; j += 32) {
+        const float v = in_s[j], xj = xt[j];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+          const float d = xi[q] - xj;
+          sum[q] += P::exp2(fmaf(-d, d, v - m[q]));
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < Q; ++q)
+        for (int o = 16; o > 0; o >>= 1) sum[q] += __shfl_xor_sync(0xffffffffu, sum[q], o);
+    };
+    if (ok) {
+      sweep();
+#pragma unroll
+      for (int q = 0; q < Q; ++q) ok &= sum[q] >= 0x1p-60f && sum[q] <= 0x1p60f;
+    }
+    if (!ok) {  // the totals, and so this branch, are the same in every lane
+#pragma unroll
+      for (int q = 0; q < Q; ++q) m[q] = -CUDART_INF_F;
+      for (int j = lane; j < n; j += 32) {
+        const float v = in_s[j], xj = xt[j];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+          const float d = xi[q] - xj;
+          m[q] = fmaxf(m[q], fmaf(-d, d, v));
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        for (int o = 16; o > 0; o >>= 1) m[q] = fmaxf(m[q], __shfl_xor_sync(0xffffffffu, m[q], o));
+        if (!(m[q] > -CUDART_INF_F)) m[q] = 0.f;  // every term vanishes
+      }
+      sweep();
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+      if (lane == q && r0 + q < i1) row(r0 + q, load(r0 + q), m[q], sum[q], 0.f);
+  }
+}
+
+// Datafit step (Table 1) in log2 units; FAST: the Wright omega of the tensor-core path.
+template <bool FAST>
+__device__ __forceinline__ float exa_datafit(const ExArgs& A, float v, float yv) {
+  using P = Prec<float>;
+  switch (A.datafit) {
+    case DF_BALANCED: return P::log2(yv) - v;
+    case DF_KL: return A.kl_coef * (P::log2(yv) - v);
+    case DF_TV: return fminf(fmaxf(P::log2(yv) - v, -A.tv_bound), A.tv_bound);
+    default: {
+      const bool pois = A.datafit == DF_POISSON;
+      if (pois && !(yv > 0.f)) return -A.tv_bound;
+      const float l2c = pois ? A.log_lam_over_eps * float(kLog2e) + P::log2(yv) : 0.f;
+      const float z = pois ? (l2c - v) * float(kLn2) + A.lam_over_eps
+                           : A.log_lam_over_eps + v * float(kLn2) + A.lam_over_eps * yv;
+      const float om = FAST ? wright_omega_fast(z) : wright_omega<float>(z);
+      return pois ? l2c - P::log2(om) - v : (A.lam_over_eps * yv - om) * float(kLog2e);
+    }
+  }
+}
+
+__device__ __forceinline__ float exa_tf32(float x) {
+  uint32_t r;
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+  return __uint_as_float(r);
+}
+
+// Sum over the CTA's T warps, the same in every thread.
+template <int T>
+__device__ __forceinline__ float exa_sum(float v, float* red) {
+  if constexpr (T == 1) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  } else {
+    return block_sum(v, red);
+  }
+}
+
+template <int EPI, bool TC, int T>
+__global__ void __launch_bounds__(32 * T) ex_apply_kernel(ExArgs A) {
+  using P = Prec<float>;
+  constexpr int NT = 32 * T;
+  extern __shared__ __align__(16) float smem[];
+  __shared__ float red[32];
+  __shared__ int last_s;
+  const int slot = blockIdx.x, prt = blockIdx.y, parts = gridDim.y;
+  if (slot >= *A.n_active) return;
+  const int p = A.active[slot], n = A.n, tid = threadIdx.x;
+  if (A.done[p]) return;
+  const size_t o = (size_t)p * n;
+  float* in_s = smem;
+  float* scr = smem + (n + 3) / 4 * 4;
+  const ExPlan pl = *A.plan;
+  float mass = 0.f;
+  if (EPI == EXA_SOURCE) {
+#pragma unroll 8
+    for (int j = tid; j < n; j += NT) in_s[j] = A.G2[o + j];
+  } else {
+#pragma unroll 8
+    for (int j = tid; j < n; j += NT) {
+      const float s = A.S[o + j], la = A.LA2[o + j];
+      in_s[j] = s > 0.f ? P::log2(s) - la : P::ninf();
+      mass += s;
+    }
+    if (TC) {
+      mass = exa_sum<T>(mass, red);
+      if (tid == 0 && prt == 0) A.mass[p] = mass;
+    }
+  }
+  float part = 0.f;
+  struct Pre { float a, b; };  // source: S, LA2 of the previous iteration; target: y
+  auto load = [&](int i) {
+    Pre q{0.f, 0.f};
+    if (EPI == EXA_SOURCE) {
+      if (A.check || TC) q.a = A.S[o + i];
+      if (A.check) q.b = A.LA2[o + i];
+    } else q.a = A.y[o + i];
+    return q;
+  };
+  auto row = [&](int i, Pre pre, float base, float sum, float di2) {
+    const size_t idx = o + i;
+    const float v = sum > 0.f ? base + (P::log2(sum) - di2) : P::ninf();
+    if (EPI == EXA_SOURCE) {
+      const float s = pre.a;
+      if (A.check && s > 0.f) {
+        // s |a_new / a_old - 1|; the difference of the references is exact, so the ratio keeps FP32
+        // relative precision; a jump beyond 2^64 is taken in log form, capped at 2^120
+        const float dl = (base - pre.b) - di2;
+        if (!(sum > 0.f)) part += s;
+        else if (dl + P::log2(sum) > 64.f) part += P::exp2(fminf(P::log2(s) + (dl + P::log2(sum)), 120.f));
+        else part += s * fabsf(sum * P::exp2(dl) - 1.f);
+      }
+      A.LA2[idx] = v;
+      if (TC) {
+        const float r = s > 0.f ? v - P::log2(s) : 0.f, hi = exa_tf32(r);
+        const size_t ro = (size_t)slot * A.ld + i;
+        A.Rhi[ro] = hi;
+        A.Rlo[ro] = exa_tf32(r - hi);
+      }
+    } else {
+      A.LB2[idx] = v;
+      A.G2[idx] = exa_datafit<TC>(A, v, pre.a);
+    }
+  };
+  if (pl.nb > 0) {
+    const int I0 = pl.nb * prt / parts, I1 = pl.nb * (prt + 1) / parts;
+    if (I1 > I0) ex_apply<T>(in_s, A.xt, n, pl, I0, I1, scr, load, row);
+  } else {
+    ex_sync<T>();
+    const float* old = A.it > 0 ? (EPI == EXA_SOURCE ? A.LA2 : A.LB2) + o : nullptr;
+    const int i0 = (int)((long long)n * prt / parts), i1 = (int)((long long)n * (prt + 1) / parts);
+    ex_direct<T>(in_s, A.xt, n, i0, i1, old, load, row);
+  }
+  if (EPI == EXA_TARGET || !A.check) return;
+
+  // ---- violation of the previous iteration's plan and the stopping decision --------------------
+  part = exa_sum<T>(part, red);
+  if (parts > 1) {
+    if (tid == 0) {
+      A.part[o + prt] = part;
+      __threadfence();
+      last_s = atomicAdd(A.count + p, 1) == parts - 1;
+    }
+    __syncthreads();
+    if (!last_s) return;
+    __threadfence();
+    if (tid == 0) {
+      part = 0.f;
+      for (int q = 0; q < parts; ++q) part += __ldcg(A.part + o + q);
+      A.count[p] = 0;
+    }
+  }
+  float dw = 0.f;
+  if (TC) {  // weight change of the previous iteration's update
+    float num = 0.f, den = 0.f;
+    for (int j = tid; j < A.k; j += NT) {
+      const float wv = A.W[(size_t)p * A.k + j];
+      num += fabsf(wv - A.Wprev[(size_t)p * A.k + j]);
+      den += fabsf(wv);
+    }
+    num = exa_sum<T>(num, red);
+    den = exa_sum<T>(den, red);
+    dw = num / den;
+  }
+  if (tid == 0) {
+    const float e = part / A.mass[p];
+    if (TC) A.dw[p] = dw;
+    else dw = A.dw[p];
+    A.err[p] = e;
+    const int st = stop_decision<float>(e, dw, A.tol, A.dw_tol, false, false, A.it, A.max_iter);
+    if (st >= 0) {
+      A.status[p] = st;
+      A.iters[p] = A.it;
+      A.done[p] = 1;
+    }
+  }
+}
+
+// Log ratios r = LA2 - log2 S as the TF32 operand, for the MM steps after an iteration's first.
+static __global__ void __launch_bounds__(256) ex_ratio_kernel(ExArgs A) {
+  const int slot = blockIdx.x;
+  if (slot >= *A.n_active) return;
+  const size_t o = (size_t)A.active[slot] * A.n, ro = (size_t)slot * A.ld;
+  for (int i = threadIdx.x; i < A.n; i += 256) {
+    const float s = A.S[o + i];
+    const float r = s > 0.f ? A.LA2[o + i] - Prec<float>::log2(s) : 0.f, hi = exa_tf32(r);
+    A.Rhi[ro + i] = hi;
+    A.Rlo[ro + i] = exa_tf32(r - hi);
+  }
+}
+
+// CTAs per problem: enough for two per SM, at most one per possible row block (and one per bin: the
+// partial violations live in the problem's own row).
+inline int exa_parts(int batch, int n, int sms) {
+  const int want = (2 * sms + batch - 1) / batch;
+  return want < 1 ? 1 : (want > EX_NB ? (EX_NB < n ? EX_NB : n) : (want < n ? want : n));
+}
+
+template <int EPI, bool TC, int T>
+static inline cudaError_t launch_ex_cfg(const ExArgs& a, int batch, int parts, cudaStream_t stream) {
+  const size_t smem = exa_smem_bytes(a.n, T);
+  if (smem > 48 * 1024) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(ex_apply_kernel<EPI, TC, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  ex_apply_kernel<EPI, TC, T><<<dim3(batch, parts), 32 * T, smem, stream>>>(a);
+  return cudaGetLastError();
+}
+#ifndef EXA_T1
+#define EXA_T1 4
+#endif
+template <int EPI, bool TC>
+static inline cudaError_t launch_ex_apply(const ExArgs& a, int batch, int sms, cudaStream_t stream) {
+  if (batch >= 4 * sms && a.n <= 8192) return launch_ex_cfg<EPI, TC, EXA_T1>(a, batch, 1, stream);
+  return launch_ex_cfg<EPI, TC, 8>(a, batch, exa_parts(batch, a.n, sms), stream);
+}
+
+// ---- MM step and source step of a batch sharing the dictionary (FP32) ---------------------------
+// One CTA takes PB problems through an iteration's weight update: NU = D^T r with r = LA2 - log2 S,
+// Table 2's update, S = D w, mm_steps times with the same LA2.  Against one CTA per problem, each
+// entry of D that is read from L2 serves PB problems, and the multiply-adds run on packed pairs of
+// problems.  Arithmetic is FP32 throughout, as in mm_kernel.
+//   phase A: a chunk of 256 rows' log ratios is staged as [row][problem]; warps take rows, lanes
+//            columns; the eight warps' sums are added in order
+//   phase C: threads take rows (Dt is read coalesced along rows), the weights are broadcast
+constexpr int MMB_NT = 256, MMB_CHUNK = 256;
+
+template <int PB, int KQ>
+struct MmbSmem {
+  static constexpr int KP = 32 * KQ;
+  static constexpr int RS = MMB_CHUNK * PB;                     // staged ratios
+  static constexpr int RED = 8 * KP * (PB < 4 ? PB : 4);        // warps' sums of up to 4 problems
+  static constexpr int U = RS > RED ? RS : RED;
+  static constexpr size_t bytes = 4 * (size_t)(U + 3 * KP * PB);  // + weights [k][PB] (new), starting weights, NU
+};
+
+template <int PB, int KQ>
+__global__ void __launch_bounds__(MMB_NT) mm_batch_kernel(MMBArgs A) {
+  using P = Prec<float>;
+  using SM = MmbSmem<PB, KQ>;
+  constexpr int KP = SM::KP, H = PB > 1 ? PB / 2 : 1, G = PB < 4 ? PB : 4;
+  extern __shared__ __align__(16) float smem[];
+  float* rs = smem;               // [MMB_CHUNK][PB], then the warps' sums
+  float* w_s = smem + SM::U;      // [KP][PB]
+  float* w0_s = w_s + KP * PB;
+  float* nu_s = w0_s + KP * PB;   // [PB][KP]
+  __shared__ float red[32];
+  __shared__ int p_s[PB];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = A.n, k = A.k;
+  const int na = *A.n_active, slot0 = blockIdx.x * PB;
+  if (slot0 >= na) return;
+  if (tid < PB) {
+    const int p = slot0 + tid < na ? A.active[slot0 + tid] : -1;
+    p_s[tid] = (p >= 0 && !A.done[p]) ? p : -1;
+  }
+  __syncthreads();
+  bool any = false;
+#pragma unroll
+  for (int q = 0; q < PB; ++q) any |= p_s[q] >= 0;
+  if (!any) return;
+  for (int e = tid; e < k * PB; e += MMB_NT) {
+    const int q = e / k, j = e - q * k, p = p_s[q];
+    const float w = p >= 0 ? A.W[(size_t)p * k + j] : 1.f;
+    w_s[j * PB + q] = w;
+    w0_s[j * PB + q] = w;
+  }
+  for (int m = 0; m < A.mm_steps; ++m) {
+    // ---- phase A ----
+    uint64_t acc[H][KQ];
+#pragma unroll
+    for (int h = 0; h < H; ++h)
+#pragma unroll
+      for (int q = 0; q < KQ; ++q) acc[h][q] = 0ull;
+    for (int c0 = 0; c0 < n; c0 += MMB_CHUNK) {
+      __syncthreads();
+      {
+        const int i = c0 + tid;  // one row of the chunk per thread
+        float s[PB], la[PB];
+#pragma unroll
+        for (int q = 0; q < PB; ++q) {
+          const int p = p_s[q];
+          const bool in = i < n && p >= 0;
+          s[q] = in ? A.S[(size_t)p * n + i] : 0.f;
+          la[q] = in ? A.LA2[(size_t)p * n + i] : 0.f;
+        }
+#pragma unroll
+        for (int q = 0; q < PB; ++q) rs[tid * PB + q] = s[q] > 0.f ? la[q] - P::log2(s[q]) : 0.f;
+      }
+      __syncthreads();
+      const int cnt = min(MMB_CHUNK, n - c0);
+      constexpr int U = KQ >= 8 ? 2 : (KQ >= 4 ? 4 : 8);
+      for (int r0 = warp * U; r0 < cnt; r0 += 8 * U) {
+        float d[U][KQ];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int q = 0; q < KQ; ++q) {
+            const int j = lane + 32 * q;
+            d[u][q] = (r0 + u < cnt && j < k) ? A.D[(size_t)(c0 + r0 + u) * k + j] : 0.f;
+          }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const float* rr = rs + (r0 + u) * PB;  // rows past cnt were staged as 0
+          uint64_t r2[H];
+          if constexpr (PB >= 4) {
+#pragma unroll
+            for (int h = 0; h < H; h += 2) {
+              const float4 v = *reinterpret_cast<const float4*>(rr + 2 * h);
+              r2[h] = f2_pack(v.x, v.y);
+              r2[h + 1] = f2_pack(v.z, v.w);
+            }
+          } else if constexpr (PB == 2) r2[0] = f2_pack(rr[0], rr[1]);
+          else r2[0] = f2_pack(rr[0], 0.f);
+#pragma unroll
+          for (int q = 0; q < KQ; ++q) {
+            const uint64_t d2 = f2_pack(d[u][q], d[u][q]);
+#pragma unroll
+            for (int h = 0; h < H; ++h) acc[h][q] = f2_fma(d2, r2[h], acc[h][q]);
+          }
+        }
+      }
+    }
+    // the warps' sums, up to four problems at a time
+#pragma unroll
+    for (int g = 0; g < PB; g += G) {
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < KQ; ++q)
+#pragma unroll
+        for (int h = 0; h < (G + 1) / 2; ++h) {
+          float a, b;
+          f2_unpack(acc[g / 2 + h][q], a, b);
+          rs[(warp * G + 2 * h) * KP + lane + 32 * q] = a;
+          if (G > 1) rs[(warp * G + 2 * h + 1) * KP + lane + 32 * q] = b;
+        }
+      __syncthreads();
+      for (int e = tid; e < G * KP; e += MMB_NT) {
+        float sum = 0.f;
+#pragma unroll
+        for (int w8 = 0; w8 < 8; ++w8) sum += rs[w8 * G * KP + e];
+        nu_s[g * KP + e] = sum;
+      }
+    }
+    __syncthreads();
+    // ---- phase B: penalty update (Table 2), as mm_kernel ----
+    for (int e = tid; e < k * PB; e += MMB_NT) {
+      const int q = e / k, j = e - q * k, p = p_s[q];
+      if (p < 0) continue;
+      const float xj = A.xcol[j], wold = w_s[j * PB + q];
+      const float nu = P::log(wold) + nu_s[q * KP + j] * float(kLn2) / xj;
+      const float shift = (A.penalty == PEN_L1 || A.penalty == PEN_ELASTIC) ? A.alpha / (A.eps * xj) : 0.f;
+      float wn;
+      if (A.penalty == PEN_L2SQ || A.penalty == PEN_ELASTIC) {
+        const float c = (A.penalty == PEN_ELASTIC ? A.beta : A.alpha) / (A.eps * xj);
+        wn = wright_omega<float>(P::log(c) + nu - shift) / c;
+      } else wn = P::exp(nu - shift);
+      w_s[j * PB + q] = wn;
+      if (m + 1 == A.mm_steps) A.W[(size_t)p * k + j] = wn;
+    }
+    __syncthreads();
+    // ---- phase C: S = D w ----
+    constexpr int IPT = PB >= 16 ? 2 : 4;  // rows per thread
+    float mass[PB];
+#pragma unroll
+    for (int q = 0; q < PB; ++q) mass[q] = 0.f;
+    for (int c0 = 0; c0 < n; c0 += MMB_NT * IPT) {
+      uint64_t s2[IPT][H];
+#pragma unroll
+      for (int t = 0; t < IPT; ++t)
+#pragma unroll
+        for (int h = 0; h < H; ++h) s2[t][h] = 0ull;
+#pragma unroll 4
+      for (int j = 0; j < k; ++j) {
+        float d[IPT];
+#pragma unroll
+        for (int t = 0; t < IPT; ++t) {
+          const int i = c0 + t * MMB_NT + tid;
+          d[t] = i < n ? A.Dt[(size_t)j * n + i] : 0.f;
+        }
+        const float* ww = w_s + j * PB;
+        uint64_t w2[H];
+        if constexpr (PB >= 4) {
+#pragma unroll
+          for (int h = 0; h < H; h += 2) {
+            const float4 v = *reinterpret_cast<const float4*>(ww + 2 * h);
+            w2[h] = f2_pack(v.x, v.y);
+            w2[h + 1] = f2_pack(v.z, v.w);
+          }
+        } else if constexpr (PB == 2) w2[0] = f2_pack(ww[0], ww[1]);
+        else w2[0] = f2_pack(ww[0], 0.f);
+#pragma unroll
+        for (int t = 0; t < IPT; ++t) {
+          const uint64_t d2 = f2_pack(d[t], d[t]);
+#pragma unroll
+          for (int h = 0; h < H; ++h) s2[t][h] = f2_fma(d2, w2[h], s2[t][h]);
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < IPT; ++t) {
+        const int i = c0 + t * MMB_NT + tid;
+        if (i >= n) continue;
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          float v[2];
+          f2_unpack(s2[t][h], v[0], v[1]);
+#pragma unroll
+          for (int c = 0; c < (PB > 1 ? 2 : 1); ++c) {
+            const int q = 2 * h + c, p = p_s[q];
+            // a subnormal mass counts as 0, as in source_marginal
+            const float s = v[c] < P::tiny() ? 0.f : v[c];
+            if (p >= 0) A.S[(size_t)p * n + i] = s;
+            mass[q] += s;
+          }
+        }
+      }
+    }
+    if (m + 1 == A.mm_steps) {
+#pragma unroll
+      for (int q = 0; q < PB; ++q) {
+        const float ms = block_sum(mass[q], red);
+        if (tid == 0 && p_s[q] >= 0) A.mass[p_s[q]] = ms;
+      }
+    }
+  }
+  // weight change of this iteration's update: ||w - w_start||_1 / ||w||_1, one warp per problem
+  __syncthreads();
+  for (int q = warp; q < PB; q += MMB_NT / 32) {
+    float num = 0.f, den = 0.f;
+    for (int j = lane; j < k; j += 32) {
+      num += fabsf(w_s[j * PB + q] - w0_s[j * PB + q]);
+      den += fabsf(w_s[j * PB + q]);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      num += __shfl_xor_sync(0xffffffffu, num, o);
+      den += __shfl_xor_sync(0xffffffffu, den, o);
+    }
+    if (lane == 0 && p_s[q] >= 0) A.dw[p_s[q]] = num / den;
+  }
+}
+
+template <int PB, int KQ>
+static inline cudaError_t launch_mmb_cfg(const MMBArgs& a, int batch, cudaStream_t s) {
+  constexpr size_t smem = MmbSmem<PB, KQ>::bytes;
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(mm_batch_kernel<PB, KQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  mm_batch_kernel<PB, KQ><<<(batch + PB - 1) / PB, MMB_NT, smem, s>>>(a);
+  return cudaGetLastError();
+}
+template <int PB>
+static inline cudaError_t launch_mmb_pb(const MMBArgs& a, int batch, cudaStream_t s) {
+  if (a.k <= 32) return launch_mmb_cfg<PB, 1>(a, batch, s);
+  if (a.k <= 64) return launch_mmb_cfg<PB, 2>(a, batch, s);
+  if (a.k <= 128) return launch_mmb_cfg<PB, 4>(a, batch, s);
+  return launch_mmb_cfg<PB, 8>(a, batch, s);
+}
+// Problems per CTA: one while the batch does not fill the SMs, then as many as leave one CTA per SM.
+static inline cudaError_t launch_mm_batch(const MMBArgs& a, int batch, int sms, cudaStream_t s) {
+  if (batch <= sms) return launch_mmb_pb<1>(a, batch, s);
+  if (batch <= 4 * sms) return launch_mmb_pb<4>(a, batch, s);
+  return launch_mmb_pb<8>(a, batch, s);
+}
+
+}  // namespace otlm

@@ -26,6 +26,7 @@
 // left out (n of them change a sum by less than its FP32 rounding for n < 2^17).
 #pragma once
 
+#include "exp_api.h"
 #include "kernels.cuh"
 
 namespace otlm {
@@ -37,18 +38,12 @@ constexpr float EX_HMAX = 0.7355f;   // half-width with 2 ln2 h^2 = 0.75
 constexpr float EX_TILT = 72.f;      // bound of 2 |D| h
 constexpr float EX_SKIP = 42.f;      // log2 units below which a block pair is left out
 
-// b = bins per block (a multiple of 32), nb = blocks; nb = 0: the grid does not qualify (not sorted,
-// too coarse or too long) and rows are summed term by term.  q: centres are multiples of q (a power
-// of two at least 2^-18 of the largest |xt|), so that differences of centres are exact.
-struct ExPlan {
-  int b, nb;
-  float q;
-};
-
-// Shared-memory scratch of the apply (floats): centres, block maxima, row references, masks, then
-// EX_M coefficients per block pair.
+// Shared-memory scratch (floats) of the apply by `warps` warps: centres, block maxima, row references,
+// masks, then EX_M coefficients per block pair of a round (four row blocks per warp).
 constexpr int EX_HEAD = 4 * EX_NB;
-__host__ __device__ constexpr int ex_scratch_floats(int pairs) { return EX_HEAD + EX_M * pairs; }
+__host__ __device__ constexpr int ex_scratch_floats(int warps) {
+  return EX_HEAD + EX_M * EX_NB * (4 * warps < EX_NB ? 4 * warps : EX_NB);
+}
 
 __device__ __forceinline__ float ex_quantum(float x0, float x1) {
   const int e = (__float_as_int(fmaxf(fabsf(x0), fabsf(x1))) >> 23) & 255;
@@ -68,7 +63,7 @@ __device__ __forceinline__ ExPlan ex_plan_warp(const float* xt, int n, bool sort
   if (!(len <= 2.f * EX_HMAX * EX_NB)) return pl;
   const float q = ex_quantum(x0, x1);
   for (int nb = max(1, (int)(len / (2.f * EX_HMAX))); nb <= EX_NB; ++nb) {
-    const int b = ((n + nb - 1) / nb + 31) / 32 * 32, cnt = (n + b - 1) / b;
+    const int b = max(32, ((n + nb - 1) / nb + 7) / 8 * 8), cnt = (n + b - 1) / b;
     bool ok = true;
     if (lane < cnt) {
       const float c = ex_center(xt, lane, b, n, q);
@@ -109,28 +104,23 @@ __device__ __forceinline__ void ex_powers(float v, uint64_t (&p)[4]) {
   p[2] = f2_mul(p[1], s);
   p[3] = f2_mul(p[2], s);
 }
-// order-preserving integer of a float, for integer maxima
-__device__ __forceinline__ int ex_ordered(float f) {
-  const int i = __float_as_int(f);
-  return i >= 0 ? i : i ^ 0x7fffffff;
-}
-__device__ __forceinline__ float ex_unordered(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
-
-// One warp: the moments of column block [j0, j1) for G consecutive row blocks with d2[g] = 2 D.
-// Lanes take columns 32 apart; the powers of dj are shared by the G row blocks; the 8 G totals are
-// formed by a transposing butterfly (31 shuffles), after which lane g * 8 + m holds M_g,m.
-template <int G>
-__device__ __forceinline__ float ex_moments(const float* in_s, const float* xt, int j0, int j1, float cJ, float aJ,
-                                            const float (&d2)[G]) {
+// One warp: moments of the column blocks J0 + (lane / L) for G consecutive row blocks, L lanes per
+// column block; d2[g] = 2 D of the lane's column block, [j0, j1) its bins (empty: zeros).  Lanes take
+// bins L apart; the powers of dj are shared by the G row blocks.  The 8 G totals over L lanes are
+// formed by a transposing butterfly (31 shuffles for L = 32, 28 for L = 8, whose four column blocks
+// share them); those of the first gs row blocks are stored at cf[(g nb + J) * 8 + m].
+template <int G, int L>
+__device__ __forceinline__ void ex_moments(const float* in_s, const float* xt, int j0, int j1, float cJ, float aJ,
+                                           const float (&d2)[G], float* cf, int nb, int J, int gs) {
   using P = Prec<float>;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, l = lane % L;
   uint64_t acc[G][4];
 #pragma unroll
   for (int g = 0; g < G; ++g)
 #pragma unroll
     for (int k = 0; k < 4; ++k) acc[g][k] = 0ull;
 #pragma unroll 2
-  for (int j = j0 + lane; j < j1; j += 32) {
+  for (int j = j0 + l; j < j1; j += L) {
     const float v = xt[j] - cJ;
     const float h = fmaf(-v, v, in_s[j] - aJ);
     uint64_t p[4];
@@ -152,15 +142,21 @@ __device__ __forceinline__ float ex_moments(const float* in_s, const float* xt, 
       else r[8 * g + 2 * k] = r[8 * g + 2 * k + 1] = 0.f;
     }
 #pragma unroll
-  for (int s = 16; s > 0; s >>= 1) {
+  for (int s = L / 2, c = 16; s > 0; s >>= 1, c >>= 1) {
     const bool up = lane & s;
 #pragma unroll
-    for (int q = 0; q < s; ++q) {
-      const float keep = up ? r[q + s] : r[q], give = up ? r[q] : r[q + s];
+    for (int q = 0; q < c; ++q) {
+      const float keep = up ? r[q + c] : r[q], give = up ? r[q] : r[q + c];
       r[q] = keep + __shfl_xor_sync(0xffffffffu, give, s);
     }
   }
-  return r[0];
+  if constexpr (L == 32) {  // lane g * 8 + m holds M_g,m
+    if ((lane >> 3) < gs) cf[((lane >> 3) * nb + J) * EX_M + (lane & 7)] = r[0];
+  } else {  // lane 2 g + m / 4 of the eight holds M_g,m .. M_g,m+3
+    static_assert(L == 8, "eight or 32 lanes per column block");
+    if ((l >> 1) < gs && J < nb)
+      *reinterpret_cast<float4*>(cf + ((l >> 1) * nb + J) * EX_M + (l & 1) * 4) = make_float4(r[0], r[1], r[2], r[3]);
+  }
 }
 
 // One warp: Q x 32 rows i0 + 32 q + lane (< i1) of a row block, summed over the column blocks of
@@ -202,49 +198,60 @@ __device__ __forceinline__ void ex_rows(const float* xt, int i0, int i1, float c
   }
 }
 
-// The apply for row blocks [I0, I1) inside a CTA of NT threads: in_s [n] in shared memory (written
+// The apply for row blocks [I0, I1) by the T warps of a CTA: in_s [n] in shared memory (written
 // before the call; the first barrier is here), xt [n] (shared or global), scr = shared scratch of
-// ex_scratch_floats((I1 - I0) nb) floats, 16-byte aligned.  row(i, base, sum, di2) is called once per
-// row by one thread, with out_i = base + (log2(sum) - di2), base an integer and sum = 0 for an empty
-// (or non-finite) input.  Ends without a barrier.
-template <int NT, class Row>
+// ex_scratch_floats(T) floats, 16-byte aligned.  row(i, pre, base, sum, di2) is called once per row by
+// one thread, with out_i = base + (log2(sum) - di2), base an integer and sum = 0 for an empty (or
+// non-finite) input; pre = load(i) was called before the row's sums, so that what the row's epilogue
+// reads arrives meanwhile.
+//   T = 1 runs a problem in one warp without any block barrier, which is what fills the SMs when
+// there are several problems per SM (the phases of a CTA of eight warps are short against their
+// barriers: 1024 problems of 1024 bins took 74 us that way, see exp_solver.cuh).
+template <int T>
+__device__ __forceinline__ void ex_sync() {
+  if constexpr (T == 1) __syncwarp();
+  else __syncthreads();
+}
+template <int T, class Load, class Row>
 __device__ __forceinline__ void ex_apply(const float* in_s, const float* xt, int n, const ExPlan& pl, int I0, int I1,
-                                         float* scr, Row row) {
+                                         float* scr, Load load, Row row) {
   using P = Prec<float>;
-  constexpr int NW = NT / 32;
   // coefficients of the polynomial for 2^(2 t) = e^(2 ln2 t), |2 ln2 t| <= 0.75: (2 ln2)^m a_m with
   // a_m the degree-7 polynomial of smallest relative error for e^t on [-0.75, 0.75] (Remez exchange)
   constexpr double K = 2.0 * kLn2;
   constexpr double K2 = K * K, K4 = K2 * K2;
   float* cent = scr;
-  float* amax = scr + EX_NB;  // integers (ordered) until they are decoded into the rounded-up maxima
+  float* amax = scr + EX_NB;
   float* ref = scr + 2 * EX_NB;
   unsigned* mask_s = reinterpret_cast<unsigned*>(scr + 3 * EX_NB);
   float* cf = scr + EX_HEAD;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nb = pl.nb, b = pl.b;
-  if (tid < EX_NB) {
-    reinterpret_cast<int*>(amax)[tid] = ex_ordered(-CUDART_INF_F);
-    if (tid < nb) cent[tid] = ex_center(xt, tid, b, n, pl.q);
-  }
-  __syncthreads();
-  // block maxima of in_j - dj^2 (32 consecutive bins lie in one block)
+  const int tid = threadIdx.x, lane = tid & 31, warp = T == 1 ? 0 : tid >> 5, nb = pl.nb, b = pl.b;
+  if (tid < nb) cent[tid] = ex_center(xt, tid, b, n, pl.q);
+  ex_sync<T>();
+  // block maxima of in_j - dj^2, rounded up
   bool bad = false;
-  for (int j0 = warp * 32; j0 < n; j0 += NT) {
-    const int J = j0 / b, j = j0 + lane;
-    const float d = j < n ? xt[j] - cent[J] : 0.f;
-    const float v = j < n ? in_s[j] : -CUDART_INF_F;
-    bad |= !(v < CUDART_INF_F);
-    const int mx = __reduce_max_sync(0xffffffffu, ex_ordered(fmaf(-d, d, v)));
-    if (lane == 0) atomicMax(reinterpret_cast<int*>(amax) + J, mx);
+  for (int J = warp; J < nb; J += T) {
+    const float c = cent[J];
+    const int j1 = min(n, (J + 1) * b);
+    float mx = -CUDART_INF_F;
+#pragma unroll 4
+    for (int j = J * b + lane; j < j1; j += 32) {
+      const float d = xt[j] - c, v = in_s[j];
+      bad |= !(v < CUDART_INF_F);
+      mx = fmaxf(mx, fmaf(-d, d, v));
+    }
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) amax[J] = ceilf(mx);
   }
-  bad = __syncthreads_or(bad);
-  // decode the maxima; which column blocks matter to each row block (bounds over the block pair)
-  float aJ = -CUDART_INF_F;
-  if (lane < nb) aJ = ceilf(ex_unordered(reinterpret_cast<int*>(amax)[lane]));
-  const float cJl = lane < nb ? cent[lane] : 0.f;
-  __syncthreads();
-  if (warp == 0 && lane < nb) amax[lane] = aJ;
-  for (int I = I0 + warp; I < I1; I += NW) {
+  if constexpr (T == 1) {
+    bad = __any_sync(0xffffffffu, bad);
+    __syncwarp();
+  } else {
+    bad = __syncthreads_or(bad);
+  }
+  // which column blocks matter to each row block (bounds over the block pair)
+  const float aJ = lane < nb ? amax[lane] : -CUDART_INF_F, cJl = lane < nb ? cent[lane] : 0.f;
+  for (int I = I0 + warp; I < I1; I += T) {
     const float dm = fabsf(cent[I] - cJl), lo = fmaxf(dm - EX_HMAX, 0.f), hi = dm + EX_HMAX;
     // every term of the pair <= top; some term of the pair >= low at every row of the block
     const float top = aJ + (lo >= EX_HMAX ? lo * (2.f * EX_HMAX - lo) : EX_HMAX * EX_HMAX);
@@ -253,86 +260,96 @@ __device__ __forceinline__ void ex_apply(const float* in_s, const float* xt, int
     const unsigned mk = __ballot_sync(0xffffffffu, !bad && lane < nb && aJ > -CUDART_INF_F && top >= low - EX_SKIP);
     if (lane == 0) mask_s[I] = mk;
   }
-  __syncthreads();
-  // moments: items of one column block and up to four row blocks
-  const int nI = I1 - I0, ng = (nI + 3) / 4;
-  for (int t = warp; t < nb * ng; t += NW) {
-    const int J = t / ng, gi = t - J * ng;
-    const int Ia = I0 + nI * gi / ng, G = I0 + nI * (gi + 1) / ng - Ia;
-    bool any = false;
-    for (int g = 0; g < G; ++g) any |= (mask_s[Ia + g] >> J) & 1;
-    if (!any) continue;
-    const float cJ = cent[J], a = amax[J];
-    const int j0 = J * b, j1 = min(n, j0 + b);
-    float m;
-    if (G == 4) {
-      const float d2[4] = {2.f * (cent[Ia] - cJ), 2.f * (cent[Ia + 1] - cJ), 2.f * (cent[Ia + 2] - cJ), 2.f * (cent[Ia + 3] - cJ)};
-      m = ex_moments<4>(in_s, xt, j0, j1, cJ, a, d2);
-    } else if (G == 3) {
-      const float d2[3] = {2.f * (cent[Ia] - cJ), 2.f * (cent[Ia + 1] - cJ), 2.f * (cent[Ia + 2] - cJ)};
-      m = ex_moments<3>(in_s, xt, j0, j1, cJ, a, d2);
-    } else if (G == 2) {
-      const float d2[2] = {2.f * (cent[Ia] - cJ), 2.f * (cent[Ia + 1] - cJ)};
-      m = ex_moments<2>(in_s, xt, j0, j1, cJ, a, d2);
-    } else {
-      const float d2[1] = {2.f * (cent[Ia] - cJ)};
-      m = ex_moments<1>(in_s, xt, j0, j1, cJ, a, d2);
-    }
-    const int g = lane >> 3;
-    if (g < G) cf[((Ia + g - I0) * nb + J) * EX_M + (lane & 7)] = m;
-  }
-  __syncthreads();
-  // coefficients: moments times c_m and the pair's scale relative to the row block's reference
-  for (int I = I0 + warp; I < I1; I += NW) {
-    const unsigned mk = mask_s[I];
-    float* c = cf + ((I - I0) * nb + lane) * EX_M;
-    const bool on = (mk >> lane) & 1;
-    const float D = on ? cent[I] - cent[lane] : 0.f;
-    const float dd = __fmul_rn(D, D), de = __fmaf_rn(D, D, -dd), di = rintf(dd);
-    const float ai = on ? amax[lane] - di : -CUDART_INF_F, df = __fadd_rn(__fsub_rn(dd, di), de);
-    const float m0 = on ? c[0] : 0.f;
-    const int k = m0 > 0.f ? ((__float_as_int(m0) >> 23) & 255) - 127 : 0;
-    float e = m0 > 0.f ? ai + (float)(k + 1) : -CUDART_INF_F;
-    for (int o = 16; o > 0; o >>= 1) e = fmaxf(e, __shfl_xor_sync(0xffffffffu, e, o));
-    const bool live = e > -CUDART_INF_F;
-    if (on) {
-      // the moments are first scaled by 2^-k, k the exponent of M_0, so that the remaining scale
-      // underflows only where the pair is below 2^-126 of the block's largest at its centre
-      const float dn = __int_as_float((127 - k) << 23);
-      const float s = live ? P::exp2((ai + (float)k - e) - df) : 0.f;
-      float4 u = *reinterpret_cast<float4*>(c), w = *reinterpret_cast<float4*>(c + 4);
-      u.x = (u.x * dn) * (s * float(0.9999999849645456)); u.y = (u.y * dn) * (s * float(1.000000111089353 * K));
-      u.z = (u.z * dn) * (s * float(0.5000009663519951 * K2)); u.w = (u.w * dn) * (s * float(0.1666651273327656 * K2 * K));
-      w.x = (w.x * dn) * (s * float(0.04165746988152903 * K4)); w.y = (w.y * dn) * (s * float(0.008338260296134993 * K4 * K));
-      w.z = (w.z * dn) * (s * float(0.0014161683551980183 * K4 * K2)); w.w = (w.w * dn) * (s * float(0.0001953347388479001 * K4 * K2 * K));
-      *reinterpret_cast<float4*>(c) = u;
-      *reinterpret_cast<float4*>(c + 4) = w;
-    }
-    if (lane == 0) ref[I] = live ? e : 0.f;
-  }
-  __syncthreads();
-  // rows: items of up to 128 rows of one block
-  const int cpb = (b + 127) / 128, per = (b / 32 + cpb - 1) / cpb;  // items per block, 32-row groups per item
-  for (int t = warp; t < nI * cpb; t += NW) {
-    const int I = I0 + t / cpb, r0 = I * b + (t % cpb) * per * 32, i1 = min(n, (I + 1) * b);
-    const float* c = cf + (I - I0) * nb * EX_M;
-    const unsigned mk = mask_s[I];
-    const float base = ref[I];
-    auto go = [&](auto qc) {
-      constexpr int Q = decltype(qc)::value;
-      float di2[Q], sum[Q];
-      ex_rows<Q>(xt, r0, i1, cent[I], cent, mk, c, di2, sum);
+  ex_sync<T>();
+  // row blocks go in groups of three or four (equal shares), a round takes up to T groups
+  const int ng = (I1 - I0 + 3) / 4, cpb = (b + 127) / 128, per = ((b + 31) / 32 + cpb - 1) / cpb;
+  const bool narrow = b < 256;  // 8 lanes per column block (four at a time) for short blocks
+  const int nr = narrow ? (nb + 3) / 4 : nb;
+  for (int g0 = 0; g0 < ng; g0 += T) {
+    const int gn = min(T, ng - g0);
+    const int Ia = I0 + (I1 - I0) * g0 / ng, Ib = I0 + (I1 - I0) * (g0 + gn) / ng;
+    // moments: items of one group and one (or four) column blocks
+    for (int t = warp; t < gn * nr; t += T) {
+      const int gi = g0 + t / nr, I = I0 + (I1 - I0) * gi / ng, G = I0 + (I1 - I0) * (gi + 1) / ng - I;
+      const int J = narrow ? (t % nr) * 4 + (lane >> 3) : t % nr;
+      bool on = false;
+      float d2[4];
+      const float cJ = J < nb ? cent[J] : 0.f, a = J < nb ? amax[J] : 0.f;
 #pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        const int i = r0 + 32 * q + lane;
-        if (i < i1) row(i, base, sum[q], di2[q]);
+      for (int g = 0; g < 4; ++g) {
+        const bool in = g < G && J < nb;
+        on |= in && ((mask_s[in ? I + g : I] >> J) & 1);
+        d2[g] = in ? 2.f * (cent[I + g] - cJ) : 0.f;
       }
-    };
-    const int groups = min(per, (i1 - r0 + 31) / 32);
-    if (groups >= 4) go(std::integral_constant<int, 4>{});
-    else if (groups == 3) go(std::integral_constant<int, 3>{});
-    else if (groups == 2) go(std::integral_constant<int, 2>{});
-    else if (groups == 1) go(std::integral_constant<int, 1>{});
+      if (!__any_sync(0xffffffffu, on)) continue;
+      const int j0 = on ? J * b : 0, j1 = on ? min(n, j0 + b) : 0;
+      float* c = cf + (I - Ia) * nb * EX_M;
+      if (G == 4) {
+        if (narrow) ex_moments<4, 8>(in_s, xt, j0, j1, cJ, a, d2, c, nb, J, 4);
+        else ex_moments<4, 32>(in_s, xt, j0, j1, cJ, a, d2, c, nb, J, 4);
+      } else {  // three (or, for fewer than three row blocks, the first ones of three)
+        const float e2[3] = {d2[0], d2[1], d2[2]};
+        if (narrow) ex_moments<3, 8>(in_s, xt, j0, j1, cJ, a, e2, c, nb, J, G);
+        else ex_moments<3, 32>(in_s, xt, j0, j1, cJ, a, e2, c, nb, J, G);
+      }
+    }
+    ex_sync<T>();
+    // coefficients: moments times c_m and the pair's scale relative to the row block's reference
+    for (int I = Ia + warp; I < Ib; I += T) {
+      const unsigned mk = mask_s[I];
+      float* c = cf + ((I - Ia) * nb + lane) * EX_M;
+      const bool on = (mk >> lane) & 1;
+      const float D = on ? cent[I] - cent[lane] : 0.f;
+      const float dd = __fmul_rn(D, D), de = __fmaf_rn(D, D, -dd), di = rintf(dd);
+      const float ai = on ? amax[lane] - di : -CUDART_INF_F, df = __fadd_rn(__fsub_rn(dd, di), de);
+      const float m0 = on ? c[0] : 0.f;
+      const int k = m0 > 0.f ? ((__float_as_int(m0) >> 23) & 255) - 127 : 0;
+      float e = m0 > 0.f ? ai + (float)(k + 1) : -CUDART_INF_F;
+      for (int o = 16; o > 0; o >>= 1) e = fmaxf(e, __shfl_xor_sync(0xffffffffu, e, o));
+      const bool live = e > -CUDART_INF_F;
+      if (on) {
+        // the moments are first scaled by 2^-k, k the exponent of M_0, so that the remaining scale
+        // underflows only where the pair is below 2^-126 of the block's largest at its centre
+        const float dn = __int_as_float((127 - k) << 23);
+        const float s = live ? P::exp2((ai + (float)k - e) - df) : 0.f;
+        float4 u = *reinterpret_cast<float4*>(c), w = *reinterpret_cast<float4*>(c + 4);
+        u.x = (u.x * dn) * (s * float(0.9999999849645456)); u.y = (u.y * dn) * (s * float(1.000000111089353 * K));
+        u.z = (u.z * dn) * (s * float(0.5000009663519951 * K2)); u.w = (u.w * dn) * (s * float(0.1666651273327656 * K2 * K));
+        w.x = (w.x * dn) * (s * float(0.04165746988152903 * K4)); w.y = (w.y * dn) * (s * float(0.008338260296134993 * K4 * K));
+        w.z = (w.z * dn) * (s * float(0.0014161683551980183 * K4 * K2)); w.w = (w.w * dn) * (s * float(0.0001953347388479001 * K4 * K2 * K));
+        *reinterpret_cast<float4*>(c) = u;
+        *reinterpret_cast<float4*>(c + 4) = w;
+      }
+      if (lane == 0) ref[I] = live ? e : 0.f;
+    }
+    ex_sync<T>();
+    // rows: items of up to 128 rows of one block
+    for (int t = warp; t < (Ib - Ia) * cpb; t += T) {
+      const int I = Ia + t / cpb, r0 = I * b + (t % cpb) * per * 32, i1 = min(n, (I + 1) * b);
+      const float* c = cf + (I - Ia) * nb * EX_M;
+      const unsigned mk = mask_s[I];
+      const float base = ref[I];
+      const int iend = min(i1, r0 + per * 32);
+      auto go = [&](auto qc) {
+        constexpr int Q = decltype(qc)::value;
+        float di2[Q], sum[Q];
+        decltype(load(0)) pre[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) pre[q] = load(min(r0 + 32 * q + lane, iend - 1));
+        ex_rows<Q>(xt, r0, iend, cent[I], cent, mk, c, di2, sum);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+          const int i = r0 + 32 * q + lane;
+          if (i < iend) row(i, pre[q], base, sum[q], di2[q]);
+        }
+      };
+      const int groups = (iend - r0 + 31) / 32;
+      if (groups >= 4) go(std::integral_constant<int, 4>{});
+      else if (groups == 3) go(std::integral_constant<int, 3>{});
+      else if (groups == 2) go(std::integral_constant<int, 2>{});
+      else if (groups == 1) go(std::integral_constant<int, 1>{});
+    }
+    ex_sync<T>();  // the round's coefficients have been read
   }
 }
 

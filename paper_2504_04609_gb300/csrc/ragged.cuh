@@ -64,7 +64,7 @@ template <int NT>
 struct RaggedSmem {
   // offsets (floats) into dynamic shared memory for a problem of n_max bins, k_max atoms
   static __host__ __device__ size_t floats(int n_max, int k_max) {
-    return state(n_max, k_max) + ex_scratch_floats(EX_NB * EX_NB);
+    return state(n_max, k_max) + ex_scratch_floats(NT / 32);
   }
   // everything but the expansion's scratch, rounded up to 16 bytes
   static __host__ __device__ size_t state(int n_max, int k_max) {
@@ -196,7 +196,7 @@ template <int NT>
 __device__ __noinline__ void ragged_apply_ex(const float* xt, const float* in, float* out, int n, ExPlan pl, float* scr,
                                              float* ratio) {
   using P = Prec<float>;
-  ex_apply<NT>(in, xt, n, pl, 0, pl.nb, scr, [&](int i, float base, float sum, float di2) {
+  ex_apply<NT / 32>(in, xt, n, pl, 0, pl.nb, scr, [](int) { return 0; }, [&](int i, int, float base, float sum, float di2) {
     if (ratio) ratio[i] = sum > 0.f ? sum * P::exp2((base - out[i]) - di2) : 0.f;
     out[i] = sum > 0.f ? base + (P::log2(sum) - di2) : P::ninf();
   });

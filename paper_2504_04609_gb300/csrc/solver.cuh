@@ -7,6 +7,7 @@
 #include <cstddef>
 #include <cstdint>
 
+#include "exp_api.h"
 #include "kernels.cuh"
 #include "objective_kernels.cuh"
 
@@ -289,6 +290,71 @@ void objective_eval(const Launch& L, const Workspace<T>& ws, const ObjWorkspace<
   L.end();
 }
 
+// Argument block of the expansion applies from the workspace: the block plan lives in the spare words
+// after the active count, a small batch's partial violations in F2 (the expansion path forms F2 on
+// the fly) and the per-problem CTA counts in err_acc (zeroed by prep_kernel, left at zero).
+inline ExPlan* ex_plan_of(const Workspace<float>& ws) { return reinterpret_cast<ExPlan*>(ws.n_active + 4); }
+inline ExArgs ex_args(const Workspace<float>& ws, const SolveParams& sp, const float* y) {
+  const double eps_ln2 = sp.eps * kLn2;
+  ExArgs a{};
+  a.active = ws.active; a.n_active = ws.n_active; a.plan = ex_plan_of(ws); a.xt = ws.xt;
+  a.n = sp.n; a.k = sp.k; a.max_iter = sp.max_iter; a.datafit = sp.datafit; a.y = y;
+  a.G2 = ws.G2; a.LA2 = ws.LA2; a.LB2 = ws.LB2; a.S = ws.S; a.mass = ws.mass;
+  a.tol = float(sp.tol); a.dw_tol = float(sp.dw_tol); a.err = ws.err; a.dw = ws.dw;
+  a.W = ws.W; a.Wprev = ws.Wprev; a.done = ws.done; a.iters = ws.iters; a.status = ws.status;
+  a.part = ws.F2; a.count = reinterpret_cast<int*>(ws.err_acc);
+  a.kl_coef = float(sp.lam / (sp.eps + sp.lam)); a.tv_bound = float(sp.lam / eps_ln2);
+  a.lam_over_eps = float(sp.lam / sp.eps); a.log_lam_over_eps = float(log(sp.lam / sp.eps));
+  return a;
+}
+// The expansion applies serve the squared-distance grid cost in FP32 arithmetic (FP32 and tensor-core
+// handles); solves with FP64 gap checks keep the applies that objective_eval shares.
+inline bool ex_serves(const SolveParams& sp, bool dense, bool checks) {
+  return !dense && !checks && sp.cost == COST_SQ && sp.n <= EXA_MAX_N;
+}
+
+// The iteration loop of solve_device with expansion applies (three launches beside the compaction).
+inline cudaError_t ex_iterate(const Launch& L, const Workspace<float>& ws, const SolveParams& sp, const float* D,
+                              const float* y) {
+  const int batch = sp.batch, sms = sm_count();
+  L.begin(KIND_OTHER);
+  cudaError_t e = ex_plan(ws.xt, sp.n, ex_plan_of(ws), L.stream);
+  L.end();
+  if (e != cudaSuccess) return e;
+  ExArgs a = ex_args(ws, sp, y);
+  MMBArgs mm{ws.active, ws.n_active, sp.n, sp.k, D, ws.Dt, ws.xcol, ws.LA2, ws.S, ws.W, ws.mass, ws.dw, ws.done,
+             sp.penalty, sp.mm_steps, float(sp.eps), float(sp.alpha), float(sp.beta)};
+  for (int it = 0;; ++it) {
+    a.it = it;
+    a.check = it > 0;
+    L.begin(KIND_APPLY);
+    e = ex_apply_source(a, batch, false, sms, L.stream);
+    L.end();
+    if (e != cudaSuccess) return e;
+    if (it >= sp.max_iter) return cudaSuccess;
+    L.begin(KIND_MM);
+    e = mm_batch(mm, batch, sms, L.stream);
+    L.end();
+    if (e != cudaSuccess) return e;
+    if (it > 0) {
+      L.begin(KIND_COMPACT);
+      compact_kernel<<<1, 1024, 0, L.stream>>>(ws.active, ws.n_active, ws.done);
+      L.end();
+    }
+    L.begin(KIND_APPLY);
+    e = ex_apply_target(a, batch, false, sms, L.stream);
+    L.end();
+    if (e != cudaSuccess) return e;
+    if ((it + 1) % sp.poll_every == 0) {
+      e = cudaMemcpyAsync(L.host_flag, ws.n_active, sizeof(int), cudaMemcpyDeviceToHost, L.stream);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(L.stream);
+      if (e == cudaSuccess && L.timer && L.timer->on) e = L.timer->harvest();
+      if (e != cudaSuccess) return e;
+      if (*L.host_flag == 0) return cudaSuccess;
+    }
+  }
+}
+
 // Run Algorithm 1 on device buffers.  Returns cudaSuccess or the first launch/copy error.
 // ow (may be null when sp.check_every == 0): the objective scratch of the gap checks.
 template <typename T>
@@ -347,7 +413,15 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
   mm.dw = ws.dw; mm.dw_tol = T(sp.dw_tol); mm.gap_on = checks && sp.gap_tol > 0;
   mm.gap_ok = checks ? ow->gap_ok : nullptr;
 
-  for (int it = 0;; ++it) {
+  bool by_expansion = false;
+  if constexpr (sizeof(T) == 4) {
+    by_expansion = ex_serves(sp, C != nullptr, checks);
+    if (by_expansion) {
+      const cudaError_t e = ex_iterate(L, ws, sp, D, y);
+      if (e != cudaSuccess) return e;
+    }
+  }
+  for (int it = 0; !by_expansion; ++it) {
     src.check = it > 0;
     launch_apply<T, EPI_SOURCE>(L, src, it == 0, batch, n, sp.cost);
     // a check: the state (w, g) whose a = K u1 was just computed is the one this iteration returns

@@ -93,3 +93,44 @@ def test_expansion_in_the_uneven_batch(grid, n, eps, datafit, penalty, alpha, ct
         o = _oracle(p, float(np.float32(eps)), datafit, penalty, alpha, T)
         assert rel_l1(w.cpu().numpy()[i * k:(i + 1) * k], o["w"]) <= TOL32
         assert rel_l1(t.cpu().numpy()[i * n:(i + 1) * n], o["t"]) <= TOL32
+
+
+@pytest.mark.parametrize("grid,n,eps,datafit,penalty,alpha", CASES)
+@pytest.mark.parametrize("B", [1, 3, 620])
+def test_expansion_in_the_shared_grid_batch(grid, n, eps, datafit, penalty, alpha, B):
+    """B = 1 and 3 split a problem's row blocks over CTAs, 620 gives one CTA of four warps to a
+    problem (620 problems are copies of three)."""
+    T, k = 8, 20
+    probs = _problems(grid, n, k, eps, 92, min(B, 3))
+    x, D = probs[0]["x"], probs[0]["D"]  # the batch shares the first problem's grid and dictionary
+    y = np.stack([probs[p % 3]["y"] for p in range(B)])
+    w0 = spectra.initial_weights(y, D).astype(np.float32)
+    dev = lambda a: torch.tensor(a, device="cuda")  # noqa: E731
+    r = api.solve(dev(x), dev(D), dev(y), eps, 1.0, alpha, datafit, penalty, dev(w0), max_iter=T)
+    assert np.all(r.iters.cpu().numpy() == T)
+    for p in range(min(B, 3)):
+        o = _oracle(dict(probs[p], D=D), eps, datafit, penalty, alpha, T)
+        for q in range(p, B, 3):
+            if q in (p, B - 3 + p):
+                assert rel_l1(r.w[q].cpu().numpy(), o["w"]) <= TOL32
+                assert rel_l1(r.t[q].cpu().numpy(), o["t"]) <= TOL32
+
+
+@pytest.mark.parametrize("k", [1, 33, 64, 129, 256])
+@pytest.mark.parametrize("B", [2, 200, 700])
+def test_batched_mm_step_sizes(k, B):
+    """Every dictionary bucket with one, four and eight problems per CTA (a ragged last CTA), two MM
+    steps, against the oracle at the FP32 bar."""
+    d = spectra.batch(93, min(B, 3), 261, k, 1)
+    y = d["y"][np.arange(B) % min(B, 3)]
+    w0 = spectra.initial_weights(y, d["D"]).astype(np.float32)
+    dev = lambda a: torch.tensor(a, device="cuda")  # noqa: E731
+    r = api.solve(dev(d["x"]), dev(d["D"]), dev(y), 5e-2, 1.0, 1e-3, "l2", "l2sq", dev(w0), max_iter=6, mm_steps=2)
+    C = spectra.squared_cost(d["x"].astype(np.float64))
+    D64 = d["D"].astype(np.float64)
+    for p in range(min(B, 3)):
+        y64 = y[p].astype(np.float64)
+        o = oracle.solve_log(C, D64, y64, 5e-2, 1.0, 1e-3, "l2", "l2sq", spectra.initial_weights(y64, D64), 6, mm_steps=2)
+        for q in (p, (B - 1) // 3 * 3 + p if (B - 1) // 3 * 3 + p < B else p):
+            assert rel_l1(r.w[q].cpu().numpy(), o["w"]) <= TOL32
+            assert rel_l1(r.t[q].cpu().numpy(), o["t"]) <= TOL32
