@@ -109,6 +109,26 @@ __device__ __forceinline__ float wright_omega_fast(float z) {
   return w;
 }
 
+// FP64: the FP32 solution above as the start (relative 1e-7) and one step of the fourth-order
+// iteration of Fritsch, Shafer & Crowley (CACM 16, 1973; Lawrence, Corless & Jeffrey, sec. 3)
+//   r = z - w - log w,  t = (1 + w)(1 + w + 2 r / 3),  w <- w (1 + r / (1 + w) (t - r / 2) / (t - r)),
+// whose error is of the order of the start's fourth power: one FP64 logarithm and one division
+// instead of five Newton steps with one of each (a double logarithm is some forty instructions of
+// GB300's slow FP64 pipe). Outside FP32's range the general iteration serves; below e^-40 omega is e^z
+// to working precision.
+__device__ __forceinline__ double wright_omega_f64(double z) {
+  if (!(z > -40.0)) return (z == z) ? ::exp(z) : z;
+  if (!(z < 1e30)) return wright_omega<double>(z);
+  const double w = (double)wright_omega_fast((float)z);
+  const double r = z - w - ::log(w), u = 1.0 + w, t = u * (u + (2.0 / 3.0) * r);
+  return w + w * (r * (t - 0.5 * r)) / (u * (t - r));
+}
+template <typename T>
+__device__ __forceinline__ T wright_omega_of(T z) {
+  if constexpr (sizeof(T) == 8) return wright_omega_f64(z);
+  else return wright_omega<T>(z);
+}
+
 // Sum over a block of `nthreads` threads; `red` holds >= 32 elements of shared scratch.
 template <typename T>
 __device__ __forceinline__ T block_sum(T v, T* red) {

@@ -34,7 +34,7 @@ __device__ __noinline__ T poisson_g2(T log_lam_over_eps, T lam_over_eps, T neg_b
   using P = Prec<T>;
   if (!(yv > T(0))) return -neg_bound;
   const T l2c = log_lam_over_eps * T(kLog2e) + P::log2(yv);
-  return l2c - P::log2(wright_omega<T>((l2c - v) * T(kLn2) + lam_over_eps)) - v;
+  return l2c - P::log2(wright_omega_of<T>((l2c - v) * T(kLn2) + lam_over_eps)) - v;
 }
 
 template <typename T>
@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(Cfg::NT) apply_kernel(ApplyArgs<T> A) {
             case DF_POISSON: gn = poisson_g2<T>(A.log_lam_over_eps, A.lam_over_eps, A.tv_bound, v, yv); break;
             default: {  // L2: g = lam y - eps omega(ln(lam/eps) + ln b + (lam/eps) y)
               const T z = A.log_lam_over_eps + v * T(kLn2) + A.lam_over_eps * yv;
-              gn = (A.lam_over_eps * yv - wright_omega<T>(z)) * T(kLog2e);
+              gn = (A.lam_over_eps * yv - wright_omega_of<T>(z)) * T(kLog2e);
             }
           }
           A.G2[idx] = gn;
@@ -492,6 +492,10 @@ struct MMArgs {
   int gap_on;       // gap_tol > 0: the gap is a stopping criterion
   int penalty;
   int mm_steps = 1;  // MM steps with the same LA2 (a = K u1)
+  // f64_mm_kernel: the first step's log ratios, 1 / a, and u2 = S / a out
+  const T* R = nullptr;
+  const T* IA = nullptr;
+  T* U2 = nullptr;
   T eps, alpha, beta;
 };
 
@@ -609,15 +613,16 @@ __global__ void __launch_bounds__(256) mm_kernel(MMArgs<T> A) {
       for (int w8 = 0; w8 < 8; ++w8) sum += red_s[w8][j];
       const T xj = A.xcol[j];
       const T wold = A.W[(size_t)p * k + j];
-      const T nu = P::log(wold) + sum * T(kLn2) / xj;
+      const T dl = sum * T(kLn2) / xj;
       // l1 and elastic net: nu shifted by alpha/(eps x_j); squared l2 and elastic net:
       // W0(c e^nu)/c = omega(log c + nu)/c with c = alpha resp. beta over eps x_j (App. A)
       const T shift = (A.penalty == PEN_L1 || A.penalty == PEN_ELASTIC) ? A.alpha / (A.eps * xj) : T(0);
       T wn;
       if (A.penalty == PEN_L2SQ || A.penalty == PEN_ELASTIC) {
         const T c = (A.penalty == PEN_ELASTIC ? A.beta : A.alpha) / (A.eps * xj);
-        wn = wright_omega<T>(P::log(c) + nu - shift) / c;
-      } else wn = P::exp(nu - shift);
+        if constexpr (sizeof(T) == 8) wn = wright_omega_of<T>(P::log(c * wold) + dl - shift) / c;  // one logarithm
+        else wn = wright_omega_of<T>(P::log(c) + (P::log(wold) + dl) - shift) / c;
+      } else wn = P::exp((P::log(wold) + dl) - shift);
       A.W[(size_t)p * k + j] = wn;
       w_s[j] = wn;
     }

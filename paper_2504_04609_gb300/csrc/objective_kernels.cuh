@@ -189,9 +189,34 @@ __global__ void __launch_bounds__(256) objective_reduce_kernel(ObjArgs<T> A) {
   // two-sum into a float pair, moved into an FP64 sum every 64 rows: FP64-grade accuracy without
   // an FP64 multiply-add per dictionary entry (the FP64 pipe is the slow one here).
   const double f2_lo = f_lo / el2;  // log2 units
+  // FP64: warps take rows, lanes columns (one FP64 instruction serves 32 columns), and the eight
+  // warps' sums are added in order.
+  if constexpr (sizeof(T) == 8) {
+    __shared__ double part_s[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int j0 = 0; j0 < k; j0 += 32) {
+      const int j = j0 + lane;
+      double acc = 0.0;
+#pragma unroll 4
+      for (int i = warp; i < n; i += 8) {
+        const double d = j < k ? A.D[(size_t)i * k + j] : 0.0;
+        double f = F2[i];
+        if (!isfinite(f)) f = f2_lo;
+        if (d > 0.0) acc = fma(d, f, acc);
+      }
+      __syncthreads();
+      part_s[warp][lane] = acc;
+      __syncthreads();
+      if (warp == 0 && j < k) {
+        acc = 0.0;
+        for (int w = 0; w < 8; ++w) acc += part_s[w][lane];
+        xtf_s[j] = acc * el2;
+      }
+    }
+  } else
   for (int j = threadIdx.x; j < k; j += blockDim.x) {
     double acc = 0.0;
-    if constexpr (sizeof(T) == 4) {
+    {
       for (int i0 = 0; i0 < n; i0 += 64) {
         float hi = 0.f, lo = 0.f;
         const int i1 = min(n, i0 + 64);
@@ -209,15 +234,6 @@ __global__ void __launch_bounds__(256) objective_reduce_kernel(ObjArgs<T> A) {
         acc += (double)hi + (double)lo;
       }
       acc *= el2;
-    } else {
-      for (int i = 0; i < n; ++i) {
-        const double d = A.D[(size_t)i * k + j];
-        if (d > 0.0) {
-          double f = el2 * (double)F2[i];
-          if (!isfinite(f)) f = f_lo;
-          acc += d * f;
-        }
-      }
     }
     xtf_s[j] = acc;
   }

@@ -28,6 +28,7 @@ struct otlm_ctx {
   void* ws = nullptr;        // solver workspace (one allocation)
   void* stage = nullptr;     // device staging for otlm_solve_host (allocated on first use)
   size_t stage_bytes = 0;
+  void* f64 = nullptr;       // FP64 handles up to n_max = F64_MAX_N: stored kernel and scalings (f64.cuh)
   int* host_flag = nullptr;  // pinned
   long long launches = 0;
   size_t elem = 4;
@@ -132,7 +133,8 @@ int run_solve(otlm_ctx* h, const SolveParams& sp, const void* x, const void* C, 
                               (float*)g, (float*)t_out, iters_out, (float*)err_out, status_out);
   } else {
     e = otlm::solve_device<T>(L, ws, lay.obj ? &ow : nullptr, sp, (const T*)x, (const T*)D, (const T*)y, (T*)w,
-                              (T*)g, (T*)t_out, iters_out, (T*)err_out, status_out, (const T*)C);
+                              (T*)g, (T*)t_out, iters_out, (T*)err_out, status_out, (const T*)C,
+                              otlm::f64_carve(h->f64, c.n_max, c.batch_max));
   }
   if (e == cudaErrorLaunchTimeout) return OTLM_ETIMEOUT;
   return e == cudaSuccess ? OTLM_OK : OTLM_ECUDA;
@@ -145,7 +147,8 @@ int run_objective(otlm_ctx* h, const SolveParams& sp, const void* x, const void*
   otlm::carve_workspace<T>(h->ws, h->cfg.n_max, h->cfg.k_max, h->cfg.batch_max, &ws);
   Launch L{h->stream, &h->launches, h->host_flag, &h->timer};
   cudaError_t e = otlm::objective_device<T>(L, ws, sp, (const T*)x, (const T*)D, (const T*)y, (const T*)w,
-                                            (const T*)g, primal, dual);
+                                            (const T*)g, primal, dual,
+                                            otlm::f64_carve(h->f64, h->cfg.n_max, h->cfg.batch_max));
   return e == cudaSuccess ? OTLM_OK : OTLM_ECUDA;
 }
 
@@ -298,8 +301,15 @@ int otlm_create(otlm_handle* out, const otlm_config* cfg, void* cuda_stream) {
     delete h;
     return OTLM_ENOMEM;
   }
+  // the stored kernel is an option: without room for it the log-sum-exp applies serve
+  if (c.precision == OTLM_PREC_FP64 && c.n_max <= otlm::F64_MAX_N &&
+      cudaMalloc(&h->f64, otlm::f64_bytes(c.n_max, c.batch_max)) != cudaSuccess) {
+    h->f64 = nullptr;
+    (void)cudaGetLastError();
+  }
   if (cudaMallocHost(&h->host_flag, sizeof(int)) != cudaSuccess) {
     cudaFree(h->ws);
+    if (h->f64) cudaFree(h->f64);
     delete h;
     return OTLM_ECUDA;
   }
@@ -311,6 +321,7 @@ void otlm_destroy(otlm_handle h) {
   if (!h) return;
   cudaStreamSynchronize(h->stream);
   cudaFree(h->ws);
+  if (h->f64) cudaFree(h->f64);
   if (h->stage) cudaFree(h->stage);
   cudaFreeHost(h->host_flag);
   if (h->timer_ready) h->timer.destroy();

@@ -8,6 +8,7 @@
 #include <cstdint>
 
 #include "exp_api.h"
+#include "f64.cuh"
 #include "kernels.cuh"
 #include "objective_kernels.cuh"
 
@@ -336,7 +337,8 @@ inline cudaError_t ex_iterate(const Launch& L, const Workspace<float>& ws, const
     e = mm_batch(mm, batch, sms, L.stream);
     L.end();
     if (e != cudaSuccess) return e;
-    if (it > 0) {
+    const bool poll = (it + 1) % sp.poll_every == 0;
+    if (poll && it > 0) {  // finished problems are skipped by their flag in between
       L.begin(KIND_COMPACT);
       compact_kernel<<<1, 1024, 0, L.stream>>>(ws.active, ws.n_active, ws.done);
       L.end();
@@ -345,7 +347,7 @@ inline cudaError_t ex_iterate(const Launch& L, const Workspace<float>& ws, const
     e = ex_apply_target(a, batch, false, sms, L.stream);
     L.end();
     if (e != cudaSuccess) return e;
-    if ((it + 1) % sp.poll_every == 0) {
+    if (poll) {
       e = cudaMemcpyAsync(L.host_flag, ws.n_active, sizeof(int), cudaMemcpyDeviceToHost, L.stream);
       if (e == cudaSuccess) e = cudaStreamSynchronize(L.stream);
       if (e == cudaSuccess && L.timer && L.timer->on) e = L.timer->harvest();
@@ -360,7 +362,7 @@ inline cudaError_t ex_iterate(const Launch& L, const Workspace<float>& ws, const
 template <typename T>
 cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorkspace<T>* ow, const SolveParams& sp,
                          const T* x, const T* D, const T* y, T* w, T* g, T* t_out, int* iters_out, T* err_out,
-                         int* status_out, const T* C = nullptr) {
+                         int* status_out, const T* C = nullptr, const F64Buf& f64 = F64Buf()) {
   const int batch = sp.batch, n = sp.n, k = sp.k;
   const double eps_ln2 = sp.eps * kLn2;
   const bool checks = ow && sp.check_every > 0;
@@ -421,7 +423,52 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
       if (e != cudaSuccess) return e;
     }
   }
-  for (int it = 0; !by_expansion; ++it) {
+  bool linear = false;
+  if constexpr (sizeof(T) == 8) {
+    linear = f64 && !C && !checks;
+    if (linear) {
+      const int abs_cost = sp.cost == COST_ABS;
+      L.begin(KIND_OTHER);
+      f64_build_kernel<<<1184, 256, 0, L.stream>>>(ws.xt, n, f64.K, abs_cost);
+      L.end();
+      L.begin(KIND_OTHER);
+      f64_scale_kernel<<<1184, 256, 0, L.stream>>>(ws.G2, f64.U1, y, f64.LY, (size_t)batch * n);
+      L.end();
+      src.G2 = ws.G2;
+      mm.R = ws.F2; mm.IA = f64.IA; mm.U2 = f64.U2;
+      for (int it = 0;; ++it) {
+        src.check = it > 0;
+        L.begin(KIND_APPLY);
+        cudaError_t e = launch_f64_apply<EPI_SOURCE>(src, f64, ws.LA2, ws.F2, ws.done, batch, abs_cost, 1, sm_count(), L.stream);
+        L.end();
+        if (e != cudaSuccess) return e;
+        mm.it = it;
+        L.begin(KIND_MM);
+        e = launch_f64_mm(mm, batch, L.stream);
+        L.end();
+        if (e != cudaSuccess) return e;
+        if (it >= sp.max_iter) break;
+        const bool poll = (it + 1) % sp.poll_every == 0;
+        if (poll && it > 0) {  // finished problems are skipped by their flag in between
+          L.begin(KIND_COMPACT);
+          compact_kernel<<<1, 1024, 0, L.stream>>>(ws.active, ws.n_active, ws.done);
+          L.end();
+        }
+        L.begin(KIND_APPLY);
+        e = launch_f64_apply<EPI_TARGET>(tgt, f64, ws.LA2, nullptr, ws.done, batch, abs_cost, 1, sm_count(), L.stream);
+        L.end();
+        if (e != cudaSuccess) return e;
+        if (poll) {
+          e = cudaMemcpyAsync(L.host_flag, ws.n_active, sizeof(int), cudaMemcpyDeviceToHost, L.stream);
+          if (e == cudaSuccess) e = cudaStreamSynchronize(L.stream);
+          if (e == cudaSuccess && L.timer && L.timer->on) e = L.timer->harvest();
+          if (e != cudaSuccess) return e;
+          if (*L.host_flag == 0) break;
+        }
+      }
+    }
+  }
+  for (int it = 0; !by_expansion && !linear; ++it) {
     src.check = it > 0;
     launch_apply<T, EPI_SOURCE>(L, src, it == 0, batch, n, sp.cost);
     // a check: the state (w, g) whose a = K u1 was just computed is the one this iteration returns
