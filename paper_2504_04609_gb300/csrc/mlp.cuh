@@ -8,10 +8,8 @@
 //             KL datafit) are masked out of the loss.
 //   loss      mean over unmasked entries of (z - t_norm)^2
 // Weights are stored in BF16 for the forward pass (FP32 accumulation) with FP32 master copies
-// updated by AdamW.  Training contractions go through one register-tiled SIMT kernel with strided
-// operands (C = A B with A(m,k), B(k,n) given by element strides), which covers the forward pass
-// (B = W^T), the input gradient (B = W) and the weight gradient (A = dH^T).  Inference runs the
-// forward pass on the tcgen05 GEMM (below).
+// updated by AdamW.  Inference runs on the tcgen05 GEMM (tc_gemm.cuh) with BF16 hi/lo activations;
+// training contractions keep FP32 products and rounding (below).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -23,175 +21,293 @@ namespace mlp {
 
 constexpr int LAYERS = 4;
 
-// ---- GEMM: C[m][n] (row stride ldc) = sum_k A(m,k) B(k,n) (+ bias[n]) --------------------------
-// A(m,k) = A[m * sam + k * sak] (float), B(k,n) = B[k * sbk + n * sbn] (TB = float or bf16).
-// Epilogue: PRE != null stores the pre-activation, C = GELU(pre) when gelu, accumulate into C when
-// acc_out.  Tile 64 x 64, k-chunk 16, 256 threads, 4 x 4 outputs per thread.
-template <typename TB>
-__device__ __forceinline__ float ldB(const TB* p) { return static_cast<float>(*p); }
-template <>
-__device__ __forceinline__ float ldB<__nv_bfloat16>(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad(float z) {
   return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
 }
 
-template <typename TB>
-__global__ void __launch_bounds__(256) gemm_kernel(int M, int N, int K, const float* A, long long sam, long long sak,
-                                                   const TB* B, long long sbk, long long sbn, float* C, int ldc,
-                                                   const float* bias, float* pre, int gelu_on, int acc_out) {
-  constexpr int BM = 64, BN = 64, BK = 16;
-  __shared__ float As[BK][BM + 4];
-  __shared__ float Bs[BK][BN + 4];
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += BK) {
-    // the contiguous dimension of each operand is the fastest-varying thread index (coalesced)
-    for (int e = tid; e < BM * BK; e += 256) {
-      const int mm = sak == 1 ? e / BK : e % BM, kk = sak == 1 ? e % BK : e / BM;
-      const int m = m0 + mm, k = k0 + kk;
-      As[kk][mm] = (m < M && k < K) ? A[m * sam + k * sak] : 0.f;
-    }
-    for (int e = tid; e < BN * BK; e += 256) {
-      const int nn = sbk == 1 ? e / BK : e % BN, kk = sbk == 1 ? e % BK : e / BN;
-      const int n = n0 + nn, k = k0 + kk;
-      Bs[kk][nn] = (n < N && k < K) ? ldB<TB>(B + k * sbk + n * sbn) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
+// ---- training ------------------------------------------------------------------------------------
+// FP32 contractions C[m][n] = sum_k A(m,k) B(k,n) on the FP32 pipe: tiles of 128 x 64, 128 threads of
+// 8 x 8 outputs (64 multiply-adds per four 16-byte shared loads), k blocks of 16 prefetched into
+// registers while the previous block is used, and the reduction split over blockIdx.z so that two CTAs
+// fit each SM (the layers' 512 x 512 outputs are 32 tiles).  The kernels that consume C add the
+// partial-sum planes in order.  Operands are contiguous along k (AK, BK: rows of the batch, weights)
+// or along m / n (the weight gradient reads dZ^T H without a transpose); row pitches are multiples of
+// four floats (eight BF16) and padded with zeros.
+//   n = 2048, width 512, batch 512, one step: 1615 us on 64 x 64 tiles of 4 x 4 outputs with neither
+//   split nor prefetch. TF32 hi/lo operands on the tensor cores took 293 us, but their accumulator
+//   truncates: the loss came out 1.3e-6 from the 64-bit value (FP32: 1.7e-7), so they were left out.
+constexpr int GM = 128, GN = 64, GK = 16, GT = 128;
+
+__device__ __forceinline__ void unpack8(const uint4& q, float (&v)[8]) {
+  const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
+    v[2 * i] = __uint_as_float(w[i] << 16);
+    v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+  }
+}
+
+// TB: float or BF16 weights.  lda, ldb: row pitches (rows of m for AK, else of k; rows of n for BK,
+// else of k).  C planes [z][M][ldc].
+template <bool AK, bool BK, typename TB>
+__global__ void __launch_bounds__(GT, 2) train_gemm_kernel(int M, int N, int K, const float* A, int lda, const TB* B,
+                                                           int ldb, float* C, int ldc, size_t plane, int kper) {
+  constexpr bool BH = sizeof(TB) == 2;
+  __shared__ __align__(16) float As[2][GK][GM + 4];
+  __shared__ __align__(16) float Bs[2][GK][GN + 4];
+  const int t = threadIdx.x, tx = t % 8, ty = t / 8;
+  const int m0 = blockIdx.y * GM, n0 = blockIdx.x * GN;
+  const int k_beg = blockIdx.z * kper, k_end = min(K, k_beg + kper);
+  float4 ra[4];
+  float4 rb[2];
+  uint4 rh;
+  const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if constexpr (AK) {  // row m, four k
+        const int m = m0 + t / 4 + 32 * q, k = k0 + (t % 4) * 4;
+        ra[q] = (m < M && k < k_end) ? *reinterpret_cast<const float4*>(A + (size_t)m * lda + k) : z4;
+      } else {  // row k, four m
+        const int k = k0 + t / 32 + 4 * q, m = m0 + (t % 32) * 4;
+        ra[q] = (k < k_end && m < M) ? *reinterpret_cast<const float4*>(A + (size_t)k * lda + m) : z4;
+      }
+    }
+    if constexpr (BH) {
+      if constexpr (BK) {  // row n, eight k
+        const int n = n0 + t / 2, k = k0 + (t % 2) * 8;
+        rh = (n < N && k < k_end) ? *reinterpret_cast<const uint4*>(B + (size_t)n * ldb + k) : make_uint4(0, 0, 0, 0);
+      } else {  // row k, eight n
+        const int k = k0 + t / 8, n = n0 + (t % 8) * 8;
+        rh = (k < k_end && n < N) ? *reinterpret_cast<const uint4*>(B + (size_t)k * ldb + n) : make_uint4(0, 0, 0, 0);
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {  // row k, four n
+        const int k = k0 + t / 16 + 8 * q, n = n0 + (t % 16) * 4;
+        rb[q] = (k < k_end && n < N) ? *reinterpret_cast<const float4*>(B + (size_t)k * ldb + n) : z4;
+      }
+    }
+  };
+  auto store = [&](int s) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if constexpr (AK) {
+        const int m = t / 4 + 32 * q, k = (t % 4) * 4;
+        As[s][k][m] = ra[q].x; As[s][k + 1][m] = ra[q].y; As[s][k + 2][m] = ra[q].z; As[s][k + 3][m] = ra[q].w;
+      } else {
+        *reinterpret_cast<float4*>(&As[s][t / 32 + 4 * q][(t % 32) * 4]) = ra[q];
+      }
+    }
+    if constexpr (BH) {
+      float v[8];
+      unpack8(rh, v);
+      if constexpr (BK) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) Bs[s][(t % 2) * 8 + i][t / 2] = v[i];
+      } else {
+        *reinterpret_cast<float4*>(&Bs[s][t / 8][(t % 8) * 8]) = make_float4(v[0], v[1], v[2], v[3]);
+        *reinterpret_cast<float4*>(&Bs[s][t / 8][(t % 8) * 8 + 4]) = make_float4(v[4], v[5], v[6], v[7]);
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) *reinterpret_cast<float4*>(&Bs[s][t / 16 + 8 * q][(t % 16) * 4]) = rb[q];
+    }
+  };
+  float acc[8][8] = {};
+  load(k_beg);
+  store(0);
+  __syncthreads();
+  int s = 0;
+  for (int k0 = k_beg; k0 < k_end; k0 += GK, s ^= 1) {
+    const bool more = k0 + GK < k_end;
+    if (more) load(k0 + GK);
+#pragma unroll
+    for (int kk = 0; kk < GK; ++kk) {
+      const float4 a0 = *reinterpret_cast<const float4*>(&As[s][kk][ty * 4]);
+      const float4 a1 = *reinterpret_cast<const float4*>(&As[s][kk][64 + ty * 4]);
+      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[s][kk][tx * 4]);
+      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[s][kk][32 + tx * 4]);
+      const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+      const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    }
+    if (more) {
+      store(s ^ 1);
+      __syncthreads();
+    }
+  }
+  float* out = C + blockIdx.z * plane;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int m = m0 + (i / 4) * 64 + ty * 4 + i % 4;
     if (m >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= N) continue;
-      float v = acc[i][j] + (bias ? bias[n] : 0.f);
-      const size_t idx = (size_t)m * ldc + n;
-      if (pre) pre[idx] = v;
-      if (gelu_on) v = gelu(v);
-      C[idx] = acc_out ? C[idx] + v : v;
+    for (int h = 0; h < 2; ++h) {
+      const int n = n0 + h * 32 + tx * 4;
+      if (n < ldc)  // the pitch's padding columns get sums of zero columns
+        *reinterpret_cast<float4*>(out + (size_t)m * ldc + n) =
+            make_float4(acc[i][4 * h], acc[i][4 * h + 1], acc[i][4 * h + 2], acc[i][4 * h + 3]);
     }
   }
 }
 
-template <typename TB>
-inline void gemm(cudaStream_t s, int M, int N, int K, const float* A, long long sam, long long sak, const TB* B,
-                 long long sbk, long long sbn, float* C, int ldc, const float* bias = nullptr, float* pre = nullptr,
-                 bool gelu_on = false, bool acc_out = false) {
-  const dim3 grid((N + 63) / 64, (M + 63) / 64);
-  gemm_kernel<TB><<<grid, 256, 0, s>>>(M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, bias, pre, gelu_on, acc_out);
+__device__ __forceinline__ float plane_sum(const float* Z, int splits, size_t plane, size_t e) {
+  float v = 0.f;
+  for (int z = 0; z < splits; ++z) v += Z[z * plane + e];
+  return v;
+}
+__device__ __forceinline__ float4 plane_sum4(const float* Z, int splits, size_t plane, size_t e) {
+  float4 v = *reinterpret_cast<const float4*>(Z + e);
+  for (int z = 1; z < splits; ++z) {
+    const float4 u = *reinterpret_cast<const float4*>(Z + z * plane + e);
+    v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+  }
+  return v;
 }
 
-// features: x0[b] = [ n y_b / sum(y_b), log sum(y_b) ]  (one CTA per row)
-__global__ void features_kernel(const float* y, int n, float* x0) {
+// features: x0[b] = [ n y_b / sum(y_b), log sum(y_b) ]  (one CTA per row, pitch ld)
+__global__ void __launch_bounds__(256) features_kernel(const float* y, int n, float* x0, int ld) {
   __shared__ float red[32];
   const int b = blockIdx.x;
   float s = 0.f;
   for (int i = threadIdx.x; i < n; i += blockDim.x) s += y[(size_t)b * n + i];
   s = block_sum(s, red);
   const float inv = s > 0.f ? (float)n / s : 0.f;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) x0[(size_t)b * (n + 1) + i] = y[(size_t)b * n + i] * inv;
-  if (threadIdx.x == 0) x0[(size_t)b * (n + 1) + n] = s > 0.f ? logf(s) : 0.f;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) x0[(size_t)b * ld + i] = y[(size_t)b * n + i] * inv;
+  if (threadIdx.x == 0) x0[(size_t)b * ld + n] = s > 0.f ? logf(s) : 0.f;
 }
 
-// loss and output gradient: d = 2 (z - t_norm) / count over unmasked entries; per-CTA partial
-// loss sums and counts (deterministic: reduced in a fixed order by loss_finish_kernel).
-__global__ void loss_kernel(const float* z, const float* t, const float* mean, const float* std_, int rows, int cols,
-                            float* dz, float* part_loss, float* part_cnt) {
+// Elementwise kernels over [rows][dout] in groups of four columns (pitch ld, a multiple of four;
+// padding columns stay 0): grid.x covers ld / 4, grid.y the rows.
+// hidden layer: pre = Z + bias (kept for the backward pass), h = GELU(pre)
+__global__ void __launch_bounds__(128) act_train_kernel(const float* Z, int splits, size_t plane, int dout, int ld,
+                                                        const float* bias, float* pre, float* h) {
+  const int c = (blockIdx.x * 128 + threadIdx.x) * 4;
+  if (c >= ld) return;
+  const size_t e = (size_t)blockIdx.y * ld + c;
+  const float4 v4 = plane_sum4(Z, splits, plane, e);
+  float v[4] = {v4.x, v4.y, v4.z, v4.w}, g[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    v[q] += c + q < dout ? bias[c + q] : 0.f;
+    g[q] = c + q < dout ? gelu(v[q]) : 0.f;
+  }
+  *reinterpret_cast<float4*>(pre + e) = make_float4(v[0], v[1], v[2], v[3]);
+  *reinterpret_cast<float4*>(h + e) = make_float4(g[0], g[1], g[2], g[3]);
+}
+// output layer and loss: z = Z + bias, dz = z - t_norm over unmasked entries (0 elsewhere; the scale
+// 2 / count enters with the gradients); a row's sum of squares and count go to part[row]
+__global__ void __launch_bounds__(256) loss_train_kernel(const float* Z, int splits, size_t plane, int dout, int ld,
+                                                         const float* bias, const float* t, const float* mean,
+                                                         const float* std_, float* dz, float2* part) {
   __shared__ float red[32];
+  const int b = blockIdx.x;
   float l = 0.f, c = 0.f;
-  const size_t total = (size_t)rows * cols;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const int j = (int)(e % cols);
-    const float tv = t[e];
+  for (int f = threadIdx.x; f < ld; f += 256) {
+    const size_t e = (size_t)b * ld + f;
+    if (f >= dout) {
+      dz[e] = 0.f;
+      continue;
+    }
+    const float v = plane_sum(Z, splits, plane, e) + bias[f], tv = t[(size_t)b * dout + f];
     const bool ok = isfinite(tv);
-    const float r = ok ? z[e] - (tv - mean[j]) / std_[j] : 0.f;
-    dz[e] = r;  // scaled by 2/count in loss_scale_kernel
+    const float r = ok ? v - (tv - mean[f]) / std_[f] : 0.f;
+    dz[e] = r;
     l += r * r;
     c += ok ? 1.f : 0.f;
   }
   l = block_sum(l, red);
   c = block_sum(c, red);
+  if (threadIdx.x == 0) part[b] = make_float2(l, c);
+}
+__global__ void __launch_bounds__(256) loss_finish_kernel(const float2* part, int parts, float* loss_scale) {
+  __shared__ float red[32];
+  float l = 0.f, c = 0.f;
+  for (int i = threadIdx.x; i < parts; i += 256) {
+    l += part[i].x;
+    c += part[i].y;
+  }
+  l = block_sum(l, red);
+  c = block_sum(c, red);
   if (threadIdx.x == 0) {
-    part_loss[blockIdx.x] = l;
-    part_cnt[blockIdx.x] = c;
+    loss_scale[0] = c > 0.f ? l / c : 0.f;    // loss
+    loss_scale[1] = c > 0.f ? 2.f / c : 0.f;  // gradient scale
   }
 }
+// dZ of a hidden layer: (dZ W) * GELU'(pre)
+__global__ void __launch_bounds__(128) gelu_back_kernel(const float* Z, int splits, size_t plane, int din, int ld,
+                                                        const float* pre, float* dz) {
+  const int c = (blockIdx.x * 128 + threadIdx.x) * 4;
+  if (c >= ld) return;
+  const size_t e = (size_t)blockIdx.y * ld + c;
+  const float4 v = plane_sum4(Z, splits, plane, e), p = *reinterpret_cast<const float4*>(pre + e);
+  *reinterpret_cast<float4*>(dz + e) =
+      make_float4(v.x * gelu_grad(p.x), c + 1 < din ? v.y * gelu_grad(p.y) : 0.f, c + 2 < din ? v.z * gelu_grad(p.z) : 0.f,
+                  c + 3 < din ? v.w * gelu_grad(p.w) : 0.f);
+}
 
-__global__ void loss_finish_kernel(const float* part_loss, const float* part_cnt, int parts, float* loss_scale) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    float l = 0.f, c = 0.f;
-    for (int i = 0; i < parts; ++i) {
-      l += part_loss[i];
-      c += part_cnt[i];
-    }
-    loss_scale[0] = c > 0.f ? l / c : 0.f;      // loss
-    loss_scale[1] = c > 0.f ? 2.f / c : 0.f;    // gradient scale
+// A layer's gradient, 2 / count times: dW from its partial-sum planes [dout][pitch] (CTAs below
+// wblocks) and db_o = sum_b dZ_bo (32 columns per CTA above).  With step == 0 it is written to G;
+// otherwise AdamW runs on it directly: the FP32 master parameters, the moments, and the BF16 copy of
+// the weights (row pitch inp) that the forward passes read.
+struct LayerUpdate {
+  const float* Z;
+  int splits, pitch, dout, din, batch, ldz, wblocks, inp;
+  size_t plane;
+  const float* dz;
+  const float* scale;
+  float *G, *P, *M, *V;      // the layer's weights, then its biases
+  __nv_bfloat16* w16;
+  int step;                  // 0: write G; 1: AdamW
+  float lr, b1, b2, eps, wd, bc1, bc2;
+};
+__device__ __forceinline__ float layer_step(const LayerUpdate& A, size_t e, float gr) {
+  if (!A.step) {
+    A.G[e] = gr;
+    return 0.f;
   }
+  const float mm = A.b1 * A.M[e] + (1.f - A.b1) * gr;
+  const float vv = A.b2 * A.V[e] + (1.f - A.b2) * gr * gr;
+  A.M[e] = mm;
+  A.V[e] = vv;
+  const float p = A.P[e], upd = (mm / A.bc1) / (sqrtf(vv / A.bc2) + A.eps);
+  const float np = p - A.lr * (upd + A.wd * p);
+  A.P[e] = np;
+  return np;
 }
-
-__global__ void scale_kernel(float* v, size_t count, const float* scale) {
-  const float s = *scale;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x)
-    v[e] *= s;
-}
-
-// dH *= GELU'(pre)
-__global__ void gelu_back_kernel(float* dh, const float* pre, size_t count) {
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x)
-    dh[e] *= gelu_grad(pre[e]);
-}
-
-// db[j] = sum_b dz[b][j]  (one thread per column)
-__global__ void colsum_rows_kernel(const float* dz, int rows, int cols, float* db) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= cols) return;
-  float s = 0.f;
-  for (int b = 0; b < rows; ++b) s += dz[(size_t)b * cols + j];
-  db[j] = s;
-}
-
-// AdamW on the FP32 master parameters, then the BF16 copy of each weight used by the forward pass.
-__global__ void adamw_kernel(float* p, const float* g, float* m, float* v, __nv_bfloat16* p16, size_t count, float lr,
-                             float b1, float b2, float eps, float wd, float bc1, float bc2) {
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x) {
-    const float gr = g[e];
-    const float mm = b1 * m[e] + (1.f - b1) * gr;
-    const float vv = b2 * v[e] + (1.f - b2) * gr * gr;
-    m[e] = mm;
-    v[e] = vv;
-    const float upd = (mm / bc1) / (sqrtf(vv / bc2) + eps);
-    const float np = p[e] - lr * (upd + wd * p[e]);
-    p[e] = np;
-    p16[e] = __float2bfloat16_rn(np);
+__global__ void __launch_bounds__(256) layer_update_kernel(LayerUpdate A) {
+  const float s = *A.scale;
+  if ((int)blockIdx.x < A.wblocks) {
+    for (int o = blockIdx.x; o < A.dout; o += A.wblocks)
+      for (int i = threadIdx.x; i < A.din; i += 256) {
+        const float np = layer_step(A, (size_t)o * A.din + i, s * plane_sum(A.Z, A.splits, A.plane, (size_t)o * A.pitch + i));
+        if (A.step) A.w16[(size_t)o * A.inp + i] = __float2bfloat16_rn(np);
+      }
+    return;
+  }
+  __shared__ float red[8][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, o = ((int)blockIdx.x - A.wblocks) * 32 + lane;
+  float a = 0.f;
+  if (o < A.dout)
+    for (int b = warp; b < A.batch; b += 8) a += A.dz[(size_t)b * A.ldz + o];
+  red[warp][lane] = a;
+  __syncthreads();
+  if (warp == 0 && o < A.dout) {
+    a = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) a += red[w][lane];
+    (void)layer_step(A, (size_t)A.dout * A.din + o, s * a);
   }
 }
 
 __global__ void fill_kernel(float* p, size_t count, float v) {
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x)
     p[e] = v;
-}
-
-__global__ void to_bf16_kernel(const float* p, __nv_bfloat16* p16, size_t count) {
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x)
-    p16[e] = __float2bfloat16_rn(p[e]);
 }
 
 // Deterministic initialisation: uniform(-a, a) from a counter-based hash (splitmix64 of

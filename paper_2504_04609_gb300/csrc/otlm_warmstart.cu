@@ -21,11 +21,9 @@ struct otlm_ws_ctx {
   size_t woff[LAYERS] = {}, boff[LAYERS] = {}, nparams = 0;
   void* mem = nullptr;
   float *P = nullptr, *G = nullptr, *M = nullptr, *V = nullptr;
-  __nv_bfloat16* P16 = nullptr;
-  float* act[LAYERS + 1] = {};
+  float* zout = nullptr;           // [batch_max][n + k] the last layer's outputs (inference)
   float* pre[LAYERS] = {};
-  float* dh[2] = {};
-  float *mean = nullptr, *stdv = nullptr, *part = nullptr, *loss_scale = nullptr;
+  float *mean = nullptr, *stdv = nullptr, *loss_scale = nullptr;
   long long step = 0;
   // tensor-core forward pass (inference): padded BF16 weights, a zero lo part, activations as BF16
   // hi/lo pairs (ping-pong), split partial sums, and the GEMMs' error flag
@@ -36,63 +34,100 @@ struct otlm_ws_ctx {
   __nv_bfloat16 *Hhi[2] = {}, *Hlo[2] = {};
   float* Zs = nullptr;             // [TC_MAX_SPLITS][batch_max][dmax]
   int* tc_err = nullptr;
-  bool tc_dirty = true;
+  bool dirty = true;               // W16p is stale (parameters set from outside since the last refresh)
+  // training: the layers' inputs and the current dZ (ping-pong), row pitches of multiples of four with
+  // zero padding, and the partial sums of a weight gradient
+  int xp[LAYERS + 1] = {};
+  float *X[LAYERS] = {}, *dZ[2] = {}, *Gs = nullptr;
+  size_t gs_floats = 0;
+  float2* lpart = nullptr;
   // per-output normalisation statistics: FP64 partial sums and counts per (row chunk, output)
   double* norm_part = nullptr;
-  int* norm_cnt = nullptr;            // W16p is stale (weights changed since the last refresh)
+  int* norm_cnt = nullptr;
 };
 
 namespace {
 
-constexpr int LOSS_PARTS = 296;
-
 size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
-void forward(otlm_ws_ctx* w, int batch, const float* y) {
-  cudaStream_t s = w->stream;
-  features_kernel<<<batch, 256, 0, s>>>(y, w->n, w->act[0]);
-  for (int l = 0; l < LAYERS; ++l) {
-    const int din = w->d[l], dout = w->d[l + 1];
-    const bool hidden = l < LAYERS - 1;
-    gemm<__nv_bfloat16>(s, batch, dout, din, w->act[l], din, 1, w->P16 + w->woff[l], 1, din, w->act[l + 1], dout,
-                        w->P + w->boff[l], hidden ? w->pre[l + 1] : nullptr, hidden);
-  }
+int pitch4(int v) { return (v + 3) / 4 * 4; }
+
+// The BF16 weights of both passes after the parameters were set from outside.
+void refresh_weights(otlm_ws_ctx* w) {
+  if (!w->dirty) return;
+  for (int l = 0; l < LAYERS; ++l)
+    pad_bf16_kernel<<<1184, 256, 0, w->stream>>>(w->P + w->woff[l], w->d[l + 1], w->d[l], w->inp[l], w->W16p[l]);
+  w->dirty = false;
 }
 
-// forward, loss and gradients into w->G; loss (and 2/count) in w->loss_scale
-void backward(otlm_ws_ctx* w, int batch, const float* y, const float* target) {
+// One training GEMM: partial-sum planes [splits][M][ldc], the reduction split so that two CTAs fit
+// each SM, with at most `room` floats of planes.
+template <bool AK, bool BK, typename TB>
+void train_gemm(cudaStream_t s, int M, int N, int K, const float* A, int lda, const TB* B, int ldb, float* C, int ldc,
+                size_t room, int* splits, size_t* plane) {
+  const int tiles = ((M + GM - 1) / GM) * ((N + GN - 1) / GN), kb = (K + GK - 1) / GK;
+  int z = 2 * otlm::tc::num_sms() / tiles;
+  z = z > kb / 2 ? kb / 2 : z;
+  z = z > TC_MAX_SPLITS ? TC_MAX_SPLITS : z;
+  *plane = (size_t)M * ldc;
+  while (z > 1 && z * *plane > room) --z;
+  z = z < 1 ? 1 : z;
+  const int per = (kb + z - 1) / z;
+  z = (kb + per - 1) / per;
+  *splits = z;
+  train_gemm_kernel<AK, BK, TB><<<dim3((N + GN - 1) / GN, (M + GM - 1) / GM, z), GT, 0, s>>>(M, N, K, A, lda, B, ldb, C,
+                                                                                            ldc, *plane, per * GK);
+}
+
+// forward, loss and gradients: into w->G (u.step == 0) or straight into AdamW's step; loss (and
+// 2/count) in w->loss_scale.  u carries the optimiser's scalars.
+cudaError_t backward(otlm_ws_ctx* w, int batch, const float* y, const float* target, LayerUpdate u) {
   cudaStream_t s = w->stream;
-  forward(w, batch, y);
-  const int dz = w->d[LAYERS];
-  loss_kernel<<<LOSS_PARTS, 256, 0, s>>>(w->act[LAYERS], target, w->mean, w->stdv, batch, dz, w->dh[0], w->part,
-                                         w->part + LOSS_PARTS);
-  loss_finish_kernel<<<1, 32, 0, s>>>(w->part, w->part + LOSS_PARTS, LOSS_PARTS, w->loss_scale);
-  scale_kernel<<<1184, 256, 0, s>>>(w->dh[0], (size_t)batch * dz, w->loss_scale + 1);
-  int cur = 0;
-  for (int l = LAYERS - 1; l >= 0; --l) {
-    const int din = w->d[l], dout = w->d[l + 1];
-    float* dcur = w->dh[cur];
-    // dW[o][i] = sum_b dcur[b][o] act[l][b][i]
-    gemm<float>(s, dout, din, batch, dcur, 1, dout, w->act[l], din, 1, w->G + w->woff[l], din);
-    colsum_rows_kernel<<<(dout + 255) / 256, 256, 0, s>>>(dcur, batch, dout, w->G + w->boff[l]);
-    if (l > 0) {
-      float* dnext = w->dh[cur ^ 1];
-      // dprev[b][i] = sum_o dcur[b][o] W[o][i]  (the BF16 weights the forward pass used)
-      gemm<__nv_bfloat16>(s, batch, din, dout, dcur, dout, 1, w->P16 + w->woff[l], din, 1, dnext, din);
-      gelu_back_kernel<<<1184, 256, 0, s>>>(dnext, w->pre[l], (size_t)batch * din);
-      cur ^= 1;
+  const size_t zroom = (size_t)TC_MAX_SPLITS * w->batch_max * w->dmax;
+  refresh_weights(w);
+  features_kernel<<<batch, 256, 0, s>>>(y, w->n, w->X[0], w->xp[0]);
+  int splits = 1;
+  size_t plane = 0;
+  for (int l = 0; l < LAYERS; ++l) {
+    const int din = w->d[l], dout = w->d[l + 1], ld = w->xp[l + 1];
+    train_gemm<true, true, __nv_bfloat16>(s, batch, dout, din, w->X[l], w->xp[l], w->W16p[l], w->inp[l], w->Zs, ld, zroom,
+                                          &splits, &plane);
+    const float* bias = w->P + w->boff[l];
+    if (l < LAYERS - 1) {
+      act_train_kernel<<<dim3((ld + 511) / 512, batch), 128, 0, s>>>(w->Zs, splits, plane, dout, ld, bias, w->pre[l + 1],
+                                                                     w->X[l + 1]);
+    } else {
+      loss_train_kernel<<<batch, 256, 0, s>>>(w->Zs, splits, plane, dout, ld, bias, target, w->mean, w->stdv, w->dZ[0],
+                                              w->lpart);
+      loss_finish_kernel<<<1, 256, 0, s>>>(w->lpart, batch, w->loss_scale);
     }
   }
+  int cur = 0;
+  for (int l = LAYERS - 1; l >= 0; --l) {
+    const int din = w->d[l], dout = w->d[l + 1], ldz = w->xp[l + 1], ldx = w->xp[l];
+    const float* dz = w->dZ[cur];
+    if (l > 0) {  // dH[b][i] = sum_o dZ[b][o] W[o][i], before the layer's weights are stepped
+      train_gemm<true, false, __nv_bfloat16>(s, batch, din, dout, dz, ldz, w->W16p[l], w->inp[l], w->Zs, ldx, zroom, &splits,
+                                             &plane);
+      gelu_back_kernel<<<dim3((ldx + 511) / 512, batch), 128, 0, s>>>(w->Zs, splits, plane, din, ldx, w->pre[l],
+                                                                      w->dZ[cur ^ 1]);
+    }
+    // dW[o][i] = sum_b dZ[b][o] X[b][i]
+    train_gemm<false, false, float>(s, dout, din, batch, dz, ldz, w->X[l], ldx, w->Gs, ldx, w->gs_floats, &splits, &plane);
+    u.Z = w->Gs; u.splits = splits; u.plane = plane; u.pitch = ldx; u.dout = dout; u.din = din; u.batch = batch;
+    u.dz = dz; u.ldz = ldz; u.scale = w->loss_scale + 1; u.wblocks = dout < 1184 ? dout : 1184; u.inp = w->inp[l];
+    u.G = w->G + w->woff[l]; u.P = w->P + w->woff[l]; u.M = w->M + w->woff[l]; u.V = w->V + w->woff[l];
+    u.w16 = w->W16p[l];
+    layer_update_kernel<<<u.wblocks + (dout + 31) / 32, 256, 0, s>>>(u);
+    cur ^= 1;
+  }
+  return cudaGetLastError();
 }
 
-// Forward pass on the tensor cores into w->act[LAYERS] (inference only: no pre-activations).
+// Forward pass on the tensor cores into w->zout (inference only: no pre-activations).
 cudaError_t forward_tc(otlm_ws_ctx* w, int batch, const float* y) {
   cudaStream_t s = w->stream;
-  if (w->tc_dirty) {
-    for (int l = 0; l < LAYERS; ++l)
-      pad_bf16_kernel<<<1184, 256, 0, s>>>(w->P + w->woff[l], w->d[l + 1], w->d[l], w->inp[l], w->W16p[l]);
-    w->tc_dirty = false;
-  }
+  refresh_weights(w);
   cudaError_t e = cudaMemsetAsync(w->tc_err, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   features_split_kernel<<<batch, 256, 0, s>>>(y, w->n, w->inp[0], w->Hhi[0], w->Hlo[0]);
@@ -112,7 +147,7 @@ cudaError_t forward_tc(otlm_ws_ctx* w, int batch, const float* y) {
     const bool last = l == LAYERS - 1;
     act_split_kernel<<<1184, 256, 0, s>>>(w->Zs, g.splits, plane, batch, dout, w->P + w->boff[l],
                                           last ? nullptr : w->Hhi[cur ^ 1], last ? nullptr : w->Hlo[cur ^ 1],
-                                          last ? 0 : w->inp[l + 1], last ? w->act[LAYERS] : nullptr);
+                                          last ? 0 : w->inp[l + 1], last ? w->zout : nullptr);
     cur ^= 1;
   }
   return cudaGetLastError();
@@ -132,10 +167,8 @@ int otlm_ws_create(otlm_ws* out, int n, int k, int width, int batch_max, unsigne
   w->stream = static_cast<cudaStream_t>(stream);
   const int d[LAYERS + 1] = {n + 1, width, width, width, n + k};
   size_t off = 0;
-  int dmax = 0;
   for (int l = 0; l <= LAYERS; ++l) {
     w->d[l] = d[l];
-    dmax = dmax > d[l] ? dmax : d[l];
   }
   for (int l = 0; l < LAYERS; ++l) {
     w->woff[l] = off;
@@ -144,12 +177,20 @@ int otlm_ws_create(otlm_ws* out, int n, int k, int width, int batch_max, unsigne
     off += d[l + 1];
   }
   w->nparams = off;
-  size_t bytes = 4 * align256(4 * off) + align256(2 * off);
-  size_t actb = 0;
-  for (int l = 0; l <= LAYERS; ++l) actb += align256(4 * (size_t)batch_max * d[l]);
-  for (int l = 1; l < LAYERS; ++l) actb += align256(4 * (size_t)batch_max * d[l]);
-  actb += 2 * align256(4 * (size_t)batch_max * dmax);
-  bytes += actb + 2 * align256(4 * (size_t)(n + k)) + align256(4 * 2 * LOSS_PARTS) + 256;
+  size_t bytes = 4 * align256(4 * off);
+  // training: layer inputs, pre-activations, dZ twice, partial sums of the largest weight gradient
+  size_t trainb = 0;
+  int dzp = 0;
+  for (int l = 0; l <= LAYERS; ++l) w->xp[l] = pitch4(d[l]);
+  for (int l = 0; l < LAYERS; ++l) {
+    dzp = dzp > w->xp[l + 1] ? dzp : w->xp[l + 1];
+    trainb += align256(4 * (size_t)batch_max * w->xp[l]);
+    if (l > 0) trainb += align256(4 * (size_t)batch_max * w->xp[l]);
+    const size_t g = 4 * (size_t)d[l + 1] * w->xp[l];
+    w->gs_floats = w->gs_floats > g ? w->gs_floats : g;
+  }
+  trainb += 2 * align256(4 * (size_t)batch_max * dzp) + align256(4 * w->gs_floats) + align256(8 * (size_t)batch_max);
+  bytes += trainb + align256(4 * (size_t)batch_max * d[LAYERS]) + 2 * align256(4 * (size_t)(n + k)) + 256;
   size_t w16b = 0, zero_elems = 0;
   int maxp = 0;
   for (int l = 0; l < LAYERS; ++l) {
@@ -158,7 +199,7 @@ int otlm_ws_create(otlm_ws* out, int n, int k, int width, int batch_max, unsigne
     const size_t el = (size_t)d[l + 1] * w->inp[l];
     zero_elems = zero_elems > el ? zero_elems : el;
     maxp = maxp > w->inp[l] ? maxp : w->inp[l];
-    w->dmax = w->dmax > d[l + 1] ? w->dmax : d[l + 1];
+    w->dmax = w->dmax > w->xp[l + 1] ? w->dmax : w->xp[l + 1];
   }
   bytes += w16b + align256(2 * zero_elems) + 4 * align256(2 * (size_t)batch_max * maxp) +
            align256(4 * (size_t)TC_MAX_SPLITS * batch_max * w->dmax) + 256;
@@ -173,14 +214,16 @@ int otlm_ws_create(otlm_ws* out, int n, int k, int width, int batch_max, unsigne
   w->G = (float*)take(4 * off);
   w->M = (float*)take(4 * off);
   w->V = (float*)take(4 * off);
-  w->P16 = (__nv_bfloat16*)take(2 * off);
-  for (int l = 0; l <= LAYERS; ++l) w->act[l] = (float*)take(4 * (size_t)batch_max * d[l]);
-  for (int l = 1; l < LAYERS; ++l) w->pre[l] = (float*)take(4 * (size_t)batch_max * d[l]);
-  w->dh[0] = (float*)take(4 * (size_t)batch_max * dmax);
-  w->dh[1] = (float*)take(4 * (size_t)batch_max * dmax);
+  w->zout = (float*)take(4 * (size_t)batch_max * d[LAYERS]);
+  char* zeroed = p;  // the padded training buffers, cleared below
+  for (int l = 1; l < LAYERS; ++l) w->pre[l] = (float*)take(4 * (size_t)batch_max * w->xp[l]);
+  for (int l = 0; l < LAYERS; ++l) w->X[l] = (float*)take(4 * (size_t)batch_max * w->xp[l]);
+  for (int c = 0; c < 2; ++c) w->dZ[c] = (float*)take(4 * (size_t)batch_max * dzp);
+  const size_t zeroed_bytes = p - zeroed;
+  w->Gs = (float*)take(4 * w->gs_floats);
+  w->lpart = (float2*)take(8 * (size_t)batch_max);
   w->mean = (float*)take(4 * (size_t)(n + k));
   w->stdv = (float*)take(4 * (size_t)(n + k));
-  w->part = (float*)take(4 * 2 * LOSS_PARTS);
   w->loss_scale = (float*)take(256);
   for (int l = 0; l < LAYERS; ++l) w->W16p[l] = (__nv_bfloat16*)take(2 * (size_t)d[l + 1] * w->inp[l]);
   w->zero16 = (__nv_bfloat16*)take(2 * zero_elems);
@@ -196,6 +239,7 @@ int otlm_ws_create(otlm_ws* out, int n, int k, int width, int batch_max, unsigne
   // the zero lo part of the weights, and zero padding columns of the weights and activations
   // (never read past the tensor maps' extents, cleared all the same)
   cudaError_t e = cudaMemsetAsync(w->W16p[0], 0, w16b + align256(2 * zero_elems) + 4 * align256(2 * (size_t)batch_max * maxp), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(zeroed, 0, zeroed_bytes, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(w->P, 0, 4 * off, s);
   for (int l = 0; l < LAYERS && e == cudaSuccess; ++l) {
     const float a = std::sqrt(6.f / (float)(d[l] + d[l + 1]));
@@ -204,7 +248,6 @@ int otlm_ws_create(otlm_ws* out, int n, int k, int width, int batch_max, unsigne
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(w->M, 0, 4 * off, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(w->V, 0, 4 * off, s);
-  to_bf16_kernel<<<1184, 256, 0, s>>>(w->P, w->P16, off);
   // identity normalisation (mean 0, std 1) until the caller sets one
   if (e == cudaSuccess) e = cudaMemsetAsync(w->mean, 0, 4 * (size_t)(n + k), s);
   if (e == cudaSuccess) {
@@ -248,15 +291,13 @@ int otlm_ws_set_params(otlm_ws w, const float* in) {
   if (!w || !in) return OTLM_EINVAL;
   if (cudaMemcpyAsync(w->P, in, 4 * w->nparams, cudaMemcpyDeviceToDevice, w->stream) != cudaSuccess)
     return OTLM_ECUDA;
-  to_bf16_kernel<<<1184, 256, 0, w->stream>>>(w->P, w->P16, w->nparams);
-  w->tc_dirty = true;
+  w->dirty = true;
   return cudaGetLastError() == cudaSuccess ? OTLM_OK : OTLM_ECUDA;
 }
 
 int otlm_ws_gradients(otlm_ws w, int batch, const float* y, const float* target, float* grad_out, float* loss_out) {
   if (!w || !y || !target || batch < 1 || batch > w->batch_max) return OTLM_EINVAL;
-  backward(w, batch, y, target);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = backward(w, batch, y, target, LayerUpdate{});
   if (e == cudaSuccess && grad_out)
     e = cudaMemcpyAsync(grad_out, w->G, 4 * w->nparams, cudaMemcpyDeviceToDevice, w->stream);
   if (e == cudaSuccess && loss_out) e = cudaMemcpyAsync(loss_out, w->loss_scale, 4, cudaMemcpyDeviceToDevice, w->stream);
@@ -267,14 +308,11 @@ int otlm_ws_train_step(otlm_ws w, int batch, const float* y, const float* target
                        float* loss_out) {
   if (!w || !y || !target || batch < 1 || batch > w->batch_max || !(lr > 0) || !(weight_decay >= 0))
     return OTLM_EINVAL;
-  backward(w, batch, y, target);
   w->step += 1;
-  const float b1 = 0.9f, b2 = 0.999f;
-  const float bc1 = 1.f - std::pow(b1, (float)w->step), bc2 = 1.f - std::pow(b2, (float)w->step);
-  adamw_kernel<<<1184, 256, 0, w->stream>>>(w->P, w->G, w->M, w->V, w->P16, w->nparams, (float)lr, b1, b2, 1e-8f,
-                                            (float)weight_decay, bc1, bc2);
-  w->tc_dirty = true;
-  cudaError_t e = cudaGetLastError();
+  LayerUpdate u{};
+  u.step = 1; u.lr = (float)lr; u.b1 = 0.9f; u.b2 = 0.999f; u.eps = 1e-8f; u.wd = (float)weight_decay;
+  u.bc1 = 1.f - std::pow(u.b1, (float)w->step); u.bc2 = 1.f - std::pow(u.b2, (float)w->step);
+  cudaError_t e = backward(w, batch, y, target, u);
   if (e == cudaSuccess && loss_out) e = cudaMemcpyAsync(loss_out, w->loss_scale, 4, cudaMemcpyDeviceToDevice, w->stream);
   return e == cudaSuccess ? OTLM_OK : OTLM_ECUDA;
 }
@@ -282,7 +320,7 @@ int otlm_ws_train_step(otlm_ws w, int batch, const float* y, const float* target
 int otlm_ws_predict(otlm_ws w, int batch, const float* y, double eps, const float* cold_w, float* g0, float* w0) {
   if (!w || !y || !cold_w || !g0 || !w0 || batch < 1 || batch > w->batch_max || !(eps > 0)) return OTLM_EINVAL;
   if (forward_tc(w, batch, y) != cudaSuccess) return OTLM_ECUDA;
-  decode_kernel<<<1184, 256, 0, w->stream>>>(w->act[LAYERS], w->mean, w->stdv, batch, w->n, w->k, (float)eps, cold_w,
+  decode_kernel<<<1184, 256, 0, w->stream>>>(w->zout, w->mean, w->stdv, batch, w->n, w->k, (float)eps, cold_w,
                                              g0, w0, w->tc_err);
   return cudaGetLastError() == cudaSuccess ? OTLM_OK : OTLM_ECUDA;
 }
