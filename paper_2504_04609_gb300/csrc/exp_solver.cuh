@@ -121,6 +121,9 @@ __device__ __forceinline__ float exa_tf32(float x) {
   return __uint_as_float(r);
 }
 
+#ifndef EXA_MINB
+#define EXA_MINB 7
+#endif
 // Sum over the CTA's T warps, the same in every thread.
 template <int T>
 __device__ __forceinline__ float exa_sum(float v, float* red) {
@@ -133,7 +136,7 @@ __device__ __forceinline__ float exa_sum(float v, float* red) {
 }
 
 template <int EPI, bool TC, int T>
-__global__ void __launch_bounds__(32 * T) ex_apply_kernel(ExArgs A) {
+__global__ void __launch_bounds__(32 * T, T == 4 ? EXA_MINB : 1) ex_apply_kernel(ExArgs A) {
   using P = Prec<float>;
   constexpr int NT = 32 * T;
   extern __shared__ __align__(16) float smem[];
@@ -298,15 +301,15 @@ static inline cudaError_t launch_ex_apply(const ExArgs& a, int batch, int sms, c
 // entry of D that is read from L2 serves PB problems, and the multiply-adds run on packed pairs of
 // problems.  Arithmetic is FP32 throughout, as in mm_kernel.
 //   phase A: a chunk of 256 rows' log ratios is staged as [row][problem]; warps take rows, lanes
-//            columns; the eight warps' sums are added in order
+//            columns; the warps' sums are added in order
 //   phase C: threads take rows (Dt is read coalesced along rows), the weights are broadcast
-constexpr int MMB_NT = 256, MMB_CHUNK = 256;
+constexpr int MMB_NT = 256, MMB_NW = MMB_NT / 32, MMB_CHUNK = MMB_NT;
 
 template <int PB, int KQ>
 struct MmbSmem {
   static constexpr int KP = 32 * KQ;
   static constexpr int RS = MMB_CHUNK * PB;                     // staged ratios
-  static constexpr int RED = 8 * KP * (PB < 4 ? PB : 4);        // warps' sums of up to 4 problems
+  static constexpr int RED = MMB_NW * KP * (PB < 4 ? PB : 4);        // warps' sums of up to 4 problems
   static constexpr int U = RS > RED ? RS : RED;
   static constexpr size_t bytes = 4 * (size_t)(U + 3 * KP * PB);  // + weights [k][PB] (new), starting weights, NU
 };
@@ -366,15 +369,24 @@ __global__ void __launch_bounds__(MMB_NT) mm_batch_kernel(MMBArgs A) {
       __syncthreads();
       const int cnt = min(MMB_CHUNK, n - c0);
       constexpr int U = KQ >= 8 ? 2 : (KQ >= 4 ? 4 : 8);
-      for (int r0 = warp * U; r0 < cnt; r0 += 8 * U) {
-        float d[U][KQ];
+      float d[U][KQ];
+      auto load = [&](int r0) {
 #pragma unroll
         for (int u = 0; u < U; ++u)
 #pragma unroll
           for (int q = 0; q < KQ; ++q) {
             const int j = lane + 32 * q;
-            d[u][q] = (r0 + u < cnt && j < k) ? A.D[(size_t)(c0 + r0 + u) * k + j] : 0.f;
+            d[u][q] = (r0 + u < cnt && j < k) ? __ldg(A.D + (size_t)(c0 + r0 + u) * k + j) : 0.f;
           }
+      };
+      load(warp * U);
+      for (int r0 = warp * U; r0 < cnt; r0 += MMB_NW * U) {
+        float cur[U][KQ];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int q = 0; q < KQ; ++q) cur[u][q] = d[u][q];
+        if (r0 + MMB_NW * U < cnt) load(r0 + MMB_NW * U);  // the next rows arrive while these are used
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const float* rr = rs + (r0 + u) * PB;  // rows past cnt were staged as 0
@@ -390,7 +402,7 @@ __global__ void __launch_bounds__(MMB_NT) mm_batch_kernel(MMBArgs A) {
           else r2[0] = f2_pack(rr[0], 0.f);
 #pragma unroll
           for (int q = 0; q < KQ; ++q) {
-            const uint64_t d2 = f2_pack(d[u][q], d[u][q]);
+            const uint64_t d2 = f2_pack(cur[u][q], cur[u][q]);
 #pragma unroll
             for (int h = 0; h < H; ++h) acc[h][q] = f2_fma(d2, r2[h], acc[h][q]);
           }
@@ -414,7 +426,7 @@ __global__ void __launch_bounds__(MMB_NT) mm_batch_kernel(MMBArgs A) {
       for (int e = tid; e < G * KP; e += MMB_NT) {
         float sum = 0.f;
 #pragma unroll
-        for (int w8 = 0; w8 < 8; ++w8) sum += rs[w8 * G * KP + e];
+        for (int w8 = 0; w8 < MMB_NW; ++w8) sum += rs[w8 * G * KP + e];
         nu_s[g * KP + e] = sum;
       }
     }
@@ -436,7 +448,7 @@ __global__ void __launch_bounds__(MMB_NT) mm_batch_kernel(MMBArgs A) {
     }
     __syncthreads();
     // ---- phase C: S = D w ----
-    constexpr int IPT = PB >= 16 ? 2 : 4;  // rows per thread
+    constexpr int IPT = 2, JB = 8;  // rows per thread, columns of D in flight
     float mass[PB];
 #pragma unroll
     for (int q = 0; q < PB; ++q) mass[q] = 0.f;
@@ -446,30 +458,34 @@ __global__ void __launch_bounds__(MMB_NT) mm_batch_kernel(MMBArgs A) {
       for (int t = 0; t < IPT; ++t)
 #pragma unroll
         for (int h = 0; h < H; ++h) s2[t][h] = 0ull;
-#pragma unroll 4
-      for (int j = 0; j < k; ++j) {
-        float d[IPT];
+      for (int j0 = 0; j0 < k; j0 += JB) {
+        float d[JB][IPT];
 #pragma unroll
-        for (int t = 0; t < IPT; ++t) {
-          const int i = c0 + t * MMB_NT + tid;
-          d[t] = i < n ? A.Dt[(size_t)j * n + i] : 0.f;
-        }
-        const float* ww = w_s + j * PB;
-        uint64_t w2[H];
-        if constexpr (PB >= 4) {
+        for (int jj = 0; jj < JB; ++jj)
 #pragma unroll
-          for (int h = 0; h < H; h += 2) {
-            const float4 v = *reinterpret_cast<const float4*>(ww + 2 * h);
-            w2[h] = f2_pack(v.x, v.y);
-            w2[h + 1] = f2_pack(v.z, v.w);
+          for (int t = 0; t < IPT; ++t) {
+            const int i = c0 + t * MMB_NT + tid;
+            d[jj][t] = (i < n && j0 + jj < k) ? __ldg(A.Dt + (size_t)(j0 + jj) * n + i) : 0.f;
           }
-        } else if constexpr (PB == 2) w2[0] = f2_pack(ww[0], ww[1]);
-        else w2[0] = f2_pack(ww[0], 0.f);
 #pragma unroll
-        for (int t = 0; t < IPT; ++t) {
-          const uint64_t d2 = f2_pack(d[t], d[t]);
+        for (int jj = 0; jj < JB; ++jj) {
+          const float* ww = w_s + min(j0 + jj, k - 1) * PB;  // (past k: times 0)
+          uint64_t w2[H];
+          if constexpr (PB >= 4) {
 #pragma unroll
-          for (int h = 0; h < H; ++h) s2[t][h] = f2_fma(d2, w2[h], s2[t][h]);
+            for (int h = 0; h < H; h += 2) {
+              const float4 v = *reinterpret_cast<const float4*>(ww + 2 * h);
+              w2[h] = f2_pack(v.x, v.y);
+              w2[h + 1] = f2_pack(v.z, v.w);
+            }
+          } else if constexpr (PB == 2) w2[0] = f2_pack(ww[0], ww[1]);
+          else w2[0] = f2_pack(ww[0], 0.f);
+#pragma unroll
+          for (int t = 0; t < IPT; ++t) {
+            const uint64_t d2 = f2_pack(d[jj][t], d[jj][t]);
+#pragma unroll
+            for (int h = 0; h < H; ++h) s2[t][h] = f2_fma(d2, w2[h], s2[t][h]);
+          }
         }
       }
 #pragma unroll
@@ -532,10 +548,11 @@ static inline cudaError_t launch_mmb_pb(const MMBArgs& a, int batch, cudaStream_
   if (a.k <= 128) return launch_mmb_cfg<PB, 4>(a, batch, s);
   return launch_mmb_cfg<PB, 8>(a, batch, s);
 }
-// Problems per CTA: one while the batch does not fill the SMs, then as many as leave one CTA per SM.
+// Problems per CTA: one while the batch does not fill the SMs, then as many as leave two CTAs per SM
+// (latency of the loads of D) and, for the largest batches, eight (traffic of D).
 static inline cudaError_t launch_mm_batch(const MMBArgs& a, int batch, int sms, cudaStream_t s) {
   if (batch <= sms) return launch_mmb_pb<1>(a, batch, s);
-  if (batch <= 4 * sms) return launch_mmb_pb<4>(a, batch, s);
+  if (batch <= 16 * sms) return launch_mmb_pb<4>(a, batch, s);
   return launch_mmb_pb<8>(a, batch, s);
 }
 
