@@ -59,4 +59,18 @@ cudaError_t ex_apply_target(const ExArgs& a, int batch, bool tc, int sms, cudaSt
 cudaError_t ex_ratio(const ExArgs& a, int batch, cudaStream_t stream);
 cudaError_t mm_batch(const MMBArgs& a, int batch, int sms, cudaStream_t stream);
 
+// A small batch sharing grid, dictionary and eps solved in one launch (ragged.cuh, compiled in
+// otlm_api.cu); outputs as otlm_solve, any of g, t_out, iters, err, status, dw may be null.
+struct SmallSolve {
+  int batch, n, k, datafit, penalty, max_iter, mm_steps;
+  double eps, lam, alpha, beta, tol;
+  const float *x, *D, *y;
+  float *w, *g, *t_out;
+  int* iters;
+  float* err;
+  int* status;
+  float* dw;
+};
+cudaError_t small_solve(const SmallSolve& c, cudaStream_t stream);
+
 }  // namespace otlm

@@ -279,6 +279,19 @@ void ragged_args(otlm_ctx* h, int batch, const int* n, const int* k, const float
 
 }  // namespace
 
+namespace otlm {
+cudaError_t small_solve(const SmallSolve& c, cudaStream_t stream) {
+  RaggedArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.batch = c.batch; a.x = c.x; a.D = c.D; a.y = c.y; a.w = c.w; a.g_in = c.g; a.g_out = c.g; a.t_out = c.t_out;
+  a.iters = c.iters; a.err = c.err; a.status = c.status; a.dw = c.dw;
+  a.datafit = c.datafit; a.penalty = c.penalty; a.max_iter = c.max_iter;
+  a.lam = (float)c.lam; a.alpha = (float)c.alpha; a.tol = (float)c.tol; a.beta = (float)c.beta; a.mm_steps = c.mm_steps;
+  a.n_all = c.n; a.k_all = c.k; a.eps_all = (float)c.eps; a.xs_all = (float)(1.0 / std::sqrt(c.eps * kLn2));
+  return ragged_small(a, stream);
+}
+}  // namespace otlm
+
 extern "C" {
 
 int otlm_create(otlm_handle* out, const otlm_config* cfg, void* cuda_stream) {

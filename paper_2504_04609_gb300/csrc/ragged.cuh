@@ -52,6 +52,10 @@ struct RaggedArgs {
   int n_max, k_max;
   long long tot_n, tot_D, tot_k;  // packed sizes of x/y, D and w (sum n, sum n k, sum k)
   int smem_floats;                // dynamic shared memory of the launch, in floats
+  // a small batch sharing one grid, dictionary and eps (n == null; one CTA per problem, no queue)
+  int n_all, k_all;
+  float eps_all, xs_all;          // xs_all = 1 / sqrt(eps ln2)
+  float* dw;                      // [batch] weight change of the last update, or null
   // rows per thread by size bucket (n in (256 b, 256 (b + 1)]), as log2 R; raised to the fewest
   // that cover n with this CTA size (0: always the fewest)
   unsigned char rows_log2[16];
@@ -68,7 +72,7 @@ struct RaggedSmem {
   }
   // everything but the expansion's scratch, rounded up to 16 bytes
   static __host__ __device__ size_t state(int n_max, int k_max) {
-    return (6 * (size_t)n_max + 2 * (size_t)k_max + (NT / 32) * (size_t)k_max + 64 + 3) / 4 * 4;
+    return (6 * (size_t)n_max + 3 * (size_t)k_max + (NT / 32) * (size_t)k_max + 64 + 3) / 4 * 4;
   }
 };
 
@@ -312,10 +316,13 @@ __device__ __noinline__ float ragged_dw_any(const float* D, const float* W, cons
 template <int NT, int R>
 __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
   using P = Prec<float>;
-  const int n = A.n[p], k = A.k[p];
-  const float eps = A.eps[p];
+  const bool shared = A.n == nullptr;
+  const int n = shared ? A.n_all : A.n[p], k = shared ? A.k_all : A.k[p];
+  const float eps = shared ? A.eps_all : A.eps[p];
   const float eps_ln2 = eps * float(kLn2);
-  const long long on = A.off_n[p], oD = A.off_D[p], ok = A.off_k[p];
+  const long long on = shared ? (long long)p * n : A.off_n[p], oD = shared ? 0 : A.off_D[p],
+                  ok = shared ? (long long)p * k : A.off_k[p];
+  const float* x = A.x + (shared ? 0 : on);
   // a problem whose sizes or offsets fall outside the packed arrays is marked invalid and not
   // touched; the barrier also separates the previous problem's last reads from this one's writes
   const bool valid = n >= 2 && n <= A.n_max && k >= 1 && k <= A.k_max && (n + NT - 1) / NT <= R && on >= 0 &&
@@ -339,16 +346,17 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
   float* S = LB2 + A.n_max;
   float* W = S + A.n_max;
   float* xcol = W + A.k_max;
-  float* red_k = xcol + A.k_max;  // [NT/32][k_max]
+  float* Wp = xcol + A.k_max;     // weights before the last update
+  float* red_k = Wp + A.k_max;    // [NT/32][k_max]
   float* red = red_k + (NT / 32) * A.k_max;  // 32 floats + scalars
   float* scr = sm + RaggedSmem<NT>::state(A.n_max, A.k_max);  // the expansion's scratch
   __shared__ ExPlan plan_s;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int NW = NT / 32;
 
-  const float xs = rsqrtf(eps_ln2);
+  const float xs = shared ? A.xs_all : rsqrtf(eps_ln2);
   for (int i = tid; i < n; i += NT) {
-    xt[i] = A.x[on + i] * xs;
+    xt[i] = x[i] * xs;
     G2[i] = A.g_in ? A.g_in[on + i] / eps_ln2 : 0.f;
   }
   for (int j = tid; j < k; j += NT) W[j] = A.w[ok + j];
@@ -408,6 +416,7 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
         for (int w8 = 0; w8 < NW; ++w8) sum += red_k[w8 * A.k_max + j];
         const float xj = xcol[j];
         const float dl = sum * float(kLn2) / xj;
+        if (m == 0) Wp[j] = W[j];
         const float nu = P::log(W[j]) + dl;
         const float shift = (A.penalty == PEN_L1 || A.penalty == PEN_ELASTIC) ? A.alpha / (eps * xj) : 0.f;
         float wn;
@@ -458,10 +467,20 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
     if (A.g_out) A.g_out[on + i] = G2[i] * eps_ln2;
     if (A.t_out) A.t_out[on + i] = it > 0 ? P::exp2(G2[i] + LB2[i]) : 0.f;
   }
+  if (A.dw) {  // ||w - w_before||_1 / ||w||_1 of the last update
+    float num = 0.f, den = 0.f;
+    for (int j = tid; j < k; j += NT) {
+      num += fabsf(W[j] - Wp[j]);
+      den += fabsf(W[j]);
+    }
+    num = block_sum_f(num, red);
+    den = block_sum_f(den, red);
+    if (tid == 0) A.dw[p] = it > 0 ? num / den : CUDART_NAN_F;
+  }
   if (tid == 0) {
-    A.iters[p] = it;
-    A.err[p] = e;
-    A.status[p] = st;
+    if (A.iters) A.iters[p] = it;
+    if (A.err) A.err[p] = e;
+    if (A.status) A.status[p] = st;
   }
   __syncthreads();
 }
@@ -472,14 +491,20 @@ template <int NT, int RMAX>
 __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) ragged_kernel(RaggedArgs A) {
   extern __shared__ __align__(16) float sm[];
   __shared__ int s_idx;
-  for (;;) {
-    if (threadIdx.x == 0) s_idx = atomicAdd(A.next, 1);
-    __syncthreads();
-    const int idx = s_idx;
-    __syncthreads();
-    if (idx >= A.batch) break;
-    const int p = A.order[idx];
-    const int n = A.n[p];
+  const bool shared = A.n == nullptr;  // one CTA per problem, no queue
+  for (bool first = true;; first = false) {
+    int p = blockIdx.x;
+    if (shared) {
+      if (!first) break;
+    } else {
+      if (threadIdx.x == 0) s_idx = atomicAdd(A.next, 1);
+      __syncthreads();
+      const int idx = s_idx;
+      __syncthreads();
+      if (idx >= A.batch) break;
+      p = A.order[idx];
+    }
+    const int n = shared ? A.n_all : A.n[p];
     // rows per thread: the tuned choice for n's size bucket, at least the fewest that cover n
     // (more rows per thread amortise each column's shared-memory reads over more exponentials,
     // fewer keep more threads busy)
@@ -491,7 +516,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) ragged_kernel(RaggedArg
     else if (RMAX >= 8 && rows <= 8) ragged_solve_one<NT, (RMAX >= 8 ? 8 : 2)>(A, p, sm);
     else if (RMAX >= 16 && rows <= 16) ragged_solve_one<NT, (RMAX >= 16 ? 16 : 2)>(A, p, sm);
     else if (RMAX >= 32 && rows <= 32) ragged_solve_one<NT, (RMAX >= 32 ? 32 : 2)>(A, p, sm);
-    else if (threadIdx.x == 0) {  // more rows per thread than this CTA size supports
+    else if (threadIdx.x == 0 && !shared) {  // more rows per thread than this CTA size supports
       A.iters[p] = 0;
       A.err[p] = CUDART_NAN_F;
       A.status[p] = ST_INVALID;
@@ -520,6 +545,25 @@ inline cudaError_t ragged_prepare(int v, int n_max, int k_max, int* blocks_per_s
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, nt, bytes);
   *smem = bytes;
   return e;
+}
+
+// A small batch sharing grid, dictionary and eps, whole solves in one launch (one CTA per problem).
+// The smallest calls are latency: an iteration of three launches is 20 to 30 us whatever its size,
+// while a CTA that keeps its problem in shared memory pays barriers only.
+inline cudaError_t ragged_small(const RaggedArgs& a0, cudaStream_t s) {
+  RaggedArgs a = a0;
+  const int v = a.n_all <= 512 ? 1 : 2;
+  int bps = 0;
+  size_t smem = 0;
+  const cudaError_t e = ragged_prepare(v, a.n_all, a.k_all, &bps, &smem);
+  if (e != cudaSuccess) return e;
+  if (bps < 1) return cudaErrorInvalidConfiguration;
+  a.n_max = a.n_all; a.k_max = a.k_all;
+  a.tot_n = (long long)a.batch * a.n_all; a.tot_D = (long long)a.n_all * a.k_all; a.tot_k = (long long)a.batch * a.k_all;
+  a.smem_floats = (int)(smem / 4);
+  if (v == 1) ragged_kernel<256, 16><<<a.batch, 256, smem, s>>>(a);
+  else ragged_kernel<512, 8><<<a.batch, 512, smem, s>>>(a);
+  return cudaGetLastError();
 }
 
 inline void ragged_launch(int v, dim3 grid, size_t smem, cudaStream_t s, const RaggedArgs& a) {

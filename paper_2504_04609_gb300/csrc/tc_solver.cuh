@@ -722,6 +722,19 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
   const int batch = sp.batch, n = sp.n, k = sp.k;
   const double eps_ln2 = sp.eps * kLn2;
   const bool checks = ow && sp.check_every > 0;
+  // small batches: whole solves in one launch, as on an FP32 handle (with more than one problem per SM
+  // of a long grid the batched kernels below win)
+  if (sp.single_until == 0.0 && ex_serves(sp, C != nullptr, checks) && small_prefers(sp, sm_count()) &&
+      (batch <= sm_count() || n <= 2048)) {
+    const SmallSolve sc{batch, n, k, sp.datafit, sp.penalty, sp.max_iter, sp.mm_steps, sp.eps, sp.lam, sp.alpha, sp.beta,
+                        sp.tol, x, D, y, w, g, t_out, iters_out, err_out, status_out, ws.dw};
+    L.begin(KIND_APPLY);
+    cudaError_t r = small_solve(sc, L.stream);
+    L.end();
+    if (r == cudaSuccess) r = cudaStreamSynchronize(L.stream);
+    if (r == cudaSuccess && L.timer && L.timer->on) r = L.timer->harvest();
+    return r;
+  }
   PrepArgs<float> pa;
   pa.x = x; pa.D = D; pa.w_in = w; pa.g_in = g; pa.y = y;
   pa.xt = ws.xt; pa.Dt = ws.Dt; pa.xcol = ws.xcol; pa.W = ws.W; pa.G2 = ws.G2;
