@@ -183,13 +183,13 @@ __global__ void __launch_bounds__(256) features_kernel(const float* y, int n, fl
 }
 
 // Elementwise kernels over [rows][dout] in groups of four columns (pitch ld, a multiple of four;
-// padding columns stay 0): grid.x covers ld / 4, grid.y the rows.
+// padding columns stay 0): grid.x = rows, grid.y covers ld / 4.
 // hidden layer: pre = Z + bias (kept for the backward pass), h = GELU(pre)
 __global__ void __launch_bounds__(128) act_train_kernel(const float* Z, int splits, size_t plane, int dout, int ld,
                                                         const float* bias, float* pre, float* h) {
-  const int c = (blockIdx.x * 128 + threadIdx.x) * 4;
+  const int c = (blockIdx.y * 128 + threadIdx.x) * 4;
   if (c >= ld) return;
-  const size_t e = (size_t)blockIdx.y * ld + c;
+  const size_t e = (size_t)blockIdx.x * ld + c;
   const float4 v4 = plane_sum4(Z, splits, plane, e);
   float v[4] = {v4.x, v4.y, v4.z, v4.w}, g[4];
 #pragma unroll
@@ -242,9 +242,9 @@ __global__ void __launch_bounds__(256) loss_finish_kernel(const float2* part, in
 // dZ of a hidden layer: (dZ W) * GELU'(pre)
 __global__ void __launch_bounds__(128) gelu_back_kernel(const float* Z, int splits, size_t plane, int din, int ld,
                                                         const float* pre, float* dz) {
-  const int c = (blockIdx.x * 128 + threadIdx.x) * 4;
+  const int c = (blockIdx.y * 128 + threadIdx.x) * 4;
   if (c >= ld) return;
-  const size_t e = (size_t)blockIdx.y * ld + c;
+  const size_t e = (size_t)blockIdx.x * ld + c;
   const float4 v = plane_sum4(Z, splits, plane, e), p = *reinterpret_cast<const float4*>(pre + e);
   *reinterpret_cast<float4*>(dz + e) =
       make_float4(v.x * gelu_grad(p.x), c + 1 < din ? v.y * gelu_grad(p.y) : 0.f, c + 2 < din ? v.z * gelu_grad(p.z) : 0.f,
@@ -326,8 +326,8 @@ __global__ void init_kernel(float* p, size_t count, float a, unsigned long long 
 }
 
 // ---- tensor-core forward pass (inference) ------------------------------------------------------
-// Each layer is Z = H W^T on gemm3_kernel<KIND_BF16> with A = W (the BF16 weights; their lo part
-// is an all-zero buffer, so the three hi/lo products are W times the activations to ~16 bits) and
+// Each layer is Z = H W^T on gemm3_kernel<KIND_BF16> with A = W (the BF16 weights, exact: two products
+// give W times the activations to ~16 bits) and
 // B = the activations as a BF16 hi/lo pair, K-major with a row pitch padded to 8 elements (TMA
 // rows are 16-byte multiples).  Z may be split over the reduction (partial-sum planes); the
 // activation kernel adds the planes in order, the bias and GELU, and writes the next operand.
@@ -360,33 +360,49 @@ __global__ void features_split_kernel(const float* y, int n, int inp, __nv_bfloa
   if (threadIdx.x == 0) split_bf16(s > 0.f ? logf(s) : 0.f, hhi + row + n, hlo + row + n);
 }
 
-// v = sum over the `splits` partial-sum planes of Z [rows][dout] + bias; hidden layers write
-// GELU(v) as the next BF16 hi/lo operand (row pitch outp), the last layer writes v to zout.
-__global__ void act_split_kernel(const float* Z, int splits, size_t plane, int rows, int dout, const float* bias,
-                                 __nv_bfloat16* ohi, __nv_bfloat16* olo, int outp, float* zout) {
-  const size_t total = (size_t)rows * dout;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const int b = (int)(e / dout), f = (int)(e - (size_t)b * dout);
-    float v = 0.f;
-    for (int z = 0; z < splits; ++z) v += Z[z * plane + e];
-    v += bias[f];
-    if (zout) zout[e] = v;
-    else split_bf16(gelu(v), ohi + (size_t)b * outp + f, olo + (size_t)b * outp + f);
+// Hidden layer: v = sum over the `splits` planes of Z [rows][dout] + bias, GELU(v) as the next BF16
+// hi/lo operand (row pitch outp, a multiple of eight). grid.x = row, four columns per thread.
+__global__ void __launch_bounds__(256) act_split_kernel(const float* Z, int splits, size_t plane, int dout,
+                                                        const float* bias, __nv_bfloat16* ohi, __nv_bfloat16* olo,
+                                                        int outp) {
+  const int f0 = (blockIdx.y * 256 + threadIdx.x) * 4;
+  if (f0 >= dout) return;
+  const size_t e = (size_t)blockIdx.x * dout + f0, o = (size_t)blockIdx.x * outp + f0;
+  float v[4] = {0.f, 0.f, 0.f, 0.f};
+  const bool vec = dout % 4 == 0 && plane % 4 == 0;  // 16-byte aligned rows and planes
+  for (int z = 0; z < splits; ++z) {
+    if (vec) {
+      const float4 q = *reinterpret_cast<const float4*>(Z + z * plane + e);
+      v[0] += q.x; v[1] += q.y; v[2] += q.z; v[3] += q.w;
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (f0 + c < dout) v[c] += Z[z * plane + e + c];
+    }
   }
+  __align__(8) __nv_bfloat16 hi[4], lo[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) split_bf16(f0 + c < dout ? gelu(v[c] + bias[f0 + c]) : 0.f, hi + c, lo + c);
+  *reinterpret_cast<uint2*>(ohi + o) = *reinterpret_cast<uint2*>(hi);  // padding columns get zeros
+  *reinterpret_cast<uint2*>(olo + o) = *reinterpret_cast<uint2*>(lo);
 }
 
-// predictions -> warm start: g0 = eps * (z * std + mean) for the first n outputs (the potential
-// g / eps), w0 = exp(z * std + mean) for the last k (log w); non-finite predictions fall back to
-// the cold start (g0 = 0, w0 = cold_w) so that a bad network can only cost iterations, and so does
-// every row when *fail is set (a tensor-core GEMM of the forward pass gave up a wait).
-__global__ void decode_kernel(const float* z, const float* mean, const float* std_, int rows, int n, int k, float eps,
-                              const float* cold_w, float* g0, float* w0, const int* fail) {
-  const int cols = n + k;
-  const size_t total = (size_t)rows * cols;
+// Output layer -> warm start: z = sum over the planes + bias; g0 = eps * (z * std + mean) for the first
+// n outputs (the potential g / eps), w0 = exp(z * std + mean) for the last k (log w); non-finite
+// predictions fall back to the cold start (g0 = 0, w0 = cold_w) so that a bad network can only cost
+// iterations, and so does every row when *fail is set (a GEMM of the forward pass gave up a wait).
+// grid.x = row, 256 threads over 1024 outputs.
+__global__ void __launch_bounds__(256) decode_kernel(const float* Z, int splits, size_t plane, const float* bias,
+                                                     const float* mean, const float* std_, int n, int k, float eps,
+                                                     const float* cold_w, float* g0, float* w0, const int* fail) {
+  const int cols = n + k, b = blockIdx.x;
   const bool failed = fail && *fail;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const int b = (int)(e / cols), j = (int)(e % cols);
-    const float v = failed ? CUDART_NAN_F : z[e] * std_[j] + mean[j];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int j = blockIdx.y * 1024 + q * 256 + threadIdx.x;
+    if (j >= cols) continue;
+    const float z = plane_sum(Z, splits, plane, (size_t)b * cols + j) + bias[j];
+    const float v = failed ? CUDART_NAN_F : z * std_[j] + mean[j];
     if (j < n) {
       g0[(size_t)b * n + j] = isfinite(v) ? eps * v : 0.f;
     } else {

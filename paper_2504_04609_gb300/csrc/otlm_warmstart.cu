@@ -21,16 +21,14 @@ struct otlm_ws_ctx {
   size_t woff[LAYERS] = {}, boff[LAYERS] = {}, nparams = 0;
   void* mem = nullptr;
   float *P = nullptr, *G = nullptr, *M = nullptr, *V = nullptr;
-  float* zout = nullptr;           // [batch_max][n + k] the last layer's outputs (inference)
   float* pre[LAYERS] = {};
   float *mean = nullptr, *stdv = nullptr, *loss_scale = nullptr;
   long long step = 0;
-  // tensor-core forward pass (inference): padded BF16 weights, a zero lo part, activations as BF16
+  // tensor-core forward pass (inference): padded BF16 weights, activations as BF16
   // hi/lo pairs (ping-pong), split partial sums, and the GEMMs' error flag
   int inp[LAYERS] = {};            // row pitch of layer l's input operand (d[l] rounded up to 8)
   int dmax = 0;                    // widest layer output
   __nv_bfloat16* W16p[LAYERS] = {};
-  __nv_bfloat16* zero16 = nullptr;
   __nv_bfloat16 *Hhi[2] = {}, *Hlo[2] = {};
   float* Zs = nullptr;             // [TC_MAX_SPLITS][batch_max][dmax]
   int* tc_err = nullptr;
@@ -94,7 +92,7 @@ cudaError_t backward(otlm_ws_ctx* w, int batch, const float* y, const float* tar
                                           &splits, &plane);
     const float* bias = w->P + w->boff[l];
     if (l < LAYERS - 1) {
-      act_train_kernel<<<dim3((ld + 511) / 512, batch), 128, 0, s>>>(w->Zs, splits, plane, dout, ld, bias, w->pre[l + 1],
+      act_train_kernel<<<dim3(batch, (ld + 511) / 512), 128, 0, s>>>(w->Zs, splits, plane, dout, ld, bias, w->pre[l + 1],
                                                                      w->X[l + 1]);
     } else {
       loss_train_kernel<<<batch, 256, 0, s>>>(w->Zs, splits, plane, dout, ld, bias, target, w->mean, w->stdv, w->dZ[0],
@@ -109,7 +107,7 @@ cudaError_t backward(otlm_ws_ctx* w, int batch, const float* y, const float* tar
     if (l > 0) {  // dH[b][i] = sum_o dZ[b][o] W[o][i], before the layer's weights are stepped
       train_gemm<true, false, __nv_bfloat16>(s, batch, din, dout, dz, ldz, w->W16p[l], w->inp[l], w->Zs, ldx, zroom, &splits,
                                              &plane);
-      gelu_back_kernel<<<dim3((ldx + 511) / 512, batch), 128, 0, s>>>(w->Zs, splits, plane, din, ldx, w->pre[l],
+      gelu_back_kernel<<<dim3(batch, (ldx + 511) / 512), 128, 0, s>>>(w->Zs, splits, plane, din, ldx, w->pre[l],
                                                                       w->dZ[cur ^ 1]);
     }
     // dW[o][i] = sum_b dZ[b][o] X[b][i]
@@ -124,8 +122,8 @@ cudaError_t backward(otlm_ws_ctx* w, int batch, const float* y, const float* tar
   return cudaGetLastError();
 }
 
-// Forward pass on the tensor cores into w->zout (inference only: no pre-activations).
-cudaError_t forward_tc(otlm_ws_ctx* w, int batch, const float* y) {
+// Forward pass on the tensor cores, decoded into the warm start (inference only).
+cudaError_t forward_tc(otlm_ws_ctx* w, int batch, const float* y, float eps, const float* cold_w, float* g0, float* w0) {
   cudaStream_t s = w->stream;
   refresh_weights(w);
   cudaError_t e = cudaMemsetAsync(w->tc_err, 0, sizeof(int), s);
@@ -137,17 +135,25 @@ cudaError_t forward_tc(otlm_ws_ctx* w, int batch, const float* y) {
     const int din = w->d[l], dout = w->d[l + 1];
     otlm::tc::GemmArgs g{};
     g.out = w->Zs; g.M = dout; g.N = batch; g.Kd = din; g.ld_out = dout; g.err = w->tc_err;
-    g.splits = otlm::tc::choose_splits(((dout + otlm::tc::BM - 1) / otlm::tc::BM) * ((batch + otlm::tc::BN - 1) / otlm::tc::BN),
-                                       (din + 63) / 64);
+    // split the reduction only as far as the tiles leave SMs idle (every split is a plane of FP32 sums:
+    // 4096 rows ran as seven planes of 8 MB in the input layer and eight of 35 MB in the output layer),
+    // and drain the accumulators after every k block
+    const int tiles = ((dout + otlm::tc::BM - 1) / otlm::tc::BM) * ((batch + otlm::tc::BN - 1) / otlm::tc::BN);
+    const int want = otlm::tc::num_sms() / tiles, nkb = (din + 63) / 64;
+    g.splits = want < 1 ? 1 : (want > nkb ? nkb : want);
+    g.chunk = 1;
     if (g.splits > TC_MAX_SPLITS) g.splits = TC_MAX_SPLITS;
+    g.a_exact = 1;  // BF16 weights: two products
     g.split_stride = plane;
-    e = otlm::tc::launch_gemm3<otlm::tc::KIND_BF16>(w->W16p[l], w->zero16, w->inp[l], w->Hhi[cur], w->Hlo[cur],
+    e = otlm::tc::launch_gemm3<otlm::tc::KIND_BF16>(w->W16p[l], w->W16p[l], w->inp[l], w->Hhi[cur], w->Hlo[cur],
                                                     w->inp[l], dout, batch, din, g, s);
     if (e != cudaSuccess) return e;
-    const bool last = l == LAYERS - 1;
-    act_split_kernel<<<1184, 256, 0, s>>>(w->Zs, g.splits, plane, batch, dout, w->P + w->boff[l],
-                                          last ? nullptr : w->Hhi[cur ^ 1], last ? nullptr : w->Hlo[cur ^ 1],
-                                          last ? 0 : w->inp[l + 1], last ? w->zout : nullptr);
+    if (l < LAYERS - 1)
+      act_split_kernel<<<dim3(batch, (dout + 1023) / 1024), 256, 0, s>>>(w->Zs, g.splits, plane, dout, w->P + w->boff[l],
+                                                                        w->Hhi[cur ^ 1], w->Hlo[cur ^ 1], w->inp[l + 1]);
+    else
+      decode_kernel<<<dim3(batch, (dout + 1023) / 1024), 256, 0, s>>>(w->Zs, g.splits, plane, w->P + w->boff[l], w->mean, w->stdv,
+                                                                     w->n, w->k, eps, cold_w, g0, w0, w->tc_err);
     cur ^= 1;
   }
   return cudaGetLastError();
@@ -190,18 +196,16 @@ int otlm_ws_create(otlm_ws* out, int n, int k, int width, int batch_max, unsigne
     w->gs_floats = w->gs_floats > g ? w->gs_floats : g;
   }
   trainb += 2 * align256(4 * (size_t)batch_max * dzp) + align256(4 * w->gs_floats) + align256(8 * (size_t)batch_max);
-  bytes += trainb + align256(4 * (size_t)batch_max * d[LAYERS]) + 2 * align256(4 * (size_t)(n + k)) + 256;
-  size_t w16b = 0, zero_elems = 0;
+  bytes += trainb + 2 * align256(4 * (size_t)(n + k)) + 256;
+  size_t w16b = 0;
   int maxp = 0;
   for (int l = 0; l < LAYERS; ++l) {
     w->inp[l] = (d[l] + 7) / 8 * 8;
     w16b += align256(2 * (size_t)d[l + 1] * w->inp[l]);
-    const size_t el = (size_t)d[l + 1] * w->inp[l];
-    zero_elems = zero_elems > el ? zero_elems : el;
     maxp = maxp > w->inp[l] ? maxp : w->inp[l];
     w->dmax = w->dmax > w->xp[l + 1] ? w->dmax : w->xp[l + 1];
   }
-  bytes += w16b + align256(2 * zero_elems) + 4 * align256(2 * (size_t)batch_max * maxp) +
+  bytes += w16b + 4 * align256(2 * (size_t)batch_max * maxp) +
            align256(4 * (size_t)TC_MAX_SPLITS * batch_max * w->dmax) + 256;
   bytes += align256(8 * (size_t)NORM_CHUNKS * (n + k)) + align256(4 * (size_t)NORM_CHUNKS * (n + k));
   if (cudaMalloc(&w->mem, bytes) != cudaSuccess) {
@@ -214,7 +218,6 @@ int otlm_ws_create(otlm_ws* out, int n, int k, int width, int batch_max, unsigne
   w->G = (float*)take(4 * off);
   w->M = (float*)take(4 * off);
   w->V = (float*)take(4 * off);
-  w->zout = (float*)take(4 * (size_t)batch_max * d[LAYERS]);
   char* zeroed = p;  // the padded training buffers, cleared below
   for (int l = 1; l < LAYERS; ++l) w->pre[l] = (float*)take(4 * (size_t)batch_max * w->xp[l]);
   for (int l = 0; l < LAYERS; ++l) w->X[l] = (float*)take(4 * (size_t)batch_max * w->xp[l]);
@@ -226,7 +229,6 @@ int otlm_ws_create(otlm_ws* out, int n, int k, int width, int batch_max, unsigne
   w->stdv = (float*)take(4 * (size_t)(n + k));
   w->loss_scale = (float*)take(256);
   for (int l = 0; l < LAYERS; ++l) w->W16p[l] = (__nv_bfloat16*)take(2 * (size_t)d[l + 1] * w->inp[l]);
-  w->zero16 = (__nv_bfloat16*)take(2 * zero_elems);
   for (int c = 0; c < 2; ++c) {
     w->Hhi[c] = (__nv_bfloat16*)take(2 * (size_t)batch_max * maxp);
     w->Hlo[c] = (__nv_bfloat16*)take(2 * (size_t)batch_max * maxp);
@@ -236,9 +238,8 @@ int otlm_ws_create(otlm_ws* out, int n, int k, int width, int batch_max, unsigne
   w->norm_part = (double*)take(8 * (size_t)NORM_CHUNKS * (n + k));
   w->norm_cnt = (int*)take(4 * (size_t)NORM_CHUNKS * (n + k));
   cudaStream_t s = w->stream;
-  // the zero lo part of the weights, and zero padding columns of the weights and activations
-  // (never read past the tensor maps' extents, cleared all the same)
-  cudaError_t e = cudaMemsetAsync(w->W16p[0], 0, w16b + align256(2 * zero_elems) + 4 * align256(2 * (size_t)batch_max * maxp), s);
+  // zero padding columns of the weights and activations
+  cudaError_t e = cudaMemsetAsync(w->W16p[0], 0, w16b + 4 * align256(2 * (size_t)batch_max * maxp), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(zeroed, 0, zeroed_bytes, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(w->P, 0, 4 * off, s);
   for (int l = 0; l < LAYERS && e == cudaSuccess; ++l) {
@@ -319,10 +320,7 @@ int otlm_ws_train_step(otlm_ws w, int batch, const float* y, const float* target
 
 int otlm_ws_predict(otlm_ws w, int batch, const float* y, double eps, const float* cold_w, float* g0, float* w0) {
   if (!w || !y || !cold_w || !g0 || !w0 || batch < 1 || batch > w->batch_max || !(eps > 0)) return OTLM_EINVAL;
-  if (forward_tc(w, batch, y) != cudaSuccess) return OTLM_ECUDA;
-  decode_kernel<<<1184, 256, 0, w->stream>>>(w->zout, w->mean, w->stdv, batch, w->n, w->k, (float)eps, cold_w,
-                                             g0, w0, w->tc_err);
-  return cudaGetLastError() == cudaSuccess ? OTLM_OK : OTLM_ECUDA;
+  return forward_tc(w, batch, y, (float)eps, cold_w, g0, w0) == cudaSuccess ? OTLM_OK : OTLM_ECUDA;
 }
 
 int otlm_ws_make_targets(otlm_ws w, int batch, const float* g, const float* wts, double eps, double g_floor,

@@ -49,6 +49,8 @@ constexpr int A_TILE = BM * BK_BYTES;                     // 16 KiB
 constexpr int B_TILE = BN * BK_BYTES;                     // 16 KiB
 constexpr int STAGE_BYTES = 2 * A_TILE + 2 * B_TILE;      // 64 KiB: A hi, B hi, A lo, B lo
 constexpr int STAGES_SINGLE = STAGE_BYTES * STAGES / (A_TILE + B_TILE);  // 6 stages of A hi, B hi
+constexpr int STAGE_TWO = A_TILE + 2 * B_TILE;                            // 48 KiB: A hi, B hi, B lo
+constexpr int STAGES_TWO = STAGE_BYTES * STAGES / STAGE_TWO;              // 4
 constexpr int EPI_BYTES = 64 * BM * 4;                    // 32 KiB: 64 output columns of 128 rows
 constexpr int NBARS = 2 * STAGES_SINGLE + 5;              // full[6], empty[6], acc_full[2], acc_empty[2], drain
 constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + EPI_BYTES + NBARS * 8 + 16;
@@ -183,6 +185,11 @@ struct GemmArgs {
   int bulk;            // set by launch_gemm3: every output column segment is 16-byte aligned and a
                        // multiple of 16 bytes long, so the tile leaves through shared memory as
                        // one bulk copy per column
+  int chunk;           // > 0 (gemm3_kernel): the accumulator is drained every `chunk` k blocks and the
+                       // chunks are added in FP32 registers: the tensor cores' accumulator truncates, so
+                       // its chain of additions, not the operands, would set the error
+  int a_exact;         // A has no lo part (BF16 weights): the two products Ahi Bhi + Ahi Blo, A_lo unread
+                       // (gemm3_kernel only)
   const int* hilo;     // null: the three products; otherwise, while *hilo == 0 (read at launch),
                        // the single product hi x hi: only the hi tiles are loaded
   int store_direct;    // 1: the epilogue stores from registers, one 128-byte segment per warp and
@@ -298,9 +305,10 @@ __global__ void __launch_bounds__(THREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ncols = g.n_cols ? *g.n_cols : g.N;
   const bool three = !g.hilo || *g.hilo != 0;  // the three products, or hi x hi alone
-  const int nst = three ? STAGES : STAGES_SINGLE;  // ring stages of this launch
+  const bool two = three && g.a_exact;                          // Ahi (Bhi + Blo)
+  const int nst = two ? STAGES_TWO : three ? STAGES : STAGES_SINGLE;  // ring stages of this launch
   const unsigned long long lim = g.wait_ns ? g.wait_ns : WAIT_NS;
-  const uint32_t st_bytes = three ? STAGE_BYTES : A_TILE + B_TILE;
+  const uint32_t st_bytes = two ? STAGE_TWO : three ? STAGE_BYTES : A_TILE + B_TILE;
   const int mt = (g.M + BM - 1) / BM, nt = (g.N + BN - 1) / BN;
   const int units = mt * nt * g.splits;
   const int nkb_all = (g.Kd + BK - 1) / BK;
@@ -332,7 +340,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   auto a_hi = [&](int s) { return ring + static_cast<uint32_t>(s) * st_bytes; };
   auto b_hi = [&](int s) { return a_hi(s) + A_TILE; };
   auto a_lo = [&](int s) { return a_hi(s) + A_TILE + B_TILE; };
-  auto b_lo = [&](int s) { return a_hi(s) + 2 * A_TILE + B_TILE; };
+  auto b_lo = [&](int s) { return a_hi(s) + (two ? A_TILE + B_TILE : 2 * A_TILE + B_TILE); };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES_SINGLE; ++s) {
@@ -386,7 +394,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           tma_load_2d(a_hi(s), &tA_hi, full0 + 8 * s, kc, m0);
           tma_load_2d(b_hi(s), &tB_hi, full0 + 8 * s, kc, n0);
           if (three) {
-            tma_load_2d(a_lo(s), &tA_lo, full0 + 8 * s, kc, m0);
+            if (!two) tma_load_2d(a_lo(s), &tA_lo, full0 + 8 * s, kc, m0);
             tma_load_2d(b_lo(s), &tB_lo, full0 + 8 * s, kc, n0);
           }
           last_round[s] = r;
@@ -401,12 +409,13 @@ __global__ void __launch_bounds__(THREADS, 1)
   } else if (warp == 1 && lane == 0) {
     // ---- MMA issuer: unit i accumulates into TMEM columns (i & 1) * BN ----
     // One loop per product count, descriptors advanced by tile offsets (as in the two-SM kernel).
-    auto mma_role = [&](auto three_c) {
-      constexpr bool THREE = decltype(three_c)::value;
+    auto mma_role = [&](auto np_c) {
+      constexpr int NP = decltype(np_c)::value;  // products
       constexpr uint32_t id = idesc<KIND>(BM, BN);
-      constexpr uint32_t ST16 = (THREE ? STAGE_BYTES : A_TILE + B_TILE) >> 4;
-      constexpr int NST = THREE ? STAGES : STAGES_SINGLE;
-      constexpr uint32_t O_BH = A_TILE >> 4, O_AL = (A_TILE + B_TILE) >> 4, O_BL = (2 * A_TILE + B_TILE) >> 4;
+      constexpr uint32_t ST16 = (NP == 3 ? STAGE_BYTES : NP == 2 ? STAGE_TWO : A_TILE + B_TILE) >> 4;
+      constexpr int NST = NP == 3 ? STAGES : NP == 2 ? STAGES_TWO : STAGES_SINGLE;
+      constexpr uint32_t O_BH = A_TILE >> 4, O_AL = (A_TILE + B_TILE) >> 4,
+                         O_BL = (NP == 3 ? 2 * A_TILE + B_TILE : A_TILE + B_TILE) >> 4;
       const uint64_t d_ring = sw128_desc(ring);
       uint64_t sd = d_ring;  // stage s
       int s = 0, r = 0;      // ring stage and round of the next k block
@@ -417,16 +426,22 @@ __global__ void __launch_bounds__(THREADS, 1)
         coords(u, &m0, &n0, &z);
         if (n0 >= ncols) continue;
         krange(z, &kb0, &nkb);
-        const int b = i & 1, use = i >> 1;
-        if (use >= 1 && !mbar_wait(acce0 + 8 * b, (use - 1) & 1, lim)) {  // the epilogue has drained buffer b
-          atomicCAS(g.err, 0, ERR_WAIT_ACC);
-          atomicExch(fail, 1);
-          break;
-        }
-        tc_fence_after();
-        const uint32_t d = tmem + static_cast<uint32_t>(b * BN);
+        const int ck = g.chunk > 0 ? g.chunk : nkb;  // k blocks per accumulation
+        uint32_t d = 0;
         int issued = 0;
         for (int kb = 0; kb < nkb; ++kb) {
+          if (kb % ck == 0) {  // a new accumulation, into buffer i & 1
+            const int b = i & 1, use = i >> 1;
+            if (use >= 1 && !mbar_wait(acce0 + 8 * b, (use - 1) & 1, lim)) {  // the epilogue has drained buffer b
+              atomicCAS(g.err, 0, ERR_WAIT_ACC);
+              atomicExch(fail, 1);
+              stop = true;
+              break;
+            }
+            tc_fence_after();
+            d = tmem + static_cast<uint32_t>(b * BN);
+            issued = 0;
+          }
           if (!mbar_wait(full0 + 8 * s, r & 1, lim)) {
             atomicCAS(g.err, 0, ERR_WAIT_TMA);
             atomicExch(fail, 1);
@@ -438,10 +453,8 @@ __global__ void __launch_bounds__(THREADS, 1)
           for (int kk = 0; kk < BK_BYTES / 32; ++kk) {  // 32 bytes of k per MMA: +2 in the address field
             const uint64_t ah = sd + 2 * kk, bh = sd + O_BH + 2 * kk;
             umma<KIND>(d, ah, bh, id, issued);
-            if constexpr (THREE) {
-              umma<KIND>(d, ah, sd + O_BL + 2 * kk, id, 1);
-              umma<KIND>(d, sd + O_AL + 2 * kk, bh, id, 1);
-            }
+            if constexpr (NP >= 2) umma<KIND>(d, ah, sd + O_BL + 2 * kk, id, 1);
+            if constexpr (NP == 3) umma<KIND>(d, sd + O_AL + 2 * kk, bh, id, 1);
             issued = 1;
           }
           umma_commit(empty0 + 8 * s);
@@ -451,14 +464,17 @@ __global__ void __launch_bounds__(THREADS, 1)
           } else {
             sd += ST16;
           }
+          if ((kb + 1) % ck == 0 || kb + 1 == nkb) {
+            umma_commit(accf0 + 8 * (i & 1));  // fires once the accumulation's MMAs have completed
+            ++i;
+          }
         }
         if (stop) break;
-        umma_commit(accf0 + 8 * b);  // fires once the unit's MMAs have completed
-        ++i;
       }
     };
-    if (three) mma_role(std::true_type{});
-    else mma_role(std::false_type{});
+    if (two) mma_role(std::integral_constant<int, 2>{});
+    else if (three) mma_role(std::integral_constant<int, 3>{});
+    else mma_role(std::integral_constant<int, 1>{});
     umma_commit(drain);  // fires once every MMA issued above has completed: TMEM may be released
     (void)mbar_wait(drain, 0, lim);
   } else if (warp >= 4) {
@@ -469,14 +485,62 @@ __global__ void __launch_bounds__(THREADS, 1)
       int m0, n0, z;
       coords(u, &m0, &n0, &z);
       if (n0 >= ncols) continue;
-      const int b = i & 1, use = i >> 1;
-      const bool ok = mbar_wait(accf0 + 8 * b, use & 1, lim);
-      if (!ok) atomicCAS(g.err, 0, ERR_WAIT_ACC);
-      if (bar_or_epi(!ok || *(volatile int*)fail)) {  // the four warps leave together
+      auto wait_acc = [&]() -> bool {  // the four warps leave together
+        const bool ok = mbar_wait(accf0 + 8 * (i & 1), (i >> 1) & 1, lim);
+        if (!ok) atomicCAS(g.err, 0, ERR_WAIT_ACC);
+        return !bar_or_epi(!ok || *(volatile int*)fail);
+      };
+      if (g.chunk > 0) {
+        int kb0, nkb;
+        krange(z, &kb0, &nkb);
+        float sum[BN];
+#pragma unroll
+        for (int c = 0; c < BN; ++c) sum[c] = 0.f;
+        bool stop = false;
+        for (int kb = 0; kb < nkb; kb += g.chunk) {
+          if (!wait_acc()) {
+            stop = true;
+            break;
+          }
+          tc_fence_after();
+          const int b = i & 1;
+          const uint32_t tq = tmem + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(b * BN);
+#pragma unroll
+          for (int h = 0; h < BN / 64; ++h) {
+            uint32_t v[64];
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < 4; ++j) tmem_ld16_nowait(tq + static_cast<uint32_t>(h * 64 + j * 16), v + 16 * j);
+            tmem_wait_ld(v);
+            if (h == BN / 64 - 1) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(acce0 + 8 * b);
+            }
+#pragma unroll
+            for (int c = 0; c < 64; ++c) sum[h * 64 + c] += __uint_as_float(v[c]);
+          }
+          ++i;
+        }
+        if (stop) {
+          atomicExch(fail, 1);
+          break;
+        }
+        const int row = m0 + q * 32 + lane;  // one 128-byte segment per warp and column
+        float* out = g.out + z * g.split_stride;
+#pragma unroll
+        for (int c = 0; c < BN; ++c) {
+          const int col = n0 + c;
+          if (col < ncols && row < g.M) out[static_cast<size_t>(g.col_map ? g.col_map[col] : col) * g.ld_out + row] = sum[c];
+        }
+        continue;
+      }
+      if (!wait_acc()) {
         atomicExch(fail, 1);
         break;
       }
       tc_fence_after();
+      const int b = i & 1;
       const uint32_t tq = tmem + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(b * BN);
       // once every TMEM read of buffer b is done, hand it back to the MMA warp
       epilogue_tile(g, g.out + z * g.split_stride, tq, stage_out, stage_s, m0, n0, ncols, q, lane, et,
