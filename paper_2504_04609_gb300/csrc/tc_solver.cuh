@@ -38,7 +38,10 @@ namespace otlm {
 // Small batches leave the applies with fewer 128 x 128 output tiles than SMs (a single target at
 // n = 8192 has 64), so for batches up to TC_SMALL_BATCH the reduction of each apply is split into up
 // to TC_APPLY_SPLITS ranges whose partial sums are added by tc_split_reduce_kernel.
+// Larger batches split while their tiles leave half of the SMs idle (256 problems of 1024 bins are 16
+// tiles: 23 us per apply on 8 SM pairs, 12 with the reduction over nine ranges and their sum).
 constexpr int TC_SMALL_BATCH = 64, TC_APPLY_SPLITS = 16;
+constexpr size_t TC_ACCP_FLOATS = (size_t)6 << 20;
 
 struct TcWorkspace {
   __nv_bfloat16 *Khi, *Klo;  // [n][ld]
@@ -60,7 +63,8 @@ struct TcWorkspace {
   float *Rhi, *Rlo;          // [batch][ld] log ratios by slot (B operand of D^T r)
   int ld;                    // row pitch of the [.][n] operands (multiple of 64 elements)
   int kp;                    // row pitch of the [.][k] operands (k_max rounded up to 4)
-  float* ACCP;               // [TC_APPLY_SPLITS][min(batch_max, TC_SMALL_BATCH) x n] split partial sums
+  float* ACCP;               // split partial sums of an apply: accp_floats
+  size_t accp_floats;
 };
 
 // A raw GEMM sum is a sum of positive terms, so it is >= 0.  A row the fix-up recomputed exactly
@@ -100,8 +104,12 @@ inline size_t carve_tc_workspace(void* base, int n_max, int k_max, int batch_max
   w.fix_cap = (unsigned long long)batch_max * n_max;
   w.fix_list = (int2*)take(8 * (size_t)batch_max * n_max);
   w.fix_cnt = (unsigned long long*)take(64);
-  w.ACCP = (float*)take(4 * (size_t)TC_APPLY_SPLITS * (batch_max < TC_SMALL_BATCH ? batch_max : TC_SMALL_BATCH) *
-                        n_max);
+  {  // batches up to TC_SMALL_BATCH in full, larger ones as far as TC_ACCP_FLOATS go
+    const size_t small = (size_t)TC_APPLY_SPLITS * (batch_max < TC_SMALL_BATCH ? batch_max : TC_SMALL_BATCH) * n_max;
+    const size_t all = (size_t)TC_APPLY_SPLITS * batch_max * n_max, cap = all < TC_ACCP_FLOATS ? all : TC_ACCP_FLOATS;
+    w.accp_floats = small > cap ? small : cap;
+    w.ACCP = (float*)take(4 * w.accp_floats);
+  }
   w.kp = kp;
   w.Dhi = (float*)take(4 * (size_t)n_max * kp);
   w.Dlo = (float*)take(4 * (size_t)n_max * kp);
@@ -241,25 +249,27 @@ struct TcCost {
   }
 };
 
+// In: the row's potentials, in(p, j) (an array, or formed from the sums and targets they came from: the
+// row kernels keep neither G2 nor F2, which only the rare listed rows and the returned state need).
+template <class In>
 __global__ void __launch_bounds__(256) tc_fixup_kernel(const int2* list, const unsigned long long* cnt,
                                                        unsigned long long* cnt_next, unsigned long long cap, int n,
-                                                       TcCost cost, const float* in, float* acc,
-                                                       const float* mshift) {
+                                                       TcCost cost, In in, float* acc, const float* mshift) {
   using P = Prec<float>;
   __shared__ float red[32];
   const unsigned long long c = *cnt < cap ? *cnt : cap;
   if (blockIdx.x == 0 && threadIdx.x == 0) *cnt_next = 0;
   for (unsigned long long e = blockIdx.x; e < c; e += gridDim.x) {
     const int2 pi = list[e];
-    const float* inp = in + (size_t)pi.x * n;
+    const int p = pi.x;
     float mx = -CUDART_INF_F;
 #pragma unroll 4
-    for (int j = threadIdx.x; j < n; j += blockDim.x) mx = fmaxf(mx, inp[j] - cost(pi.y, j, n));
+    for (int j = threadIdx.x; j < n; j += blockDim.x) mx = fmaxf(mx, in(p, j) - cost(pi.y, j, n));
     mx = block_max(mx, red);
     float sum = 0.f;
     if (mx > -CUDART_INF_F) {
 #pragma unroll 4
-      for (int j = threadIdx.x; j < n; j += blockDim.x) sum += P::exp2((inp[j] - mx) - cost(pi.y, j, n));
+      for (int j = threadIdx.x; j < n; j += blockDim.x) sum += P::exp2((in(p, j) - mx) - cost(pi.y, j, n));
     }
     sum = block_sum(sum, red);
     if (threadIdx.x == 0) {
@@ -290,6 +300,7 @@ struct TcIterArgs {
   float* Wprev;      // [P][k] weights before the last update
   const int* gap_ok; // [P] gap test of this iteration's check
   int gap_check, gap_on;
+  int keep_g2;       // the objective of gap checks reads G2: store it every iteration
   float dw_tol;
   float single_until;  // > 0: switch the applies to hi/lo once a violation is <= this
   int* done;
@@ -338,6 +349,29 @@ __device__ __forceinline__ float tc_datafit(const TcIterArgs& A, float v, float 
   }
 }
 
+// The potentials a fix-up sums: an array, the datafit step of the previous target sums (G2), or
+// log2 s - log2 a (F2) of this iteration's source sums.
+struct TcInArray {
+  const float* v;
+  int n;
+  __device__ __forceinline__ float operator()(int p, int j) const { return v[(size_t)p * n + j]; }
+};
+struct TcInG2 {
+  TcIterArgs A;
+  __device__ __forceinline__ float operator()(int p, int j) const {
+    const size_t o = (size_t)p * A.n + j;
+    return A.it > 0 ? tc_datafit(A, tc_log2_sum(A.t.ACC_tgt[o], A.t.Mtgt[p]), A.y[o]) : A.G2[o];
+  }
+};
+struct TcInF2 {
+  TcIterArgs A;
+  __device__ __forceinline__ float operator()(int p, int j) const {
+    const size_t o = (size_t)p * A.n + j;
+    const float s = A.S[o];
+    return s > 0.f ? Prec<float>::log2(s) - tc_log2_sum(A.t.ACC_src[A.it & 1][o], A.t.Msrc[A.it & 1][p]) : -CUDART_INF_F;
+  }
+};
+
 __device__ __forceinline__ void tc_store_operand(float v, __nv_bfloat16* hi_row, __nv_bfloat16* lo_row, int j) {
   const __nv_bfloat16 hi = __float2bfloat16_rn(v);
   hi_row[j] = hi;
@@ -377,7 +411,7 @@ __global__ void __launch_bounds__(NT) tc_prep_src_kernel(TcIterArgs A) {
       for (int e = 0; e < EPT; ++e) {
         const int j = e * NT + threadIdx.x;
         g[e] = tc_datafit(A, tc_log2_sum(a[e], mt), yv[e]);
-        if (j < n) G2[j] = g[e];
+        if (A.keep_g2 && j < n) G2[j] = g[e];
       }
     } else {
 #pragma unroll
@@ -579,7 +613,7 @@ __global__ void __launch_bounds__(NT) tc_operand_kernel(TcIterArgs A) {
   const int p = A.active[slot], n = A.n, cur = A.it & 1;
   const float* S = A.S + (size_t)p * n;
   const float* acc = A.t.ACC_src[cur] + (size_t)p * n;
-  float* F2 = A.F2 + (size_t)p * n;
+  float* F2 = A.F2 + (size_t)p * n;  // streamed rows only
   __nv_bfloat16* vhi = A.t.Vhi + (size_t)slot * A.t.ld;
   __nv_bfloat16* vlo = A.t.Vlo + (size_t)slot * A.t.ld;
   const float mc = A.t.Msrc[cur][p];
@@ -598,7 +632,6 @@ __global__ void __launch_bounds__(NT) tc_operand_kernel(TcIterArgs A) {
       for (int e = 0; e < EPT; ++e) {
         const int j = e * NT + threadIdx.x;
         f2[e] = sv[e] > 0.f ? P::log2(sv[e]) - tc_log2_sum(av[e], mc) : P::ninf();
-        if (j < n) F2[j] = f2[e];
         fm = fmaxf(fm, f2[e]);
         ms += sv[e];
       }
@@ -683,7 +716,8 @@ __global__ void tc_obj_decode_kernel(TcIterArgs A, const int* list, const int* c
 }
 
 // t = Q^T 1 = 2^{G2 + LB2}, LB2 = Mtgt + log2(target sum); w, g and the per-problem statistics.
-__global__ void tc_finalize_kernel(FinArgs<float> F, const float* ACC_tgt, const float* Mtgt) {
+// G2 is formed from the target sums again, as the last source operand had it.
+__global__ void tc_finalize_kernel(FinArgs<float> F, TcIterArgs A) {
   using P = Prec<float>;
   const size_t stride = (size_t)gridDim.x * blockDim.x;
   const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -691,11 +725,10 @@ __global__ void tc_finalize_kernel(FinArgs<float> F, const float* ACC_tgt, const
   for (size_t e = tid; e < bk; e += stride) F.w_out[e] = F.W[e];
   for (size_t e = tid; e < bn; e += stride) {
     const int p = (int)(e / F.n);
-    if (F.g_out) F.g_out[e] = F.G2[e] * F.gscale_inv;
-    if (F.t_out) {
-      const float lb = tc_log2_sum(ACC_tgt[e], Mtgt[p]);
-      F.t_out[e] = lb > -CUDART_INF_F ? P::exp2(F.G2[e] + lb) : 0.f;
-    }
+    const float lb = tc_log2_sum(A.t.ACC_tgt[e], A.t.Mtgt[p]);
+    const float g2 = tc_datafit(A, lb, A.y[e]);
+    if (F.g_out) F.g_out[e] = g2 * F.gscale_inv;
+    if (F.t_out) F.t_out[e] = lb > -CUDART_INF_F ? P::exp2(g2 + lb) : 0.f;
   }
   for (size_t e = tid; e < (size_t)F.batch; e += stride) {
     if (F.iters_out) F.iters_out[e] = F.iters[e];
@@ -796,6 +829,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
   ta.dw = ws.dw; ta.Wprev = ws.Wprev; ta.dw_tol = float(sp.dw_tol); ta.gap_on = checks && sp.gap_tol > 0;
   ta.gap_ok = checks ? ow->gap_ok : nullptr;
   ta.single_until = float(sp.single_until);
+  ta.keep_g2 = checks;
 
   // the applies K V^T (BF16): M = bins, N = slots mapped to problems, reduction over bins
   tc::GemmArgs ga{};
@@ -804,9 +838,10 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
   ga.hilo = tw.hilo;
   {
     const int units = ((n + tc::BM - 1) / tc::BM) * ((batch + tc::BN - 1) / tc::BN);
-    if (batch <= TC_SMALL_BATCH && units < tc::num_sms()) {
+    if (batch <= TC_SMALL_BATCH ? units < tc::num_sms() : 2 * units <= tc::num_sms()) {
       ga.splits = tc::choose_splits(units, (n + tc::KindTraits<tc::KIND_BF16>::BK - 1) / tc::KindTraits<tc::KIND_BF16>::BK);
       if (ga.splits > TC_APPLY_SPLITS) ga.splits = TC_APPLY_SPLITS;
+      while (ga.splits > 1 && (size_t)ga.splits * batch * n > tw.accp_floats) --ga.splits;
     }
     ga.split_stride = (size_t)batch * n;
     if (ga.splits > 1) ga.fix_list = nullptr;  // listed by tc_split_reduce_kernel instead
@@ -875,7 +910,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
     if (r != cudaSuccess) return r;
     L.begin(KIND_OTHER);
     tc_fixup_kernel<<<TC_FIX_GRID, 256, 0, L.stream>>>(tw.fix_list, tw.fix_cnt + 2, tw.fix_cnt + 3, ga.fix_cap, n,
-                                                    cost_tgt, ow->F2, ow->LB2, ow->M);
+                                                    cost_tgt, TcInArray{ow->F2, n}, ow->LB2, ow->M);
     L.end();
     L.begin(KIND_OTHER);
     tc_obj_decode_kernel<<<red_grid, 256, 0, L.stream>>>(ta, list, count, ow->LB2, ow->M, ow->G2n);
@@ -958,7 +993,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
     if (e != cudaSuccess) return e;
     L.begin(KIND_OTHER);
     tc_fixup_kernel<<<TC_FIX_GRID, 256, 0, L.stream>>>(tw.fix_list, tw.fix_cnt, tw.fix_cnt + 1, ga.fix_cap, n,
-                                                    cost_src, ws.G2, tw.ACC_src[it & 1], tw.Msrc[it & 1]);
+                                                    cost_src, TcInG2{ta}, tw.ACC_src[it & 1], tw.Msrc[it & 1]);
     L.end();
     // a check: the state (w, g) whose source sums were just computed is the one this iteration
     // returns if it stops here; its FP64 objective and gap come before the stopping decision
@@ -1012,7 +1047,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
     if (e != cudaSuccess) return e;
     L.begin(KIND_OTHER);
     tc_fixup_kernel<<<TC_FIX_GRID, 256, 0, L.stream>>>(tw.fix_list, tw.fix_cnt + 1, tw.fix_cnt, ga.fix_cap, n,
-                                                    cost_tgt, ws.F2, tw.ACC_tgt, tw.Mtgt);
+                                                    cost_tgt, TcInF2{ta}, tw.ACC_tgt, tw.Mtgt);
     L.end();
     if ((it + 1) % sp.poll_every == 0) {
       e = cudaMemcpyAsync(L.host_flag, ws.n_active, sizeof(int), cudaMemcpyDeviceToHost, L.stream);
@@ -1033,7 +1068,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
   fa.err_out = err_out; fa.batch = batch; fa.n = n; fa.k = k; fa.gscale_inv = float(eps_ln2);
   L.begin(KIND_OTHER);
   if (by_expansion) finalize_kernel<float><<<1184, 256, 0, L.stream>>>(fa);
-  else tc_finalize_kernel<<<1184, 256, 0, L.stream>>>(fa, tw.ACC_tgt, tw.Mtgt);
+  else tc_finalize_kernel<<<1184, 256, 0, L.stream>>>(fa, ta);
   L.end();
   e = cudaMemcpyAsync(L.host_flag, tw.err, sizeof(int), cudaMemcpyDeviceToHost, L.stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(L.stream);
