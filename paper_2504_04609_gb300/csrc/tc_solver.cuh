@@ -738,11 +738,13 @@ __global__ void tc_finalize_kernel(FinArgs<float> F, TcIterArgs A) {
 }
 
 // Where the expansion applies serve a tensor-core handle: small batches (one target at n = 16384, 20
-// iterations: 11.9 -> 2.3 ms, no kernel matrix to stream) and short grids (1024 problems of 1024 bins,
-// 50 iterations: 5.75 -> 5.08 ms); the GEMMs' n^2 is cheaper above. A caller who sets the precision
+// iterations: 11.9 -> 2.3 ms, no kernel matrix to stream) and batches whose GEMMs do not fill the SM
+// pairs (1024 problems of 1024 bins, 32 pair tiles, 50 iterations: 5.75 -> 4.61 ms); an apply takes the
+// expansion 27 us per million bins and a full GEMM less up to n = 4096 or so. A caller who sets the precision
 // schedule has asked for the GEMM's single product and keeps the GEMMs.
+constexpr long long TC_EXPANSION_BINS = 5 << 18;  // 1.25 million
 inline bool tc_prefers_expansion(int batch, int n, double single_until) {
-  return single_until == 0.0 && (batch <= TC_SMALL_BATCH || n <= 2048);
+  return single_until == 0.0 && (batch <= TC_SMALL_BATCH || (long long)batch * n <= TC_EXPANSION_BINS);
 }
 
 // Run Algorithm 1 with tensor-core applies and dictionary contractions (float buffers; x, D, y, w,
