@@ -320,7 +320,7 @@ int otlm_create(otlm_handle* out, const otlm_config* cfg, void* cuda_stream) {
     h->f64 = nullptr;
     (void)cudaGetLastError();
   }
-  if (cudaMallocHost(&h->host_flag, sizeof(int)) != cudaSuccess) {
+  if (cudaMallocHost(&h->host_flag, 4 * sizeof(int)) != cudaSuccess) {
     cudaFree(h->ws);
     if (h->f64) cudaFree(h->f64);
     delete h;
