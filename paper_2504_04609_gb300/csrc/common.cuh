@@ -7,6 +7,8 @@
 #include <math_constants.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace otlm {
 
 constexpr double kLn2 = 0.69314718055994530942;
@@ -127,6 +129,31 @@ template <typename T>
 __device__ __forceinline__ T wright_omega_of(T z) {
   if constexpr (sizeof(T) == 8) return wright_omega_f64(z);
   else return wright_omega<T>(z);
+}
+
+// Programmatic dependent launch: the kernels of an iteration are launched while their predecessor
+// still runs (launch_pdl) and wait here until it has completed and its writes are visible, so that
+// launch latency and the predecessor's tail overlap. Called by every thread before the first access
+// to memory that an earlier kernel wrote. pdl_wait also releases the next launch. early = false is an
+// ordinary launch.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <class... P>
+inline cudaError_t launch_pdl(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                              std::common_type_t<P>... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = at;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // Sum over a block of `nthreads` threads; `red` holds >= 32 elements of shared scratch.

@@ -143,6 +143,7 @@ __global__ void __launch_bounds__(32 * T, T == 4 ? EXA_MINB : 1) ex_apply_kernel
   __shared__ float red[32];
   __shared__ int last_s;
   const int slot = blockIdx.x, prt = blockIdx.y, parts = gridDim.y;
+  pdl_wait();
   if (slot >= *A.n_active) return;
   const int p = A.active[slot], n = A.n, tid = threadIdx.x;
   if (A.done[p]) return;
@@ -283,8 +284,9 @@ static inline cudaError_t launch_ex_cfg(const ExArgs& a, int batch, int parts, c
         cudaFuncSetAttribute(ex_apply_kernel<EPI, TC, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  ex_apply_kernel<EPI, TC, T><<<dim3(batch, parts), 32 * T, smem, stream>>>(a);
-  return cudaGetLastError();
+  // CTAs that leave SMs idle are launched late: early ones share SMs beside a running GEMM (one target at
+  // n = 16384, 20 iterations: 2.43 ms early, 2.23 late)
+  return launch_pdl(parts == 1, ex_apply_kernel<EPI, TC, T>, dim3(batch, parts), dim3(32 * T), smem, stream, a);
 }
 #ifndef EXA_T1
 #define EXA_T1 4
@@ -327,6 +329,7 @@ __global__ void __launch_bounds__(MMB_NT) mm_batch_kernel(MMBArgs A) {
   __shared__ float red[32];
   __shared__ int p_s[PB];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = A.n, k = A.k;
+  pdl_wait();
   const int na = *A.n_active, slot0 = blockIdx.x * PB;
   if (slot0 >= na) return;
   if (tid < PB) {
@@ -538,8 +541,7 @@ static inline cudaError_t launch_mmb_cfg(const MMBArgs& a, int batch, cudaStream
     const cudaError_t e = cudaFuncSetAttribute(mm_batch_kernel<PB, KQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  mm_batch_kernel<PB, KQ><<<(batch + PB - 1) / PB, MMB_NT, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(true, mm_batch_kernel<PB, KQ>, dim3((batch + PB - 1) / PB), dim3(MMB_NT), smem, s, a);
 }
 template <int PB>
 static inline cudaError_t launch_mmb_pb(const MMBArgs& a, int batch, cudaStream_t s) {

@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(32 * NWARP) f64_apply_kernel(ApplyArgs<double>
   __shared__ F64Row row_s[NWARP][PB];
   __shared__ double part_s[NWARP][PB];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * NWARP + warp, n = A.n;
+  pdl_wait();
   const int na = *A.n_active, b0 = blockIdx.y * PB;
   if (b0 >= na) return;
   int p[PB];
@@ -195,6 +196,7 @@ __global__ void __launch_bounds__(256) f64_mm_kernel(MMArgs<double> A) {
   __shared__ double red_s[8][KP], w_s[KP], w0_s[KP], c_s[KP], ic_s[KP], ix_s[KP], sum_s[8];
   __shared__ int stop;
   const int slot = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  pdl_wait();
   if (slot >= *A.n_active) return;
   const int p = A.active[slot], n = A.n, k = A.k;
   if (A.done[p]) return;
@@ -307,10 +309,10 @@ __global__ void __launch_bounds__(256) f64_mm_kernel(MMArgs<double> A) {
   }
 }
 static inline cudaError_t launch_f64_mm(const MMArgs<double>& a, int batch, cudaStream_t s) {
-  if (a.k <= 32) f64_mm_kernel<1><<<batch, 256, 0, s>>>(a);
-  else if (a.k <= 64) f64_mm_kernel<2><<<batch, 256, 0, s>>>(a);
-  else if (a.k <= 128) f64_mm_kernel<4><<<batch, 256, 0, s>>>(a);
-  else f64_mm_kernel<8><<<batch, 256, 0, s>>>(a);
+  if (a.k <= 32) (void)launch_pdl(true, f64_mm_kernel<1>, dim3(batch), dim3(256), 0, s, a);
+  else if (a.k <= 64) (void)launch_pdl(true, f64_mm_kernel<2>, dim3(batch), dim3(256), 0, s, a);
+  else if (a.k <= 128) (void)launch_pdl(true, f64_mm_kernel<4>, dim3(batch), dim3(256), 0, s, a);
+  else (void)launch_pdl(true, f64_mm_kernel<8>, dim3(batch), dim3(256), 0, s, a);
   return cudaGetLastError();
 }
 
@@ -322,11 +324,11 @@ static inline cudaError_t launch_f64_apply(const ApplyArgs<double>& a, const F64
                                            const int* done, int batch, int abs_cost, int lin_out, int sms,
                                            cudaStream_t s) {
   if (batch >= 4) {
-    f64_apply_kernel<EPI, 4, 8><<<dim3((a.n + 7) / 8, (batch + 3) / 4), 256, 0, s>>>(a, F, aout, R, done, abs_cost, lin_out);
+    (void)launch_pdl(true, f64_apply_kernel<EPI, 4, 8>, dim3((a.n + 7) / 8, (batch + 3) / 4), dim3(256), 0, s, a, F, aout, R, done, abs_cost, lin_out);
   } else if ((long long)a.n * batch > 8LL * sms) {
-    f64_apply_kernel<EPI, 1, 8><<<dim3((a.n + 7) / 8, batch), 256, 0, s>>>(a, F, aout, R, done, abs_cost, lin_out);
+    (void)launch_pdl(true, f64_apply_kernel<EPI, 1, 8>, dim3((a.n + 7) / 8, batch), dim3(256), 0, s, a, F, aout, R, done, abs_cost, lin_out);
   } else {
-    f64_apply_kernel<EPI, 1, 2><<<dim3((a.n + 1) / 2, batch), 64, 0, s>>>(a, F, aout, R, done, abs_cost, lin_out);
+    (void)launch_pdl(true, f64_apply_kernel<EPI, 1, 2>, dim3((a.n + 1) / 2, batch), dim3(64), 0, s, a, F, aout, R, done, abs_cost, lin_out);
   }
   return cudaGetLastError();
 }

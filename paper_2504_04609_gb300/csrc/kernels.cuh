@@ -661,6 +661,7 @@ __global__ void __launch_bounds__(256) source_init_kernel(const T* Dt, const T* 
 static __global__ void __launch_bounds__(1024) compact_kernel(int* active, int* n_active, const int* done) {
   __shared__ int warp_tot[32];
   __shared__ int total_s;
+  pdl_wait();
   const int na = *n_active;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int out = 0;

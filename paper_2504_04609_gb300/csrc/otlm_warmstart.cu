@@ -142,6 +142,7 @@ cudaError_t forward_tc(otlm_ws_ctx* w, int batch, const float* y, float eps, con
     const int want = otlm::tc::num_sms() / tiles, nkb = (din + 63) / 64;
     g.splits = want < 1 ? 1 : (want > nkb ? nkb : want);
     g.chunk = 1;
+    g.pdl = true;
     if (g.splits > TC_MAX_SPLITS) g.splits = TC_MAX_SPLITS;
     g.a_exact = 1;  // BF16 weights: two products
     g.split_stride = plane;

@@ -340,7 +340,7 @@ inline cudaError_t ex_iterate(const Launch& L, const Workspace<float>& ws, const
     const bool poll = (it + 1) % sp.poll_every == 0;
     if (poll && it > 0) {  // finished problems are skipped by their flag in between
       L.begin(KIND_COMPACT);
-      compact_kernel<<<1, 1024, 0, L.stream>>>(ws.active, ws.n_active, ws.done);
+      (void)launch_pdl(true, compact_kernel, dim3(1), dim3(1024), 0, L.stream, ws.active, ws.n_active, ws.done);
       L.end();
     }
     L.begin(KIND_APPLY);
@@ -473,7 +473,7 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
         const bool poll = (it + 1) % sp.poll_every == 0;
         if (poll && it > 0) {  // finished problems are skipped by their flag in between
           L.begin(KIND_COMPACT);
-          compact_kernel<<<1, 1024, 0, L.stream>>>(ws.active, ws.n_active, ws.done);
+          (void)launch_pdl(true, compact_kernel, dim3(1), dim3(1024), 0, L.stream, ws.active, ws.n_active, ws.done);
           L.end();
         }
         L.begin(KIND_APPLY);
@@ -501,7 +501,7 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
     mm.gap_check = check;
     launch_mm<T>(L, mm, batch);
     L.begin(KIND_COMPACT);
-    compact_kernel<<<1, 1024, 0, L.stream>>>(ws.active, ws.n_active, ws.done);
+    (void)launch_pdl(true, compact_kernel, dim3(1), dim3(1024), 0, L.stream, ws.active, ws.n_active, ws.done);
     L.end();
     if (it >= sp.max_iter) break;
     launch_apply<T, EPI_TARGET>(L, tgt, it == 0, batch, n, sp.cost);

@@ -40,6 +40,8 @@
 
 #include <type_traits>
 
+#include "common.cuh"
+
 namespace otlm {
 namespace tc {
 
@@ -195,6 +197,7 @@ struct GemmArgs {
   int store_direct;    // 1: the epilogue stores from registers, one 128-byte segment per warp and
                        // column, instead of staging and one bulk copy per column
   unsigned long long wait_ns;  // limit of every barrier wait (0: WAIT_NS)
+  bool pdl;            // launched early (launch_pdl)
   int withhold;        // self-check of the expired-wait path (otlm_check_wait_expiry): the producer of
                        // the first CTA arms its first stage but never issues the copies, so the MMA
                        // issuer's wait on that stage runs out; 0 in every solve
@@ -303,28 +306,6 @@ __global__ void __launch_bounds__(THREADS, 1)
   constexpr int BK = KindTraits<KIND>::BK;
   extern __shared__ uint8_t smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ncols = g.n_cols ? *g.n_cols : g.N;
-  const bool three = !g.hilo || *g.hilo != 0;  // the three products, or hi x hi alone
-  const bool two = three && g.a_exact;                          // Ahi (Bhi + Blo)
-  const int nst = two ? STAGES_TWO : three ? STAGES : STAGES_SINGLE;  // ring stages of this launch
-  const unsigned long long lim = g.wait_ns ? g.wait_ns : WAIT_NS;
-  const uint32_t st_bytes = two ? STAGE_TWO : three ? STAGE_BYTES : A_TILE + B_TILE;
-  const int mt = (g.M + BM - 1) / BM, nt = (g.N + BN - 1) / BN;
-  const int units = mt * nt * g.splits;
-  const int nkb_all = (g.Kd + BK - 1) / BK;
-  // work unit u -> output tile (m0, n0) and reduction split z (m fastest)
-  auto coords = [&](int u, int* m0, int* n0, int* z) {
-    *m0 = (u % mt) * BM;
-    const int r = u / mt;
-    *n0 = (r % nt) * BN;
-    *z = r / nt;
-  };
-  // split z's k blocks (the host keeps splits <= blocks, so every split has at least one)
-  auto krange = [&](int z, int* kb0, int* nkb) {
-    *kb0 = static_cast<int>(static_cast<long long>(nkb_all) * z / g.splits);
-    *nkb = static_cast<int>(static_cast<long long>(nkb_all) * (z + 1) / g.splits) - *kb0;
-  };
-
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   float* const stage_out = reinterpret_cast<float*>(base + STAGES * STAGE_BYTES);  // [64 columns][128 rows]
   uint64_t* bars = reinterpret_cast<uint64_t*>(base + STAGES * STAGE_BYTES + EPI_BYTES);
@@ -335,13 +316,6 @@ __global__ void __launch_bounds__(THREADS, 1)
   const uint32_t accf0 = smem_u32(bars + 2 * STAGES_SINGLE), acce0 = smem_u32(bars + 2 * STAGES_SINGLE + 2);
   const uint32_t drain = smem_u32(bars + 2 * STAGES_SINGLE + 4);
   const uint32_t ring = smem_u32(base), stage_s = smem_u32(stage_out);
-  // stage s of this launch's ring: A hi, B hi, then (three products) A lo, B lo; every tile starts on
-  // a 16 KiB boundary, as the 128-byte swizzle wants
-  auto a_hi = [&](int s) { return ring + static_cast<uint32_t>(s) * st_bytes; };
-  auto b_hi = [&](int s) { return a_hi(s) + A_TILE; };
-  auto a_lo = [&](int s) { return a_hi(s) + A_TILE + B_TILE; };
-  auto b_lo = [&](int s) { return a_hi(s) + (two ? A_TILE + B_TILE : 2 * A_TILE + B_TILE); };
-
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES_SINGLE; ++s) {
       mbar_init(full0 + 8 * s, 1);
@@ -365,6 +339,36 @@ __global__ void __launch_bounds__(THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();  // the set-up above overlaps the previous kernel
+  const int ncols = g.n_cols ? *g.n_cols : g.N;
+  const bool three = !g.hilo || *g.hilo != 0;  // the three products, or hi x hi alone
+  const bool two = three && g.a_exact;                          // Ahi (Bhi + Blo)
+  const int nst = two ? STAGES_TWO : three ? STAGES : STAGES_SINGLE;  // ring stages of this launch
+  const unsigned long long lim = g.wait_ns ? g.wait_ns : WAIT_NS;
+  const uint32_t st_bytes = two ? STAGE_TWO : three ? STAGE_BYTES : A_TILE + B_TILE;
+  const int mt = (g.M + BM - 1) / BM, nt = (g.N + BN - 1) / BN;
+  const int units = mt * nt * g.splits;
+  const int nkb_all = (g.Kd + BK - 1) / BK;
+  // work unit u -> output tile (m0, n0) and reduction split z (m fastest)
+  auto coords = [&](int u, int* m0, int* n0, int* z) {
+    *m0 = (u % mt) * BM;
+    const int r = u / mt;
+    *n0 = (r % nt) * BN;
+    *z = r / nt;
+  };
+  // split z's k blocks (the host keeps splits <= blocks, so every split has at least one)
+  auto krange = [&](int z, int* kb0, int* nkb) {
+    *kb0 = static_cast<int>(static_cast<long long>(nkb_all) * z / g.splits);
+    *nkb = static_cast<int>(static_cast<long long>(nkb_all) * (z + 1) / g.splits) - *kb0;
+  };
+
+  // stage s of this launch's ring: A hi, B hi, then (three products) A lo, B lo; every tile starts on
+  // a 16 KiB boundary, as the 128-byte swizzle wants
+  auto a_hi = [&](int s) { return ring + static_cast<uint32_t>(s) * st_bytes; };
+  auto b_hi = [&](int s) { return a_hi(s) + A_TILE; };
+  auto a_lo = [&](int s) { return a_hi(s) + A_TILE + B_TILE; };
+  auto b_lo = [&](int s) { return a_hi(s) + (two ? A_TILE + B_TILE : 2 * A_TILE + B_TILE); };
+
 
   if (warp == 0 && lane == 0) {
     // ---- TMA producer: the ring runs on across work units ----
@@ -673,25 +677,6 @@ __global__ void __launch_bounds__(THREADS, 1)
   const uint32_t rank = cluster_rank();
   const bool even = rank == 0;
   const int pair = static_cast<int>(blockIdx.x >> 1), npairs = static_cast<int>(gridDim.x >> 1);
-  const int ncols = g.n_cols ? *g.n_cols : g.N;
-  const bool three = !g.hilo || *g.hilo != 0;
-  const int nst = three ? P_STAGES : P_STAGES_SINGLE;
-  const int bnp = three ? BN : P_BN_SINGLE, bnh = bnp / 2;  // pair tile columns, B rows per CTA
-  const unsigned long long lim = g.wait_ns ? g.wait_ns : WAIT_NS;
-  const uint32_t st_bytes = three ? P_STAGE : P_STAGE_SINGLE;
-  const int mt = (g.M + P_BM - 1) / P_BM, nt = (g.N + bnp - 1) / bnp;
-  const int units = mt * nt;
-  const int nkb = (g.Kd + BK - 1) / BK;
-  // pair tile u: groups of P_GROUP_M row tiles, m fastest within a group, so that the pairs at work
-  // at one time share a band of A rows (2048 rows = 32 MiB of hi/lo BF16 at n = 4096) that stays in
-  // L2 while the B tiles stream, instead of all of A (which L2 does not hold across waves)
-  auto coords = [&](int u, int* m0, int* n0) {
-    const int per = P_GROUP_M * nt, grp = u / per, r = u - grp * per;
-    const int first = grp * P_GROUP_M, gsz = min(mt - first, P_GROUP_M);
-    *m0 = (first + r % gsz) * P_BM;
-    *n0 = (r / gsz) * bnp;
-  };
-
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   float* const stage_out = reinterpret_cast<float*>(base + STAGES * STAGE_BYTES);
   uint64_t* bars = reinterpret_cast<uint64_t*>(base + STAGES * STAGE_BYTES + EPI_BYTES);
@@ -702,14 +687,6 @@ __global__ void __launch_bounds__(THREADS, 1)
   const uint32_t accf0 = smem_u32(bars + 2 * P_STAGES_MAX), acce0 = smem_u32(bars + 2 * P_STAGES_MAX + 2);
   const uint32_t drain = smem_u32(bars + 2 * P_STAGES_MAX + 4);
   const uint32_t ring = smem_u32(base), stage_s = smem_u32(stage_out);
-  // stage s: A hi (16 KiB), B hi (8 KiB; 16 KiB for the single product's 128 rows), then (hi/lo) A lo,
-  // B lo; every tile on a 1 KiB (8-row atom) boundary, at the same offsets in both CTAs (the pair MMAs
-  // address the other CTA's tiles by this CTA's offsets)
-  auto a_hi = [&](int s) { return ring + static_cast<uint32_t>(s) * st_bytes; };
-  auto b_hi = [&](int s) { return a_hi(s) + A_TILE; };
-  auto a_lo = [&](int s) { return a_hi(s) + A_TILE + P_B_TILE; };
-  auto b_lo = [&](int s) { return a_hi(s) + 2 * A_TILE + P_B_TILE; };
-
   if (threadIdx.x == 0) {
     for (int s = 0; s < P_STAGES_MAX; ++s) {
       mbar_init(full0 + 8 * s, 1);   // the even CTA's producer; the bytes of both CTAs' copies
@@ -734,6 +711,34 @@ __global__ void __launch_bounds__(THREADS, 1)
   cluster_sync_all();  // both CTAs' barriers are initialised before either CTA signals the other's
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();  // the set-up above overlaps the previous kernel
+  const int ncols = g.n_cols ? *g.n_cols : g.N;
+  const bool three = !g.hilo || *g.hilo != 0;
+  const int nst = three ? P_STAGES : P_STAGES_SINGLE;
+  const int bnp = three ? BN : P_BN_SINGLE, bnh = bnp / 2;  // pair tile columns, B rows per CTA
+  const unsigned long long lim = g.wait_ns ? g.wait_ns : WAIT_NS;
+  const uint32_t st_bytes = three ? P_STAGE : P_STAGE_SINGLE;
+  const int mt = (g.M + P_BM - 1) / P_BM, nt = (g.N + bnp - 1) / bnp;
+  const int units = mt * nt;
+  const int nkb = (g.Kd + BK - 1) / BK;
+  // pair tile u: groups of P_GROUP_M row tiles, m fastest within a group, so that the pairs at work
+  // at one time share a band of A rows (2048 rows = 32 MiB of hi/lo BF16 at n = 4096) that stays in
+  // L2 while the B tiles stream, instead of all of A (which L2 does not hold across waves)
+  auto coords = [&](int u, int* m0, int* n0) {
+    const int per = P_GROUP_M * nt, grp = u / per, r = u - grp * per;
+    const int first = grp * P_GROUP_M, gsz = min(mt - first, P_GROUP_M);
+    *m0 = (first + r % gsz) * P_BM;
+    *n0 = (r / gsz) * bnp;
+  };
+
+  // stage s: A hi (16 KiB), B hi (8 KiB; 16 KiB for the single product's 128 rows), then (hi/lo) A lo,
+  // B lo; every tile on a 1 KiB (8-row atom) boundary, at the same offsets in both CTAs (the pair MMAs
+  // address the other CTA's tiles by this CTA's offsets)
+  auto a_hi = [&](int s) { return ring + static_cast<uint32_t>(s) * st_bytes; };
+  auto b_hi = [&](int s) { return a_hi(s) + A_TILE; };
+  auto a_lo = [&](int s) { return a_hi(s) + A_TILE + P_B_TILE; };
+  auto b_lo = [&](int s) { return a_hi(s) + 2 * A_TILE + P_B_TILE; };
+
 
   if (warp == 0 && lane == 0) {
     // ---- TMA producer (both CTAs): this CTA's A rows and B rows of each pair tile ----
@@ -961,8 +966,7 @@ static inline cudaError_t launch_gemm3(const void* A_hi, const void* A_lo, int l
     return cudaErrorInvalidValue;
   const long long units = static_cast<long long>((M + BM - 1) / BM) * ((N + BN - 1) / BN) * args.splits;
   const int grid = static_cast<int>(units < num_sms() ? units : num_sms());  // persistent: one CTA per SM
-  gemm3_kernel<KIND><<<grid, THREADS, SMEM_BYTES, stream>>>(ta_hi, ta_lo, tb_hi, tb_lo, a);
-  return cudaGetLastError();
+  return launch_pdl(a.pdl, gemm3_kernel<KIND>, dim3(grid), dim3(THREADS), SMEM_BYTES, stream, ta_hi, ta_lo, tb_hi, tb_lo, a);
 }
 
 // Launch the two-SM variant (same operands and arguments as launch_gemm3; no reduction split):
@@ -981,7 +985,9 @@ static inline cudaError_t launch_gemm3_pair(const void* A_hi, const void* A_lo, 
     attr = true;
   }
   if (args.splits != 1) return cudaErrorInvalidValue;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 2;
   at[0].val.clusterDim.y = 1;
@@ -991,7 +997,7 @@ static inline cudaError_t launch_gemm3_pair(const void* A_hi, const void* A_lo, 
   cfg.dynamicSmemBytes = P_SMEM_BYTES;
   cfg.stream = stream;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 1;  // the occupancy query takes the cluster size only
   if (!max_pairs) {
     cfg.gridDim = dim3(2 * (num_sms() / 2), 1, 1);
     int n = 0;
@@ -1011,6 +1017,7 @@ static inline cudaError_t launch_gemm3_pair(const void* A_hi, const void* A_lo, 
   const long long units = static_cast<long long>((M + P_BM - 1) / P_BM) * ((N + BN - 1) / BN);
   const int pairs = static_cast<int>(units < max_pairs ? units : max_pairs);
   cfg.gridDim = dim3(2 * pairs, 1, 1);
+  cfg.numAttrs = a.pdl ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, gemm3_pair_kernel<KIND>, ta_hi, ta_lo, tb_hi, tb_lo, tb_hi2, a);
 }
 

@@ -172,6 +172,7 @@ __global__ void kbuild_kernel(const float* xt, int n, int ld, __nv_bfloat16* Khi
 __global__ void tc_split_reduce_kernel(const float* part, int splits, size_t plane, const int* active,
                                        const int* n_active, int n, float* acc, int2* fix_list,
                                        unsigned long long* fix_cnt, unsigned long long fix_cap) {
+  pdl_wait();
   const size_t total = (size_t)(*n_active) * n;
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
     const int slot = (int)(e / n), i = (int)(e - (size_t)slot * n);
@@ -257,6 +258,7 @@ __global__ void __launch_bounds__(256) tc_fixup_kernel(const int2* list, const u
                                                        TcCost cost, In in, float* acc, const float* mshift) {
   using P = Prec<float>;
   __shared__ float red[32];
+  pdl_wait();
   const unsigned long long c = *cnt < cap ? *cnt : cap;
   if (blockIdx.x == 0 && threadIdx.x == 0) *cnt_next = 0;
   for (unsigned long long e = blockIdx.x; e < c; e += gridDim.x) {
@@ -318,15 +320,16 @@ enum { ROW_256x4 = 0, ROW_256x8 = 1, ROW_256x16 = 2, ROW_1024x16 = 3, ROW_STREAM
 inline int tc_row_cfg(int n) {
   return n <= 1024 ? ROW_256x4 : n <= 2048 ? ROW_256x8 : n <= 4096 ? ROW_256x16 : n <= 16384 ? ROW_1024x16 : ROW_STREAM;
 }
-#define TC_ROW_LAUNCH(KERNEL, CFG, GRID, STREAM, ...)                                       \
-  do {                                                                                      \
-    switch (CFG) {                                                                          \
-      case ROW_256x4: KERNEL<256, 4><<<(GRID), 256, 0, (STREAM)>>>(__VA_ARGS__); break;     \
-      case ROW_256x8: KERNEL<256, 8><<<(GRID), 256, 0, (STREAM)>>>(__VA_ARGS__); break;     \
-      case ROW_256x16: KERNEL<256, 16><<<(GRID), 256, 0, (STREAM)>>>(__VA_ARGS__); break;   \
-      case ROW_1024x16: KERNEL<1024, 16><<<(GRID), 1024, 0, (STREAM)>>>(__VA_ARGS__); break; \
-      default: KERNEL<256, 0><<<(GRID), 256, 0, (STREAM)>>>(__VA_ARGS__); break;            \
-    }                                                                                       \
+// (pdl: early launches, from the enclosing scope)
+#define TC_ROW_LAUNCH(KERNEL, CFG, GRID, STREAM, ...)                                                    \
+  do {                                                                                                   \
+    switch (CFG) {                                                                                       \
+      case ROW_256x4: (void)launch_pdl(pdl, KERNEL<256, 4>, dim3(GRID), dim3(256), 0, (STREAM), __VA_ARGS__); break;   \
+      case ROW_256x8: (void)launch_pdl(pdl, KERNEL<256, 8>, dim3(GRID), dim3(256), 0, (STREAM), __VA_ARGS__); break;   \
+      case ROW_256x16: (void)launch_pdl(pdl, KERNEL<256, 16>, dim3(GRID), dim3(256), 0, (STREAM), __VA_ARGS__); break; \
+      case ROW_1024x16: (void)launch_pdl(pdl, KERNEL<1024, 16>, dim3(GRID), dim3(1024), 0, (STREAM), __VA_ARGS__); break; \
+      default: (void)launch_pdl(pdl, KERNEL<256, 0>, dim3(GRID), dim3(256), 0, (STREAM), __VA_ARGS__); break; \
+    }                                                                                                    \
   } while (0)
 
 // Datafit step (Table 1) in log2 units: the new target potential from log2 of the target sum v and
@@ -385,6 +388,7 @@ __global__ void __launch_bounds__(NT) tc_prep_src_kernel(TcIterArgs A) {
   using P = Prec<float>;
   __shared__ float red[32];
   const int slot = blockIdx.x;
+  pdl_wait();
   // the product count the coming source apply takes (it reads hilo[0] at launch; nothing changes it
   // before then), for the stopping decision after it
   if (slot == 0 && threadIdx.x == 0) A.t.hilo[1] = A.t.hilo[0];
@@ -467,6 +471,7 @@ __device__ __forceinline__ void tc_violation_body(const TcIterArgs& A) {
   using P = Prec<float>;
   __shared__ float red[32];
   const int slot = blockIdx.x;
+  pdl_wait();
   if (slot >= *A.n_active) return;
   const int p = A.active[slot], n = A.n, cur = A.it & 1;
   const float* acc = A.t.ACC_src[cur] + (size_t)p * n;
@@ -580,6 +585,7 @@ inline size_t carve_tc_mm(void* base, int k_max, int batch_max, TcMMBuf* mb) {
 __global__ void __launch_bounds__(256) tc_wupd_kernel(TcIterArgs A, TcMMBuf M, int splits, int update,
                                                       int save_prev) {
   using P = Prec<float>;
+  pdl_wait();
   const int na = *A.n_active, k = A.k;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   const int slot = e / k, j = e - slot * k;
@@ -609,6 +615,7 @@ __global__ void __launch_bounds__(NT) tc_operand_kernel(TcIterArgs A) {
   using P = Prec<float>;
   __shared__ float red[32];
   const int slot = blockIdx.x;
+  pdl_wait();
   if (slot >= *A.n_active) return;
   const int p = A.active[slot], n = A.n, cur = A.it & 1;
   const float* S = A.S + (size_t)p * n;
@@ -630,7 +637,6 @@ __global__ void __launch_bounds__(NT) tc_operand_kernel(TcIterArgs A) {
       }
 #pragma unroll
       for (int e = 0; e < EPT; ++e) {
-        const int j = e * NT + threadIdx.x;
         f2[e] = sv[e] > 0.f ? P::log2(sv[e]) - tc_log2_sum(av[e], mc) : P::ninf();
         fm = fmaxf(fm, f2[e]);
         ms += sv[e];
@@ -739,7 +745,7 @@ __global__ void tc_finalize_kernel(FinArgs<float> F, TcIterArgs A) {
 
 // Where the expansion applies serve a tensor-core handle: small batches (one target at n = 16384, 20
 // iterations: 11.9 -> 2.3 ms, no kernel matrix to stream) and batches whose GEMMs do not fill the SM
-// pairs (1024 problems of 1024 bins, 32 pair tiles, 50 iterations: 5.75 -> 4.61 ms); an apply takes the
+// pairs (1024 problems of 1024 bins, 32 pair tiles, 50 iterations: 5.86 -> 4.33 ms); an apply takes the
 // expansion 27 us per million bins and a full GEMM less up to n = 4096 or so. A caller who sets the precision
 // schedule has asked for the GEMM's single product and keeps the GEMMs.
 constexpr long long TC_EXPANSION_BINS = 5 << 18;  // 1.25 million
@@ -757,6 +763,9 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
   const int batch = sp.batch, n = sp.n, k = sp.k;
   const double eps_ln2 = sp.eps * kLn2;
   const bool checks = ow && sp.check_every > 0;
+  // early launches pay where an iteration is launch latency (256 problems of 1024 bins, 20 iterations: 1.97
+  // -> 1.52 ms); where the row kernels fill the SMs for long they cost a little (4096 x 4096: 12.46 -> 12.52)
+  const bool pdl = (long long)batch * n <= 8LL << 20;
   // small batches: whole solves in one launch, as on an FP32 handle (with more than one problem per SM
   // of a long grid the batched kernels below win)
   if (sp.single_until == 0.0 && ex_serves(sp, C != nullptr, checks) && small_prefers(sp, sm_count()) &&
@@ -837,7 +846,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
   tc::GemmArgs ga{};
   ga.col_map = ws.active; ga.n_cols = ws.n_active; ga.M = n; ga.N = batch; ga.Kd = n; ga.ld_out = n;
   ga.err = tw.err; ga.fix_list = tw.fix_list; ga.fix_cap = (unsigned long long)batch * n; ga.splits = 1;
-  ga.hilo = tw.hilo;
+  ga.hilo = tw.hilo; ga.pdl = pdl;
   {
     const int units = ((n + tc::BM - 1) / tc::BM) * ((batch + tc::BN - 1) / tc::BN);
     if (batch <= TC_SMALL_BATCH ? units < tc::num_sms() : 2 * units <= tc::num_sms()) {
@@ -867,7 +876,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
     L.begin(KIND_APPLY);
     cudaError_t r = launch_apply(kt ? tw.Kthi : tw.Khi, kt ? tw.Ktlo : tw.Klo, tw.Vhi, tw.Vlo, ga);
     if (r == cudaSuccess && ga.splits > 1) {
-      tc_split_reduce_kernel<<<red_grid, 256, 0, L.stream>>>(tw.ACCP, ga.splits, ga.split_stride, ws.active,
+      (void)launch_pdl(pdl, tc_split_reduce_kernel, dim3(red_grid), dim3(256), 0, L.stream, tw.ACCP, ga.splits, ga.split_stride, ws.active,
                                                               ws.n_active, n, acc, tw.fix_list, cnt, ga.fix_cap);
       r = cudaGetLastError();
     }
@@ -876,6 +885,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
   };
   // D^T r (TF32): M = dictionary columns, N = slots (partial sums by slot), reduction over bins split
   tc::GemmArgs gr{};
+  gr.pdl = pdl;
   gr.out = mb.NU; gr.n_cols = ws.n_active; gr.M = k; gr.N = batch; gr.Kd = n; gr.ld_out = mb.ldnu; gr.err = tw.err;
   gr.splits = tc::choose_splits(((k + tc::BM - 1) / tc::BM) * ((batch + tc::BN - 1) / tc::BN),
                                 (n + tc::KindTraits<tc::KIND_TF32>::BK - 1) / tc::KindTraits<tc::KIND_TF32>::BK);
@@ -883,6 +893,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
   // s = D w (TF32, two-SM kernel): M = bins, N = slots mapped to problems, reduction over dictionary
   // columns
   tc::GemmArgs gw{};
+  gw.pdl = pdl;
   gw.out = ws.S; gw.col_map = ws.active; gw.n_cols = ws.n_active; gw.M = n; gw.N = batch; gw.Kd = k;
   gw.ld_out = n; gw.err = tw.err; gw.flush_tiny = 1; gw.splits = 1; gw.store_direct = 1;
   const int row_cfg = tc_row_cfg(n);
@@ -904,14 +915,14 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
     L.begin(KIND_APPLY);
     r = launch_apply(C ? tw.Kthi : tw.Khi, C ? tw.Ktlo : tw.Klo, tw.Vhi, tw.Vlo, go);
     if (r == cudaSuccess && go.splits > 1) {
-      tc_split_reduce_kernel<<<red_grid, 256, 0, L.stream>>>(tw.ACCP, go.splits, go.split_stride, list, count, n,
+      (void)launch_pdl(pdl, tc_split_reduce_kernel, dim3(red_grid), dim3(256), 0, L.stream, tw.ACCP, go.splits, go.split_stride, list, count, n,
                                                               ow->LB2, tw.fix_list, tw.fix_cnt + 2, go.fix_cap);
       r = cudaGetLastError();
     }
     L.end();
     if (r != cudaSuccess) return r;
     L.begin(KIND_OTHER);
-    tc_fixup_kernel<<<TC_FIX_GRID, 256, 0, L.stream>>>(tw.fix_list, tw.fix_cnt + 2, tw.fix_cnt + 3, ga.fix_cap, n,
+    (void)launch_pdl(pdl, tc_fixup_kernel<TcInArray>, dim3(TC_FIX_GRID), dim3(256), 0, L.stream, tw.fix_list, tw.fix_cnt + 2, tw.fix_cnt + 3, ga.fix_cap, n,
                                                     cost_tgt, TcInArray{ow->F2, n}, ow->LB2, ow->M);
     L.end();
     L.begin(KIND_OTHER);
@@ -928,7 +939,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
   // the initial source marginal s = D w0, through the same operand and GEMM as every iteration
   // (the mass sum_i s_i is first needed by the violation at it = 1 and set by the operand kernel)
   L.begin(KIND_OTHER);
-  tc_wupd_kernel<<<(int)(((long long)batch * k + 255) / 256), 256, 0, L.stream>>>(ta, mb, 0, 0, 0);
+  (void)launch_pdl(pdl, tc_wupd_kernel, dim3((int)(((long long)batch * k + 255) / 256)), dim3(256), 0, L.stream, ta, mb, 0, 0, 0);
   L.end();
   L.begin(KIND_OTHER);
   e = tc::launch_gemm3_pair<tc::KIND_TF32>(tw.Dhi, tw.Dlo, tw.kp, tw.Whi, tw.Wlo, tw.kp, n, batch, k, gw, L.stream);
@@ -960,7 +971,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
         L.end();
         if (e != cudaSuccess) return e;
         L.begin(KIND_MM);
-        tc_wupd_kernel<<<wgrid, 256, 0, L.stream>>>(ta, mb, gr.splits, 1, m == 0);
+        (void)launch_pdl(pdl, tc_wupd_kernel, dim3(wgrid), dim3(256), 0, L.stream, ta, mb, gr.splits, 1, m == 0);
         L.end();
         L.begin(KIND_MM);
         e = tc::launch_gemm3_pair<tc::KIND_TF32>(tw.Dhi, tw.Dlo, tw.kp, tw.Whi, tw.Wlo, tw.kp, n, batch, k, gw, L.stream);
@@ -970,7 +981,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
       const bool poll = (it + 1) % sp.poll_every == 0;
       if (poll && it > 0) {  // finished problems are skipped by their flag in between
         L.begin(KIND_COMPACT);
-        compact_kernel<<<1, 1024, 0, L.stream>>>(ws.active, ws.n_active, ws.done);
+        (void)launch_pdl(pdl, compact_kernel, dim3(1), dim3(1024), 0, L.stream, ws.active, ws.n_active, ws.done);
         L.end();
       }
       L.begin(KIND_APPLY);
@@ -994,7 +1005,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
     e = apply(tw.ACC_src[it & 1], tw.fix_cnt, false);
     if (e != cudaSuccess) return e;
     L.begin(KIND_OTHER);
-    tc_fixup_kernel<<<TC_FIX_GRID, 256, 0, L.stream>>>(tw.fix_list, tw.fix_cnt, tw.fix_cnt + 1, ga.fix_cap, n,
+    (void)launch_pdl(pdl, tc_fixup_kernel<TcInG2>, dim3(TC_FIX_GRID), dim3(256), 0, L.stream, tw.fix_list, tw.fix_cnt, tw.fix_cnt + 1, ga.fix_cap, n,
                                                     cost_src, TcInG2{ta}, tw.ACC_src[it & 1], tw.Msrc[it & 1]);
     L.end();
     // a check: the state (w, g) whose source sums were just computed is the one this iteration
@@ -1014,7 +1025,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
     L.end();
     if (e != cudaSuccess) return e;
     L.begin(KIND_MM);
-    tc_wupd_kernel<<<(int)(((long long)batch * k + 255) / 256), 256, 0, L.stream>>>(ta, mb, gr.splits, 1, 1);
+    (void)launch_pdl(pdl, tc_wupd_kernel, dim3((int)(((long long)batch * k + 255) / 256)), dim3(256), 0, L.stream, ta, mb, gr.splits, 1, 1);
     L.end();
     L.begin(KIND_MM);
     e = tc::launch_gemm3_pair<tc::KIND_TF32>(tw.Dhi, tw.Dlo, tw.kp, tw.Whi, tw.Wlo, tw.kp, n, batch, k, gw, L.stream);
@@ -1030,7 +1041,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
       L.end();
       if (e != cudaSuccess) return e;
       L.begin(KIND_MM);
-      tc_wupd_kernel<<<(int)(((long long)batch * k + 255) / 256), 256, 0, L.stream>>>(ta, mb, gr.splits, 1, 0);
+      (void)launch_pdl(pdl, tc_wupd_kernel, dim3((int)(((long long)batch * k + 255) / 256)), dim3(256), 0, L.stream, ta, mb, gr.splits, 1, 0);
       L.end();
       L.begin(KIND_MM);
       e = tc::launch_gemm3_pair<tc::KIND_TF32>(tw.Dhi, tw.Dlo, tw.kp, tw.Whi, tw.Wlo, tw.kp, n, batch, k, gw, L.stream);
@@ -1039,7 +1050,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
     }
     if (it > 0) {
       L.begin(KIND_COMPACT);
-      compact_kernel<<<1, 1024, 0, L.stream>>>(ws.active, ws.n_active, ws.done);
+      (void)launch_pdl(pdl, compact_kernel, dim3(1), dim3(1024), 0, L.stream, ws.active, ws.n_active, ws.done);
       L.end();
     }
     L.begin(KIND_MM);
@@ -1048,7 +1059,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
     e = apply(tw.ACC_tgt, tw.fix_cnt + 1, true);
     if (e != cudaSuccess) return e;
     L.begin(KIND_OTHER);
-    tc_fixup_kernel<<<TC_FIX_GRID, 256, 0, L.stream>>>(tw.fix_list, tw.fix_cnt + 1, tw.fix_cnt, ga.fix_cap, n,
+    (void)launch_pdl(pdl, tc_fixup_kernel<TcInF2>, dim3(TC_FIX_GRID), dim3(256), 0, L.stream, tw.fix_list, tw.fix_cnt + 1, tw.fix_cnt, ga.fix_cap, n,
                                                     cost_tgt, TcInF2{ta}, tw.ACC_tgt, tw.Mtgt);
     L.end();
     if ((it + 1) % sp.poll_every == 0) {
