@@ -55,7 +55,8 @@ struct TcWorkspace {
   int* hilo;                 // [0] 0: the applies use the single BF16 product, 1: hi/lo (three
                              // products); [1] the value the iteration's source apply was launched with
   int2* fix_list;            // [batch x n] underflowed sums (problem, row) listed by a GEMM
-  unsigned long long* fix_cnt;  // [2] list lengths: source GEMM, target GEMM
+  unsigned long long* fix_cnt;  // [0, 1] list lengths: source GEMM, target GEMM; [2, 3] the objective's;
+                                // [4..7] the last lengths (source, target) by parity of the iteration
   unsigned long long fix_cap;
   float *Dhi, *Dlo;          // [n][kp] dictionary as TF32 hi/lo (A operand of s = D w)
   float *Dthi, *Dtlo;        // [k][ld] transposed dictionary as TF32 hi/lo (A operand of D^T r)
@@ -224,7 +225,7 @@ __global__ void __launch_bounds__(256) kdense_kernel(const float* C, int n, int 
 }
 
 // Exact fix-up of the sums a GEMM listed as underflowed, one CTA of 256 threads per listed
-// (problem p, row i) so that a row costs a few memory round trips, not n / 32:
+// (problem p, row i) so that a row costs a few memory round trips, not n / 32 (a warp where the list is long):
 //   L = log2 sum_j 2^(in_pj - cost_ij)     (two passes over j: max, then sum; cost in log2 units)
 // stored as the negative offset L - M_p (decoded by tc_log2_sum); an empty sum stays 0.  in = G2
 // and M = Msrc for the source sums, in = F2 and M = Mtgt for the target sums.  The source and
@@ -250,37 +251,78 @@ struct TcCost {
   }
 };
 
-// In: the row's potentials, in(p, j) (an array, or formed from the sums and targets they came from: the
-// row kernels keep neither G2 nor F2, which only the rare listed rows and the returned state need).
+// In: the rows' potentials, in(p, j): an array, or formed from the sums and targets they came from. The row
+// kernels store G2 and F2 only where the last fix-up of the kind had more rows than CTAs (in.array() is
+// the array then): with few rows the stores cost more than they save (8 bytes per bin and iteration, 4096
+// x 4096, 20 iterations: 12.60 -> 12.46 ms without), with many forming them per row does (a KL batch of
+// 4096 x 2048 with empty target regions, 31 iterations: 169 ms stored, 561 formed).
+// More rows than CTAs also take a warp each instead of a CTA: no block reductions, eight times the rows
+// in flight (the same batch: 169 -> 94 ms; 1024 x 2048: 49.3 -> 31.3 ms).
+template <class In, bool ARRAY>
+__device__ __forceinline__ float tc_fix_term(const In& in, const float* v, int p, int j) {
+  if constexpr (ARRAY) return v[j];
+  else return in(p, j);
+}
+// log2 sum_j 2^(in_pj - cost_ij) of one row over the threads tid of nt (a CTA or a warp)
+template <class In, bool ARRAY, bool WARP>
+__device__ __forceinline__ float tc_fix_row(const In& in, const TcCost& cost, int p, int i, int n, float* red) {
+  using P = Prec<float>;
+  const float* v = ARRAY ? in.array() + (size_t)p * n : nullptr;
+  const int tid = WARP ? threadIdx.x & 31 : threadIdx.x, nt = WARP ? 32 : blockDim.x;
+  float mx = -CUDART_INF_F;
+#pragma unroll 8
+  for (int j = tid; j < n; j += nt) mx = fmaxf(mx, tc_fix_term<In, ARRAY>(in, v, p, j) - cost(i, j, n));
+  if constexpr (WARP) {
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  } else mx = block_max(mx, red);
+  float sum = 0.f;
+  if (mx > -CUDART_INF_F) {
+#pragma unroll 8
+    for (int j = tid; j < n; j += nt) sum += P::exp2((tc_fix_term<In, ARRAY>(in, v, p, j) - mx) - cost(i, j, n));
+  }
+  if constexpr (WARP) {
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  } else sum = block_sum(sum, red);
+  return sum > 0.f ? mx + P::log2(sum) : -CUDART_INF_F;
+}
+template <class In, bool ARRAY>
+__device__ __forceinline__ void tc_fix_rows(const int2* list, unsigned long long c, int n, const TcCost& cost,
+                                            const In& in, float* acc, const float* mshift, float* red) {
+  // a representable sum is stored raw; an underflowing one as its negative log2 offset
+  auto put = [&](int2 pi, float L) {
+    const float off = L - mshift[pi.x];
+    acc[(size_t)pi.x * n + pi.y] = !(L > -CUDART_INF_F) ? 0.f : (off >= -126.f ? Prec<float>::exp2(off) : off);
+  };
+  if (c > gridDim.x) {
+    const int warps = blockDim.x >> 5;
+    for (unsigned long long e = (unsigned long long)blockIdx.x * warps + (threadIdx.x >> 5); e < c;
+         e += (unsigned long long)gridDim.x * warps) {
+      const float L = tc_fix_row<In, ARRAY, true>(in, cost, list[e].x, list[e].y, n, red);
+      if ((threadIdx.x & 31) == 0) put(list[e], L);
+    }
+  } else {
+    for (unsigned long long e = blockIdx.x; e < c; e += gridDim.x) {
+      const float L = tc_fix_row<In, ARRAY, false>(in, cost, list[e].x, list[e].y, n, red);
+      if (threadIdx.x == 0) put(list[e], L);
+    }
+  }
+}
+// last: the list's length, kept for the next iteration's row kernel and fix-up (or null)
 template <class In>
 __global__ void __launch_bounds__(256) tc_fixup_kernel(const int2* list, const unsigned long long* cnt,
-                                                       unsigned long long* cnt_next, unsigned long long cap, int n,
-                                                       TcCost cost, In in, float* acc, const float* mshift) {
-  using P = Prec<float>;
+                                                       unsigned long long* cnt_next, unsigned long long* last,
+                                                       unsigned long long cap, int n, TcCost cost, In in, float* acc,
+                                                       const float* mshift) {
   __shared__ float red[32];
   pdl_wait();
   const unsigned long long c = *cnt < cap ? *cnt : cap;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *cnt_next = 0;
-  for (unsigned long long e = blockIdx.x; e < c; e += gridDim.x) {
-    const int2 pi = list[e];
-    const int p = pi.x;
-    float mx = -CUDART_INF_F;
-#pragma unroll 4
-    for (int j = threadIdx.x; j < n; j += blockDim.x) mx = fmaxf(mx, in(p, j) - cost(pi.y, j, n));
-    mx = block_max(mx, red);
-    float sum = 0.f;
-    if (mx > -CUDART_INF_F) {
-#pragma unroll 4
-      for (int j = threadIdx.x; j < n; j += blockDim.x) sum += P::exp2((in(p, j) - mx) - cost(pi.y, j, n));
-    }
-    sum = block_sum(sum, red);
-    if (threadIdx.x == 0) {
-      const float L = sum > 0.f ? mx + P::log2(sum) : -CUDART_INF_F;
-      // a representable sum is stored raw; an underflowing one as its negative log2 offset
-      const float off = L - mshift[pi.x];
-      acc[(size_t)pi.x * n + pi.y] = !(L > -CUDART_INF_F) ? 0.f : (off >= -126.f ? P::exp2(off) : off);
-    }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *cnt_next = 0;
+    if (last) *last = c;
   }
+  if (c == 0) return;
+  if (in.array()) tc_fix_rows<In, true>(list, c, n, cost, in, acc, mshift, red);
+  else tc_fix_rows<In, false>(list, c, n, cost, in, acc, mshift, red);
 }
 
 struct TcIterArgs {
@@ -352,15 +394,23 @@ __device__ __forceinline__ float tc_datafit(const TcIterArgs& A, float v, float 
   }
 }
 
+// Whether this iteration's row kernel stores G2 (kind 0) or F2 (kind 1): the length of the previous
+// iteration's list, fix_cnt[4 + 2 kind + parity] (the first iteration's counts as long).
+__device__ __forceinline__ bool tc_keeps(const TcIterArgs& A, int kind) {
+  return (kind == 0 && A.keep_g2) || A.t.fix_cnt[4 + 2 * kind + (A.it & 1)] > (unsigned long long)TC_FIX_GRID;
+}
+
 // The potentials a fix-up sums: an array, the datafit step of the previous target sums (G2), or
 // log2 s - log2 a (F2) of this iteration's source sums.
 struct TcInArray {
   const float* v;
   int n;
+  __device__ __forceinline__ const float* array() const { return v; }
   __device__ __forceinline__ float operator()(int p, int j) const { return v[(size_t)p * n + j]; }
 };
 struct TcInG2 {
   TcIterArgs A;
+  __device__ __forceinline__ const float* array() const { return tc_keeps(A, 0) ? A.G2 : nullptr; }
   __device__ __forceinline__ float operator()(int p, int j) const {
     const size_t o = (size_t)p * A.n + j;
     return A.it > 0 ? tc_datafit(A, tc_log2_sum(A.t.ACC_tgt[o], A.t.Mtgt[p]), A.y[o]) : A.G2[o];
@@ -368,6 +418,7 @@ struct TcInG2 {
 };
 struct TcInF2 {
   TcIterArgs A;
+  __device__ __forceinline__ const float* array() const { return tc_keeps(A, 1) ? A.F2 : nullptr; }
   __device__ __forceinline__ float operator()(int p, int j) const {
     const size_t o = (size_t)p * A.n + j;
     const float s = A.S[o];
@@ -415,7 +466,6 @@ __global__ void __launch_bounds__(NT) tc_prep_src_kernel(TcIterArgs A) {
       for (int e = 0; e < EPT; ++e) {
         const int j = e * NT + threadIdx.x;
         g[e] = tc_datafit(A, tc_log2_sum(a[e], mt), yv[e]);
-        if (A.keep_g2 && j < n) G2[j] = g[e];
       }
     } else {
 #pragma unroll
@@ -433,6 +483,11 @@ __global__ void __launch_bounds__(NT) tc_prep_src_kernel(TcIterArgs A) {
     for (int e = 0; e < EPT; ++e) {
       const int j = e * NT + threadIdx.x;
       if (j < n) tc_store_operand(P::exp2(g[e] - m), vhi, vlo, j);
+    }
+    if (A.it > 0 && tc_keeps(A, 0)) {
+#pragma unroll
+      for (int e = 0; e < EPT; ++e)
+        if (e * NT + threadIdx.x < n) G2[e * NT + threadIdx.x] = g[e];
     }
   } else {
     for (int j = threadIdx.x; j < n; j += NT) {
@@ -620,7 +675,7 @@ __global__ void __launch_bounds__(NT) tc_operand_kernel(TcIterArgs A) {
   const int p = A.active[slot], n = A.n, cur = A.it & 1;
   const float* S = A.S + (size_t)p * n;
   const float* acc = A.t.ACC_src[cur] + (size_t)p * n;
-  float* F2 = A.F2 + (size_t)p * n;  // streamed rows only
+  float* F2 = A.F2 + (size_t)p * n;
   __nv_bfloat16* vhi = A.t.Vhi + (size_t)slot * A.t.ld;
   __nv_bfloat16* vlo = A.t.Vlo + (size_t)slot * A.t.ld;
   const float mc = A.t.Msrc[cur][p];
@@ -649,6 +704,11 @@ __global__ void __launch_bounds__(NT) tc_operand_kernel(TcIterArgs A) {
     for (int e = 0; e < EPT; ++e) {
       const int j = e * NT + threadIdx.x;
       if (j < n) tc_store_operand(P::exp2(f2[e] - m), vhi, vlo, j);
+    }
+    if (tc_keeps(A, 1)) {
+#pragma unroll
+      for (int e = 0; e < EPT; ++e)
+        if (e * NT + threadIdx.x < n) F2[e * NT + threadIdx.x] = f2[e];
     }
     if (threadIdx.x == 0) {
       A.mass[p] = ms;
@@ -820,6 +880,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
   cudaError_t e = cudaMemsetAsync(tw.err, 0, sizeof(int), L.stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(tw.hilo, sp.single_until > 0 ? 0 : 0xFF, 2 * sizeof(int), L.stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(tw.fix_cnt, 0, 2 * sizeof(unsigned long long), L.stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(tw.fix_cnt + 4, 0xff, 4 * sizeof(unsigned long long), L.stream);
   if (e == cudaSuccess && checks) e = cudaMemsetAsync(ow->kmass, 0, sizeof(double), L.stream);
   if (e != cudaSuccess) return e;
   if (checks) {  // sum_ij K_ij in FP64, once per solve
@@ -922,7 +983,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
     L.end();
     if (r != cudaSuccess) return r;
     L.begin(KIND_OTHER);
-    (void)launch_pdl(pdl, tc_fixup_kernel<TcInArray>, dim3(TC_FIX_GRID), dim3(256), 0, L.stream, tw.fix_list, tw.fix_cnt + 2, tw.fix_cnt + 3, ga.fix_cap, n,
+    (void)launch_pdl(pdl, tc_fixup_kernel<TcInArray>, dim3(TC_FIX_GRID), dim3(256), 0, L.stream, tw.fix_list, tw.fix_cnt + 2, tw.fix_cnt + 3, nullptr, ga.fix_cap, n,
                                                     cost_tgt, TcInArray{ow->F2, n}, ow->LB2, ow->M);
     L.end();
     L.begin(KIND_OTHER);
@@ -1005,7 +1066,8 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
     e = apply(tw.ACC_src[it & 1], tw.fix_cnt, false);
     if (e != cudaSuccess) return e;
     L.begin(KIND_OTHER);
-    (void)launch_pdl(pdl, tc_fixup_kernel<TcInG2>, dim3(TC_FIX_GRID), dim3(256), 0, L.stream, tw.fix_list, tw.fix_cnt, tw.fix_cnt + 1, ga.fix_cap, n,
+    (void)launch_pdl(pdl, tc_fixup_kernel<TcInG2>, dim3(TC_FIX_GRID), dim3(256), 0, L.stream, tw.fix_list, tw.fix_cnt, tw.fix_cnt + 1,
+                     tw.fix_cnt + 4 + ((it + 1) & 1), ga.fix_cap, n,
                                                     cost_src, TcInG2{ta}, tw.ACC_src[it & 1], tw.Msrc[it & 1]);
     L.end();
     // a check: the state (w, g) whose source sums were just computed is the one this iteration
@@ -1059,7 +1121,8 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
     e = apply(tw.ACC_tgt, tw.fix_cnt + 1, true);
     if (e != cudaSuccess) return e;
     L.begin(KIND_OTHER);
-    (void)launch_pdl(pdl, tc_fixup_kernel<TcInF2>, dim3(TC_FIX_GRID), dim3(256), 0, L.stream, tw.fix_list, tw.fix_cnt + 1, tw.fix_cnt, ga.fix_cap, n,
+    (void)launch_pdl(pdl, tc_fixup_kernel<TcInF2>, dim3(TC_FIX_GRID), dim3(256), 0, L.stream, tw.fix_list, tw.fix_cnt + 1, tw.fix_cnt,
+                     tw.fix_cnt + 6 + ((it + 1) & 1), ga.fix_cap, n,
                                                     cost_tgt, TcInF2{ta}, tw.ACC_tgt, tw.Mtgt);
     L.end();
     if ((it + 1) % sp.poll_every == 0) {
