@@ -54,6 +54,7 @@ __device__ __forceinline__ void ex_direct(const float* in_s, const float* xt, in
     auto sweep = [&] {
 #pragma unroll
       for (int q = 0; q < Q; ++q) sum[q] = 0.f;
+#pragma unroll 4
       for (int j = lane; j < n; j += 32) {
         const float v = in_s[j], xj = xt[j];
 #pragma unroll

@@ -314,14 +314,44 @@ inline bool ex_serves(const SolveParams& sp, bool dense, bool checks) {
   return !dense && !checks && sp.cost == COST_SQ && sp.n <= EXA_MAX_N;
 }
 
-// The iteration loop of solve_device with expansion applies (three launches beside the compaction).
+// The number of blocks of a grid's plan on the host (0: the grid does not qualify), read while the
+// kernels queued in between run. A stream under capture cannot be read: `known` stays false and the
+// kernels follow the plan on the device.
+struct ExPlanRead {
+  cudaEvent_t ev = nullptr;
+  bool known = false;
+  int nb = 0;
+  cudaError_t begin(const Launch& L, const Workspace<float>& ws, int n) {
+    L.begin(KIND_OTHER);
+    cudaError_t e = ex_plan(ws.xt, n, ex_plan_of(ws), L.stream);
+    L.end();
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (e == cudaSuccess) e = cudaStreamIsCapturing(L.stream, &cap);
+    if (e != cudaSuccess || !L.host_flag || cap != cudaStreamCaptureStatusNone) return e;
+    e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(L.host_flag, &ex_plan_of(ws)->nb, sizeof(int), cudaMemcpyDeviceToHost, L.stream);
+    if (e == cudaSuccess) e = cudaEventRecord(ev, L.stream);
+    return e;
+  }
+  cudaError_t end(const Launch& L) {
+    if (!ev) return cudaSuccess;
+    const cudaError_t e = cudaEventSynchronize(ev);
+    known = e == cudaSuccess;
+    nb = *L.host_flag;
+    return e;
+  }
+  ~ExPlanRead() {
+    if (ev) cudaEventDestroy(ev);
+  }
+};
+
+// The iteration loop of solve_device with expansion applies (three launches beside the compaction);
+// the plan is on the device.
 inline cudaError_t ex_iterate(const Launch& L, const Workspace<float>& ws, const SolveParams& sp, const float* D,
                               const float* y) {
   const int batch = sp.batch, sms = sm_count();
-  L.begin(KIND_OTHER);
-  cudaError_t e = ex_plan(ws.xt, sp.n, ex_plan_of(ws), L.stream);
-  L.end();
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   ExArgs a = ex_args(ws, sp, y);
   MMBArgs mm{ws.active, ws.n_active, sp.n, sp.k, D, ws.Dt, ws.xcol, ws.LA2, ws.S, ws.W, ws.mass, ws.dw, ws.done,
              sp.penalty, sp.mm_steps, float(sp.eps), float(sp.alpha), float(sp.beta)};
@@ -364,6 +394,10 @@ inline cudaError_t ex_iterate(const Launch& L, const Workspace<float>& ws, const
 //   1024 x 64    26 / 50       26 / 54        51 / 74       101 / 86
 //   4000 x 64    68 / 99       68 / 120      136 / 169      270 / 212
 // so up to two problems per SM, and four where a problem is short.
+// Up to SMALL_ANY_N bins that holds for grids without a plan too (1024 bins, 20 iterations, one problem: 3.5
+// -> 1.9 ms, 300: 4.8 -> 3.8); longer ones then take the tiled log-domain applies (32 x 4096: 15.0 ms, one
+// launch 17.0).
+constexpr int SMALL_ANY_N = 2048;
 inline bool small_prefers(const SolveParams& sp, int sms) {
   return sp.dw_tol <= 0 && sp.n <= 4096 && sp.batch <= (sp.n <= 512 ? 4 : 2) * sms;
 }
@@ -377,8 +411,8 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
   const int batch = sp.batch, n = sp.n, k = sp.k;
   const double eps_ln2 = sp.eps * kLn2;
   const bool checks = ow && sp.check_every > 0;
-  if constexpr (sizeof(T) == 4) {
-    if (ex_serves(sp, C != nullptr, checks) && small_prefers(sp, sm_count())) {
+  auto small = [&]() -> cudaError_t {
+    if constexpr (sizeof(T) == 4) {
       const SmallSolve c{batch, n, k, sp.datafit, sp.penalty, sp.max_iter, sp.mm_steps, sp.eps, sp.lam, sp.alpha, sp.beta,
                          sp.tol, x, D, y, w, g, t_out, iters_out, err_out, status_out, ws.dw};
       L.begin(KIND_APPLY);
@@ -387,7 +421,10 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
       if (e == cudaSuccess && L.timer && L.timer->on) e = L.timer->harvest();
       return e;
     }
-  }
+    return cudaErrorInvalidValue;
+  };
+  const bool serves = sizeof(T) == 4 && ex_serves(sp, C != nullptr, checks), prefers = serves && small_prefers(sp, sm_count());
+  if (prefers && n <= SMALL_ANY_N) return small();
 
   PrepArgs<T> pa;
   pa.x = x; pa.D = D; pa.w_in = w; pa.g_in = g; pa.y = y;
@@ -401,6 +438,13 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
   L.begin(KIND_OTHER);
   prep_kernel<T><<<1184, 256, 0, L.stream>>>(pa);
   L.end();
+  ExPlanRead plan;
+  if constexpr (sizeof(T) == 4) {
+    if (serves) {
+      const cudaError_t e = plan.begin(L, ws, n);
+      if (e != cudaSuccess) return e;
+    }
+  }
   L.begin(KIND_OTHER);
   colsum_kernel<T><<<(k + 7) / 8, 256, 0, L.stream>>>(ws.Dt, ws.xcol, n, k);
   L.end();
@@ -439,7 +483,14 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
 
   bool by_expansion = false;
   if constexpr (sizeof(T) == 4) {
-    by_expansion = ex_serves(sp, C != nullptr, checks);
+    // a grid without a plan keeps the tiled log-domain applies (1024 x 1024, 20 iterations: 8.9 ms, rows summed
+    // one by one 17.8)
+    if (serves) {
+      const cudaError_t e = plan.end(L);
+      if (e != cudaSuccess) return e;
+    }
+    by_expansion = serves && (!plan.known || plan.nb > 0);
+    if (by_expansion && prefers) return small();
     if (by_expansion) {
       const cudaError_t e = ex_iterate(L, ws, sp, D, y);
       if (e != cudaSuccess) return e;

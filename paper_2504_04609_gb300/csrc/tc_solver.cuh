@@ -464,7 +464,6 @@ __global__ void __launch_bounds__(NT) tc_prep_src_kernel(TcIterArgs A) {
       }
 #pragma unroll
       for (int e = 0; e < EPT; ++e) {
-        const int j = e * NT + threadIdx.x;
         g[e] = tc_datafit(A, tc_log2_sum(a[e], mt), yv[e]);
       }
     } else {
@@ -807,10 +806,13 @@ __global__ void tc_finalize_kernel(FinArgs<float> F, TcIterArgs A) {
 // iterations: 11.9 -> 2.3 ms, no kernel matrix to stream) and batches whose GEMMs do not fill the SM
 // pairs (1024 problems of 1024 bins, 32 pair tiles, 50 iterations: 5.86 -> 4.33 ms); an apply takes the
 // expansion 27 us per million bins and a full GEMM less up to n = 4096 or so. A caller who sets the precision
-// schedule has asked for the GEMM's single product and keeps the GEMMs.
+// schedule has asked for the GEMM's single product and keeps the GEMMs. An expansion's work grows with the
+// blocks in reach, a GEMM's does not (1024 x 1024, 20 iterations: 1.84 ms at 11 blocks, 2.73 at 31, GEMMs
+// 2.31), hence the limit on the blocks above the small batches.
 constexpr long long TC_EXPANSION_BINS = 5 << 18;  // 1.25 million
-inline bool tc_prefers_expansion(int batch, int n, double single_until) {
-  return single_until == 0.0 && (batch <= TC_SMALL_BATCH || (long long)batch * n <= TC_EXPANSION_BINS);
+constexpr int TC_EXPANSION_BLOCKS = 18;
+inline bool tc_prefers_expansion(int batch, int n, int blocks) {
+  return batch <= TC_SMALL_BATCH || ((long long)batch * n <= TC_EXPANSION_BINS && blocks <= TC_EXPANSION_BLOCKS);
 }
 
 // Run Algorithm 1 with tensor-core applies and dictionary contractions (float buffers; x, D, y, w,
@@ -826,19 +828,10 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
   // early launches pay where an iteration is launch latency (256 problems of 1024 bins, 20 iterations: 1.97
   // -> 1.52 ms); where the row kernels fill the SMs for long they cost a little (4096 x 4096: 12.46 -> 12.52)
   const bool pdl = (long long)batch * n <= 8LL << 20;
-  // small batches: whole solves in one launch, as on an FP32 handle (with more than one problem per SM
-  // of a long grid the batched kernels below win)
-  if (sp.single_until == 0.0 && ex_serves(sp, C != nullptr, checks) && small_prefers(sp, sm_count()) &&
-      (batch <= sm_count() || n <= 2048)) {
-    const SmallSolve sc{batch, n, k, sp.datafit, sp.penalty, sp.max_iter, sp.mm_steps, sp.eps, sp.lam, sp.alpha, sp.beta,
-                        sp.tol, x, D, y, w, g, t_out, iters_out, err_out, status_out, ws.dw};
-    L.begin(KIND_APPLY);
-    cudaError_t r = small_solve(sc, L.stream);
-    L.end();
-    if (r == cudaSuccess) r = cudaStreamSynchronize(L.stream);
-    if (r == cudaSuccess && L.timer && L.timer->on) r = L.timer->harvest();
-    return r;
-  }
+  // the small batches' whole solves in one launch, as on an FP32 handle (with more than one problem per SM
+  // of a long grid the batched kernels win)
+  const bool serves = sp.single_until == 0.0 && ex_serves(sp, C != nullptr, checks);
+  const bool small = serves && small_prefers(sp, sm_count()) && (batch <= sm_count() || n <= 2048);
   PrepArgs<float> pa;
   pa.x = x; pa.D = D; pa.w_in = w; pa.g_in = g; pa.y = y;
   pa.xt = ws.xt; pa.Dt = ws.Dt; pa.xcol = ws.xcol; pa.W = ws.W; pa.G2 = ws.G2;
@@ -851,20 +844,35 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
   L.begin(KIND_OTHER);
   prep_kernel<float><<<1184, 256, 0, L.stream>>>(pa);
   L.end();
+  ExPlanRead plan;
+  const bool by_plan = serves && (small || tc_prefers_expansion(batch, n, 0));
+  if (by_plan) {
+    const cudaError_t e = plan.begin(L, ws, n);
+    if (e != cudaSuccess) return e;
+  }
   L.begin(KIND_OTHER);
   colsum_kernel<float><<<(k + 7) / 8, 256, 0, L.stream>>>(ws.Dt, ws.xcol, n, k);
   L.end();
-  // Expansion applies where they beat the GEMM applies: the host reads the plan of the grid (this
-  // path ends with a synchronisation anyway); a grid that does not qualify keeps the GEMMs.
-  bool by_expansion = ex_serves(sp, C != nullptr, checks) && tc_prefers_expansion(batch, n, sp.single_until);
-  if (by_expansion) {
-    cudaError_t e = ex_plan(ws.xt, n, ex_plan_of(ws), L.stream);
-    ++*L.counter;
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(L.host_flag, &ex_plan_of(ws)->nb, sizeof(int), cudaMemcpyDeviceToHost, L.stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(L.stream);
+  L.begin(KIND_OTHER);
+  tc_dsplit_kernel<<<1184, 256, 0, L.stream>>>(D, n, k, tw.kp, tw.ld, tw.Dhi, tw.Dlo, tw.Dthi, tw.Dtlo);
+  L.end();
+  // Expansion applies where they beat the GEMM applies, by the grid's plan; a grid without one keeps the
+  // GEMMs.
+  bool by_expansion = false;
+  if (by_plan) {
+    cudaError_t e = plan.end(L);
     if (e != cudaSuccess) return e;
-    by_expansion = *L.host_flag > 0;
+    by_expansion = plan.nb > 0 && tc_prefers_expansion(batch, n, plan.nb);
+    if (plan.nb > 0 && small) {
+      const SmallSolve sc{batch, n, k, sp.datafit, sp.penalty, sp.max_iter, sp.mm_steps, sp.eps, sp.lam, sp.alpha, sp.beta,
+                          sp.tol, x, D, y, w, g, t_out, iters_out, err_out, status_out, ws.dw};
+      L.begin(KIND_APPLY);
+      e = small_solve(sc, L.stream);
+      L.end();
+      if (e == cudaSuccess) e = cudaStreamSynchronize(L.stream);
+      if (e == cudaSuccess && L.timer && L.timer->on) e = L.timer->harvest();
+      return e;
+    }
   }
   if (!by_expansion) {
   L.begin(KIND_OTHER);
@@ -874,9 +882,6 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
     kbuild_kernel<<<2048, 256, 0, L.stream>>>(ws.xt, n, tw.ld, tw.Khi, tw.Klo, sp.cost == COST_ABS);
   L.end();
   }
-  L.begin(KIND_OTHER);
-  tc_dsplit_kernel<<<1184, 256, 0, L.stream>>>(D, n, k, tw.kp, tw.ld, tw.Dhi, tw.Dlo, tw.Dthi, tw.Dtlo);
-  L.end();
   cudaError_t e = cudaMemsetAsync(tw.err, 0, sizeof(int), L.stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(tw.hilo, sp.single_until > 0 ? 0 : 0xFF, 2 * sizeof(int), L.stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(tw.fix_cnt, 0, 2 * sizeof(unsigned long long), L.stream);
