@@ -9,8 +9,7 @@ source-marginal violation e <= tol, Algorithm 1 with one MM step per iteration) 
 Prints one JSON line (rank 0).  `value` = problems solved per second over all ranks (replicas:
 every rank solves its own batch, no collective on the data path).  `e2e` = the same metric through
 otlm_solve_host with pinned host buffers (host<->device copies inside the timed region).
-`roofline` = the dominant kernel (the kernel apply) against the exponent-unit peak; its launch
-durations are measured live with CUDA events on the solver's stream.  `cpu_baseline` = the FP64
+`roofline` = the dominant kernel (the kernel apply) against its peak; its launch durations are measured live with CUDA events on the solver's stream.  `cpu_baseline` = the FP64
 oracle (numpy, one thread) on a bounded sample of the same workload.
 `--impl reference` times that oracle alone (the CPU reference arm).
 """
@@ -39,7 +38,7 @@ WORKLOAD_METRICS = {
     "ragged": "OTLM problems solved/s to 1e-5 marginal tol, uneven batch (n ~ U{256..4096}) in one persistent launch",
     "warmstart": "OTLM problems solved/s to 1e-5 marginal tol, learned warm start vs cold start (n=2048)",
     "single": "OTLM single-target FP64 solve time (n=m=200, k=10, 500 iterations)",
-    "hbm": "single-target OTLM solves/s to 1e-5 marginal tol at n=16384 (stored kernel streamed from HBM)",
+    "hbm": "single-target OTLM solves/s to 1e-5 marginal tol at n=16384",
     "banded": "OTLM problems/s to 1e-5 marginal tol, banded cost + sparse dictionary at n=100000 "
               "(the paper's scalability test)",
 }
@@ -431,6 +430,28 @@ def tc_apply_roofline(workload, n, iters, apply_timing, peaks, iters_hilo=None, 
     return r
 
 
+# Tensor-core handles run grid solves without the precision schedule as block expansions where their
+# GEMMs do not fill the SM pairs.
+EXPANSION_BATCH, EXPANSION_BINS = 64, 5 << 18
+
+
+def tc_runs_expansions(batch, n, single_until):
+    return single_until == 0.0 and (batch <= EXPANSION_BATCH or batch * n <= EXPANSION_BINS)
+
+
+def expansion_apply_roofline(terms, bins, apply_timing, peaks, kernel):
+    """Roofline of a block-expansion apply: what it cannot do without is its state in HBM, 20 bytes per
+    bin (potential, previous sum and mass or target read, sum and potential written); it is bound by
+    instruction issue.  `terms` = kernel entries the plain sums would evaluate, one exp2 each."""
+    g_ms, g_cnt = apply_timing
+    peak = float(peaks.get("hbm_gbs", 6800.0))
+    achieved = 20.0 * bins / (g_ms / 1e3) / 1e9
+    return {"bound": "issue", "kernel": kernel, "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+            "traffic": None, "launch_ms_avg": g_ms / max(g_cnt, 1), "plain_sum_terms_g_per_s": terms / (g_ms / 1e3) / 1e9,
+            "peak_basis": "MEASURED_PEAKS.json hbm_gbs" if "hbm_gbs" in peaks else "fallback 6.8 TB/s",
+            "note": "state bytes against HBM (the floor); issue bound"}
+
+
 def run_ours(args, rank, world, local_rank, pool=None):
     import torch
     import torch.distributed as dist
@@ -538,24 +559,24 @@ def run_ours(args, rank, world, local_rank, pool=None):
     peaks = _peaks()
 
     it_tc = tc["iters"].astype(np.float64)
-    roofline = tc_apply_roofline(args.workload, n, tc["iters"], tc["timing"]["apply"], peaks,
-                                 tc3["iters"] if tc3 is not None else None,
-                                 tc3["timing"]["apply"] if tc3 is not None else None)
+    applies = float(np.sum(2 * it_tc + 1))
+    expansions = tc_runs_expansions(B, n, sched)
+    if expansions:
+        roofline = expansion_apply_roofline(applies * n * n, applies * n, tc["timing"]["apply"], peaks,
+                                            "ex_apply_kernel (FP32 block expansions)")
+    else:
+        roofline = tc_apply_roofline(args.workload, n, tc["iters"], tc["timing"]["apply"], peaks,
+                                     tc3["iters"] if tc3 is not None else None,
+                                     tc3["timing"]["apply"] if tc3 is not None else None)
 
-    # plain FP32 path: the log-sum-exp apply against the exponent unit
+    # plain FP32 path: block expansions of the log-domain sums
     it_fp = fp["iters"].astype(np.float64)
-    exps_step = float(n) * n * float(np.sum(2 * it_fp + 1))
-    a_ms, a_cnt = fp["timing"]["apply"]
-    ach = exps_step / (a_ms / 1e3) / 1e9
-    peak_ex = SMS * EX2_PER_SM_CLK * MAX_SM_MHZ * 1e6 / 1e9
+    fp_applies = float(np.sum(2 * it_fp + 1))
     plain = {"value": fp_value, "unit": "problems/s", "ms_per_step": fp_ms / fp_steps, "steps": fp_steps,
              "mean_iters": float(it_fp.mean()), "converged": int(np.sum(fp["status"] == 0)),
              "kernel_ms_per_step": {kk: v[0] for kk, v in fp["timing"].items()},
-             "roofline": {"bound": "alu", "kernel": "apply_kernel (FP32 log-sum-exp)", "achieved": ach,
-                          "peak": peak_ex, "unit": "Gexp2/s", "frac": ach / peak_ex, "traffic": None,
-                          "launch_ms_avg": a_ms / max(a_cnt, 1),
-                          "peak_basis": f"{SMS} SMs x {EX2_PER_SM_CLK} ex2/clk x {MAX_SM_MHZ:.0f} MHz (derived; "
-                                        "probe measured 30.3 ex2/clk/SM)"},
+             "roofline": expansion_apply_roofline(fp_applies * n * n, fp_applies * n, fp["timing"]["apply"], peaks,
+                                                  "ex_apply_kernel (FP32 block expansions)"),
              "clocks": fp["clocks"]}
     out = {
         "metric": workload_metric(args.workload),
@@ -568,11 +589,12 @@ def run_ours(args, rank, world, local_rank, pool=None):
         "higher_is_better": True,
         "scaling": "weak",
         "vs_baseline": None,
-        "dtype": "bf16x3 tensor (hi/lo split) + f32" + (", bf16x1 until a violation <= %g" % sched if sched else ""),
+        "dtype": "f32" if expansions else "bf16x3 tensor (hi/lo split) + f32" + (", bf16x1 until a violation <= %g" % sched if sched else ""),
         "data": "synthetic (seeded Gaussian-peak spectra, no dataset)",
         "config": {"workload": args.workload, "B_per_gpu": B, "n": n, "k": k, "eps": c["eps"],
                    "datafit": c["datafit"], "lam": c["lam"], "penalty": c["penalty"], "alpha": c["alpha"],
-                   "tol": c["tol"], "path": "tensor-core applies (tcgen05, BF16 hi/lo, FP32 accumulate)",
+                   "tol": c["tol"], "path": ("FP32 block expansions (GEMMs would not fill the SM pairs)" if expansions else
+                                             "tensor-core applies (tcgen05, BF16 hi/lo, FP32 accumulate)"),
                    "bf16_single_until": sched,
                    "parallelism": f"replicas x{world}",
                    "l2": "inputs larger than L2 (4096 x 4096 FP32 state arrays, 64 MiB each, several per step)",
@@ -716,10 +738,8 @@ def run_ragged(args, rank, world, local_rank, pool=None):
         if own_pool:
             pool.close()
         return None
-    exps_step = float(np.sum(n_np.astype(np.float64) ** 2 * (2 * it_np + 1)))
-    k_ms = timing["apply"][0]  # one step
-    ach = exps_step / (k_ms / 1e3) / 1e9
-    peak_ex = SMS * EX2_PER_SM_CLK * MAX_SM_MHZ * 1e6 / 1e9
+    bins = float(np.sum(n_np.astype(np.float64) * (2 * it_np + 1)))  # one step
+    exps = float(np.sum(n_np.astype(np.float64) ** 2 * (2 * it_np + 1)))
     h2d = (hx.numel() + hD.numel() + hy.numel() + hw0.numel()) * 4
     d2h = (hw.numel() + ht.numel() + hit.numel()) * 4
     out = {
@@ -735,11 +755,9 @@ def run_ragged(args, rank, world, local_rank, pool=None):
                    "converged": int(np.sum(st_np == 0)), "iters_p50": float(np.percentile(it_np, 50)),
                    "iters_p99": float(np.percentile(it_np, 99)), "iters_mean": float(it_np.mean())},
         "iters_per_s": float(it_np.sum()) * world * args.steps / (ms / 1e3),
-        "roofline": {"bound": "alu", "kernel": "ragged_kernel (persistent, whole solve)", "achieved": ach,
-                     "peak": peak_ex, "unit": "Gexp2/s", "frac": ach / peak_ex, "traffic": None,
-                     "launch_ms_avg": timing["apply"][0] / max(timing["apply"][1], 1),
-                     "note": "algorithmic exp2 = sum_p n_p^2 (2 iters_p + 1); the kernel also runs the MM and "
-                             "source steps, so the fraction is a lower bound for the apply itself"},
+        "roofline": dict(expansion_apply_roofline(exps, bins, timing["apply"], _peaks(), "ragged_kernel (persistent, whole solve)"),
+                         note="state bytes of the applies against HBM; the kernel also runs the MM and source steps, whose "
+                              "dictionary reads bound it"),
         "e2e": {"value": whole_job_rate(B, world, max(1, args.steps), e2e_s), "unit": "problems/s", "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h},
         "gpu_launches": launches,
@@ -910,9 +928,8 @@ HBM_ITERS_TO_TOL = 22
 
 
 def run_single_hbm(args, rank, world, local_rank):
-    """One target at n = 16384 on the tensor-core path: the stored kernel (BF16 hi/lo, 4 n^2 bytes =
-    1 GiB) is streamed from HBM by each of the two applies per iteration, so the apply is bound by
-    HBM bandwidth.  Each rank solves its own target (replicas)."""
+    """One target at n = 16384 on a tensor-core handle, which runs a batch this small as block
+    expansions spread over the chip.  Each rank solves its own target (replicas)."""
     import torch
     import torch.distributed as dist
 
@@ -988,29 +1005,19 @@ def run_single_hbm(args, rank, world, local_rank):
     if rank != 0:
         return None
 
-    # the apply streams the stored kernel once: 4 n^2 bytes (BF16 hi + lo) per launch; the operand
-    # (4 n bytes) and the sums (4 n bytes) are negligible beside it
-    a_ms, a_cnt = timing["apply"]
-    launch_ms = a_ms / max(a_cnt, 1)
-    achieved = 4.0 * n * n / (launch_ms / 1e3) / 1e9
-    peak = float(_peaks().get("hbm_gbs", 6800.0))
     out = {
         "metric": workload_metric(args.workload),
         "value": whole_job_rate(B, world, args.steps, ms / 1e3), "unit": "problems/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak",
         "iters_per_s": whole_job_rate(B, world, args.steps, ms / 1e3) * it,
-        "vs_baseline": None, "dtype": "bf16x3 tensor (hi/lo split) + f32",
+        "vs_baseline": None, "dtype": "f32",
         "data": "synthetic (seeded Gaussian-peak spectra, no dataset)",
         "config": {"workload": args.workload, "B_per_gpu": B, "n": n, "k": k, "eps": c["eps"], "datafit": c["datafit"],
                    "penalty": c["penalty"], "tol": c["tol"], "iters": it, "status": st,
-                   "path": "tensor-core applies with the reduction split over 16 ranges (small batch)",
-                   "l2": "the stored kernel (1 GiB) is larger than L2", "parallelism": f"replicas x{world}"},
-        "roofline": {"bound": "hbm", "kernel": "gemm3_kernel<KIND_BF16> + tc_split_reduce_kernel (one apply)",
-                     "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                     "traffic": 1081.2e6, "traffic_note": "GEMM 1079.4 MB read + 0.9 MB written, split reduce "
-                                                          "0.9 MB read (ncu, profiles/hbm_single_n16384.md)",
-                     "launch_ms_avg": launch_ms, "bytes_per_launch": 4.0 * n * n,
-                     "peak_basis": "MEASURED_PEAKS.json hbm_gbs" if "hbm_gbs" in _peaks() else "fallback 6.8 TB/s"},
+                   "path": "FP32 block expansions (small batch; no kernel matrix is stored)",
+                   "l2": "the state and the dictionary (9 MB) stay in L2", "parallelism": f"replicas x{world}"},
+        "roofline": expansion_apply_roofline((2.0 * it + 1) * n * n, (2.0 * it + 1) * n, timing["apply"], _peaks(),
+                                             "ex_apply_kernel (FP32 block expansions, one target over the chip)"),
         "kernel_ms_per_step": {kk: v[0] for kk, v in timing.items()},
         "e2e": {"value": whole_job_rate(B, world, max(1, args.steps), e2e_s), "unit": "problems/s",
                 "h2d_bytes_per_step": (hx.numel() + hD.numel() + hy.numel() + hw.numel()) * 4,
@@ -1293,10 +1300,9 @@ def main():
                 ws = out["workloads"].get("warmstart", {})
                 out["targets"] = {
                     "warm_bf16_vs_plain_fp32_ge_5x": ws.get("target_5x_met"),
-                    "memory_bound_apply_hbm_roofline_ge_0.7": (out["workloads"].get("hbm_single", {}).get("roofline", {})
-                                                       .get("frac", 0.0) >= 0.7),
-                    "note": "the HBM target applies to the memory-bound apply (single target, stored kernel); the "
-                            "log-domain FP32 applies are exponent-unit bound (plain_fp32.roofline)"}
+                    "memory_bound_apply_hbm_roofline_ge_0.7": None,
+                    "note": "no default workload streams a stored kernel any more: the single target runs block "
+                            "expansions, and the plain FP32 solve does too (the 5x target compares with it)"}
         if world > 1:
             import torch.distributed as dist
             dist.destroy_process_group()

@@ -83,14 +83,18 @@ typedef enum {            /* grid cost of otlm_solve / otlm_solve_host / otlm_ob
 
 typedef enum {
   OTLM_PREC_FP32_LOG = 0,     /* FP32, scalings carried as log2 potentials (stable at small eps) */
-  OTLM_PREC_FP64     = 1,     /* FP64 throughout, same log-domain arithmetic                   */
+  OTLM_PREC_FP64     = 1,     /* FP64 throughout: linear scalings against a stored kernel up to
+                                 n = 4096, log-domain arithmetic beyond and outside 2^+-900    */
   OTLM_PREC_BF16_TC  = 2      /* kernel applies as tensor-core GEMMs K V^T: BF16 hi/lo operands
                                  (three products, ~16 mantissa bits), FP32 accumulation, a
                                  per-problem max shift; potentials and updates in FP32.  Element
                                  type float.  Rows whose sum underflows (all significant terms
                                  below 2^-126 of the problem's largest) are recomputed exactly in
                                  the log domain.  otlm_objective on such a handle runs FP32 applies
-                                 (the in-solve objective of check_every runs tensor-core ones). */
+                                 (the in-solve objective of check_every runs tensor-core ones).
+                                 Squared grid costs without bf16_single_until run the FP32 path's
+                                 block expansions where the GEMMs would not fill the chip (batches
+                                 of up to 64 problems, or 1.25 million bins in all). */
 } otlm_precision;
 
 typedef struct otlm_config {
@@ -148,6 +152,8 @@ typedef struct otlm_ctx* otlm_handle;
 /* Create a handle and its device workspace (about (8 n_max + 2 k_max + 16) * batch_max
  * elements).  `cuda_stream` is a cudaStream_t (NULL = default stream).  The workspace is
  * owned by the handle and released by otlm_destroy.
+ * An FP64 handle with n_max <= 4096 also tries for the stored kernel's buffer; without it, its solves
+ * run in the log domain.
  * With check_every > 0 the workspace also holds the objective scratch (3 batch_max n_max elements
  * and 20 batch_max bytes).
  * Errors: OTLM_EINVAL (null pointers, sizes out of range, unknown enum, ELASTIC without a
@@ -229,7 +235,7 @@ int otlm_solve_host(otlm_handle h, int batch, int n, int k,
  * The handle must be OTLM_PREC_FP32_LOG with mm_steps <= 1 (else OTLM_EUNSUPPORTED); datafit,
  * penalty, beta, max_iter, tol and poll_every come from it; batch <= batch_max, while n and k are
  * not bounded by n_max and k_max: the banded workspace (about 4 (6 batch n + batch k + (2hw+1) n
- * + 2 nnz + 3 n) bytes) is allocated on the first call and grown when a later call needs more.
+ * + 6 nnz + 3 n) bytes) is allocated on the first call and grown when a later call needs more.
  * The band and dictionary are validated on the device before use (one host synchronisation).
  * Errors: OTLM_EINVAL (sizes, eps, lam, alpha as otlm_solve, hw out of range, NULL pointers, a
  * malformed band or dictionary), OTLM_EUNSUPPORTED, OTLM_ENOMEM, OTLM_ECUDA. */

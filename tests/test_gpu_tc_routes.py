@@ -53,6 +53,21 @@ def test_grid_solves_of_every_batch_size(B, n, k, mm_steps):
              "l2sq", 8, mm_steps)
 
 
+@pytest.mark.parametrize("precision", ["fp32", "bf16tc"])
+@pytest.mark.parametrize("B,n", [(2, 300), (2, 2100), (620, 300)])
+def test_grids_without_a_plan(precision, B, n):
+    """An unsorted grid keeps the log-domain or GEMM applies (or one launch) at every batch size."""
+    d = spectra.batch(96, 2, n, 12, 3)
+    perm = np.random.default_rng(5).permutation(n)
+    d = dict(d, x=d["x"][perm], D=np.ascontiguousarray(d["D"][perm]), y=np.ascontiguousarray(d["y"][:, perm]))
+    y = d["y"][np.arange(B) % 2]
+    w0 = spectra.initial_weights(y, d["D"]).astype(np.float32)
+    r = api.solve(_dev(d["x"]), _dev(d["D"]), _dev(y), 2e-2, 1.0, 1e-3, "l2", "l2sq", _dev(w0), max_iter=8,
+                  precision=precision)
+    _compare(dict(w=r.w, t=r.t), d, B, oracle.solve_log, spectra.squared_cost(d["x"].astype(np.float64)), 2e-2, 1e-3, "l2",
+             "l2sq", 8)
+
+
 @pytest.mark.parametrize("B", [65, 150, 256])
 @pytest.mark.parametrize("n", [300, 1000])
 def test_dense_cost_split_reductions_of_mid_size_batches(B, n):
