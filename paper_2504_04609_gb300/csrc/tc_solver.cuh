@@ -38,8 +38,9 @@ namespace otlm {
 // Small batches leave the applies with fewer 128 x 128 output tiles than SMs (a single target at
 // n = 8192 has 64), so for batches up to TC_SMALL_BATCH the reduction of each apply is split into up
 // to TC_APPLY_SPLITS ranges whose partial sums are added by tc_split_reduce_kernel.
-// Larger batches split while their tiles leave half of the SMs idle (256 problems of 1024 bins are 16
-// tiles: 23 us per apply on 8 SM pairs, 12 with the reduction over nine ranges and their sum).
+// Larger batches split while their tiles leave three quarters of the SMs idle (256 problems of 1024 bins are
+// 16 tiles: 23 us per apply on 8 SM pairs, 12 with the reduction over nine ranges and their sum); at 64 tiles
+// (1024 x 1024, 20 iterations on the GEMMs) the SM pairs without the split are: 1.87 ms, 2.39 split.
 constexpr int TC_SMALL_BATCH = 64, TC_APPLY_SPLITS = 16;
 constexpr size_t TC_ACCP_FLOATS = (size_t)6 << 20;
 
@@ -807,8 +808,8 @@ __global__ void tc_finalize_kernel(FinArgs<float> F, TcIterArgs A) {
 // pairs (1024 problems of 1024 bins, 32 pair tiles, 50 iterations: 5.86 -> 4.33 ms); an apply takes the
 // expansion 27 us per million bins and a full GEMM less up to n = 4096 or so. A caller who sets the precision
 // schedule has asked for the GEMM's single product and keeps the GEMMs. An expansion's work grows with the
-// blocks in reach, a GEMM's does not (1024 x 1024, 20 iterations: 1.84 ms at 11 blocks, 2.73 at 31, GEMMs
-// 2.31), hence the limit on the blocks above the small batches.
+// blocks in reach, a GEMM's does not (1024 x 1024, 20 iterations: 1.83 ms at eps = 1e-2, 2.73 at 1e-3, GEMMs
+// 1.87), hence the limit on the blocks above the small batches.
 constexpr long long TC_EXPANSION_BINS = 5 << 18;  // 1.25 million
 constexpr int TC_EXPANSION_BLOCKS = 18;
 inline bool tc_prefers_expansion(int batch, int n, int blocks) {
@@ -915,7 +916,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
   ga.hilo = tw.hilo; ga.pdl = pdl;
   {
     const int units = ((n + tc::BM - 1) / tc::BM) * ((batch + tc::BN - 1) / tc::BN);
-    if (batch <= TC_SMALL_BATCH ? units < tc::num_sms() : 2 * units <= tc::num_sms()) {
+    if (batch <= TC_SMALL_BATCH ? units < tc::num_sms() : 4 * units <= tc::num_sms()) {
       ga.splits = tc::choose_splits(units, (n + tc::KindTraits<tc::KIND_BF16>::BK - 1) / tc::KindTraits<tc::KIND_BF16>::BK);
       if (ga.splits > TC_APPLY_SPLITS) ga.splits = TC_APPLY_SPLITS;
       while (ga.splits > 1 && (size_t)ga.splits * batch * n > tw.accp_floats) --ga.splits;
