@@ -70,6 +70,12 @@ struct F64Row {
 __device__ __forceinline__ double f64_log2a(const F64Buf& F, const double* a, size_t idx) {
   return F.IA[idx] > 0.0 ? ::log2(a[idx]) : a[idx];
 }
+// log2(a / s) of a linear a with ia = 1 / a and s > 0: one logarithm while s ia is a normal number.  Far
+// from every atom s passes through 2^-1022 .. 2^-1074 and s ia is rounded to few bits or to 0.
+__device__ __forceinline__ double f64_log_ratio(double a, double ia, double s) {
+  const double q = s * ia;
+  return q >= 0x1p-1022 && q <= 0x1p1023 ? -::log2(q) : ::log2(a) - ::log2(s);
+}
 
 template <int EPI, int PB, int NWARP>
 __global__ void __launch_bounds__(32 * NWARP) f64_apply_kernel(ApplyArgs<double> A, F64Buf F, const double* aout, double* R,
@@ -151,7 +157,7 @@ __global__ void __launch_bounds__(32 * NWARP) f64_apply_kernel(ApplyArgs<double>
           const double ia = rw.log ? 0.0 : 1.0 / rw.v;
           A.out[idx] = rw.v;
           F.IA[idx] = ia;
-          R[idx] = s > 0.0 ? (rw.log ? rw.v - P::log2(s) : -P::log2(s * ia)) : 0.0;
+          R[idx] = s > 0.0 ? (rw.log ? rw.v - P::log2(s) : f64_log_ratio(rw.v, ia, s)) : 0.0;
         }
       } else {
         const double v = rw.log ? rw.v : P::log2(rw.v);
@@ -231,7 +237,7 @@ __global__ void __launch_bounds__(256) f64_mm_kernel(MMArgs<double> A) {
           r = A.R[o + i];
         } else {
           const double s = S[i], ia = A.IA[o + i];
-          r = s > 0.0 ? (ia > 0.0 ? -P::log2(s * ia) : A.LA2[o + i] - P::log2(s)) : 0.0;
+          r = s > 0.0 ? (ia > 0.0 ? f64_log_ratio(A.LA2[o + i], ia, s) : A.LA2[o + i] - P::log2(s)) : 0.0;
         }
       }
       const int cnt = min(32, n - base);
