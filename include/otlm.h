@@ -84,7 +84,8 @@ typedef enum {            /* grid cost of otlm_solve / otlm_solve_host / otlm_ob
 typedef enum {
   OTLM_PREC_FP32_LOG = 0,     /* FP32, scalings carried as log2 potentials (stable at small eps) */
   OTLM_PREC_FP64     = 1,     /* FP64 throughout: linear scalings against a stored kernel up to
-                                 n = 4096, log-domain arithmetic beyond and outside 2^+-900    */
+                                 n = 4096, log-domain arithmetic beyond and for every sum that a
+                                 term outside FP64's range could matter to                     */
   OTLM_PREC_BF16_TC  = 2      /* kernel applies as tensor-core GEMMs K V^T: BF16 hi/lo operands
                                  (three products, ~16 mantissa bits), FP32 accumulation, a
                                  per-problem max shift; potentials and updates in FP32.  Element

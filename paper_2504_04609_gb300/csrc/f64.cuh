@@ -6,8 +6,12 @@
 // scalings are kept in the linear domain, u = 2^G2, where FP64's range (2^+-1022) holds them:
 //   a_i = sum_j K_ij u1_j,   b_j = sum_i K_ij u2_i        (K is symmetric for a grid cost)
 // one multiply-add per element, rows spread over all SMs.  The potentials' logarithms stay the
-// state.  A sum outside [2^-900, 2^900] (where terms that matter may have left the range) is redone
-// from the potentials around its largest term.
+// state.  A sum is taken only where nothing that left the range can matter to it, and redone from the
+// potentials around its largest term elsewhere:
+//   - within [2^-900, 2^900]: what a scaling below 2^-1022 lost is at most n 2^-1074 in all;
+//   - at least 2^-1000 times the problem's largest scaling: an entry K_ij below 2^-1022 is off by at
+//     most 2^-1074, which a scaling of 2^1000 (transport beyond sqrt(1022 eps ln2)) makes visible; n times
+//     that times the largest scaling is then below 2^-62 of the sum (n <= 4096).
 //   one target, n = 200, k = 10, 500 iterations: 765 ms with log-sum-exp tiles of 4 problems x 128
 //   rows (2 CTAs on 2 SMs), 17 ms now, three launches of 8 to 12 us per iteration whose serial FP64
 //   logarithms are what is left; objective of 16 problems, n = 512: 3.2 ms -> 149 us.
@@ -95,22 +99,33 @@ __global__ void __launch_bounds__(32 * NWARP) f64_apply_kernel(ApplyArgs<double>
   }
   const double* U = EPI == EPI_SOURCE ? F.U1 : F.U2;
   double acc[PB];
+  int top[PB];  // largest upper half of the scalings (>= 0): their order, and the exponent
 #pragma unroll
-  for (int q = 0; q < PB; ++q) acc[q] = 0.0;
+  for (int q = 0; q < PB; ++q) {
+    acc[q] = 0.0;
+    top[q] = 0;
+  }
 #pragma unroll 4
   for (int j = i < n ? lane : n; j < n; j += 32) {
     const double k = F.K[(size_t)i * n + j];
 #pragma unroll
     for (int q = 0; q < PB; ++q)
-      if (p[q] >= 0) acc[q] = fma(k, U[(size_t)p[q] * n + j], acc[q]);
+      if (p[q] >= 0) {
+        const double u = U[(size_t)p[q] * n + j];
+        acc[q] = fma(k, u, acc[q]);
+        top[q] = max(top[q], __double2hiint(u));
+      }
   }
 #pragma unroll
   for (int q = 0; q < PB; ++q) {
     for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+    top[q] = __reduce_max_sync(0xffffffffu, top[q]);
     if (p[q] < 0 || i >= n) continue;
     const size_t o = (size_t)p[q] * n;
     F64Row rw{acc[q], 0};
-    if (!(acc[q] >= 0x1p-900 && acc[q] <= 0x1p900)) {  // rare: from the potentials, around the largest term
+    // the largest scaling is below 2^(exponent + 1); its bound of the sum, at least 2^-900
+    const int low = max((top[q] >> 20) - 1023 + 1 - 1000, -900);
+    if (!(acc[q] >= __hiloint2double((low + 1023) << 20, 0) && acc[q] <= 0x1p900)) {  // rare: from the potentials
       const double xi = A.xt[i];
       auto term = [&](int j) {
         const double d = xi - A.xt[j];
