@@ -125,6 +125,11 @@ __device__ __forceinline__ double wright_omega_f64(double z) {
   const double r = z - w - ::log(w), u = 1.0 + w, t = u * (u + (2.0 / 3.0) * r);
   return w + w * (r * (t - 0.5 * r)) / (u * (t - r));
 }
+// log(c w) with one logarithm while the product is a normal number.
+__device__ __forceinline__ double log_product(double c, double w) {
+  const double v = c * w;
+  return v >= 0x1p-1022 && v <= 0x1p1023 ? ::log(v) : ::log(c) + ::log(w);
+}
 template <typename T>
 __device__ __forceinline__ T wright_omega_of(T z) {
   if constexpr (sizeof(T) == 8) return wright_omega_f64(z);

@@ -286,8 +286,10 @@ __global__ void __launch_bounds__(256) f64_mm_kernel(MMArgs<double> A) {
       // l1 and elastic net: shifted by alpha / (eps x_j) = alpha ix / (eps ln2)
       const double shift = (A.penalty == PEN_L1 || A.penalty == PEN_ELASTIC) ? A.alpha * ix_s[j] / (A.eps * kLn2) : 0.0;
       double wn;
-      if (A.penalty == PEN_L2SQ || A.penalty == PEN_ELASTIC) wn = wright_omega_f64(P::log(c_s[j] * wold) + dl - shift) * ic_s[j];
-      else wn = fabs(dl - shift) < 600.0 ? wold * P::exp(dl - shift) : P::exp(P::log(wold) + dl - shift);
+      if (A.penalty == PEN_L2SQ || A.penalty == PEN_ELASTIC) {
+        const double om = wright_omega_f64(log_product(c_s[j], wold) + dl - shift);
+        wn = ic_s[j] <= 0x1p1023 ? om * ic_s[j] : om / c_s[j];
+      } else wn = fabs(dl - shift) < 600.0 ? wold * P::exp(dl - shift) : P::exp(P::log(wold) + dl - shift);
       w_s[j] = wn;
       if (m + 1 == A.mm_steps) A.W[(size_t)p * k + j] = wn;
     }

@@ -620,7 +620,7 @@ __global__ void __launch_bounds__(256) mm_kernel(MMArgs<T> A) {
       T wn;
       if (A.penalty == PEN_L2SQ || A.penalty == PEN_ELASTIC) {
         const T c = (A.penalty == PEN_ELASTIC ? A.beta : A.alpha) / (A.eps * xj);
-        if constexpr (sizeof(T) == 8) wn = wright_omega_of<T>(P::log(c * wold) + dl - shift) / c;  // one logarithm
+        if constexpr (sizeof(T) == 8) wn = wright_omega_of<T>(log_product(c, wold) + dl - shift) / c;
         else wn = wright_omega_of<T>(P::log(c) + (P::log(wold) + dl) - shift) / c;
       } else wn = P::exp((P::log(wold) + dl) - shift);
       A.W[(size_t)p * k + j] = wn;

@@ -1,6 +1,7 @@
 """FP64 solves and objective where products or kernel entries leave FP64's range, against the FP64
-oracle at the path's 1e-9: source marginals down to the subnormals, and transport so far that
-exp(-C / eps) underflows where mass still moves.  The oracle works on logarithms throughout."""
+oracle at the path's 1e-9: source marginals down to the subnormals, weights whose product with the
+penalty's coefficient is subnormal, and transport so far that exp(-C / eps) underflows where mass
+still moves.  The oracle works on logarithms throughout."""
 import numpy as np
 import pytest
 from scipy.special import logsumexp
@@ -101,3 +102,28 @@ def test_objective_of_transport_beyond_the_stored_kernel(datafit, B):
     t = Q.sum(axis=0)
     fit = np.sum(t * np.log(t / y[0]) - t + y[0]) if datafit == "kl" else np.abs(t - y[0]).sum()
     np.testing.assert_allclose(out[400][0], eps * kl + fit + 1e-2 * o["w"].sum(), rtol=TOL64)
+
+
+@pytest.mark.parametrize("n_max", [0, 4097])
+@pytest.mark.parametrize("penalty", ["l2sq", "elastic"])
+@pytest.mark.parametrize("w_start,coef", [(1e-300, 1e-20), (0.5, 1e-312)])
+def test_weights_whose_product_with_the_coefficient_is_subnormal(n_max, penalty, w_start, coef):
+    """w = 1e-300 with alpha / (eps x_j) = 1e-18, and a coefficient whose reciprocal overflows (stored
+    kernel and log-sum-exp applies)."""
+    rng = np.random.default_rng(73)
+    n, k = 200, 3
+    x = np.arange(n) / (n - 1)
+    D = _peaks(x, [0.25, 0.5, 0.7], 0.03)
+    y = (D @ rng.gamma(2.0, 1.0, (k, 2)) + 1e-3).T.copy()
+    w0 = np.full((2, k), w_start)
+    dev = lambda a: torch.tensor(a, dtype=torch.float64, device="cuda")  # noqa: E731
+    w = dev(w0)
+    alpha, beta = (coef, 0.0) if penalty == "l2sq" else (1e-3, coef)
+    h = api.Handle(max(n, n_max), k, 2, "fp64", "kl", penalty, 2, 0.0, 5, stream=torch.cuda.current_stream().cuda_stream,
+                   beta=beta)
+    h.solve(dev(x), dev(D), dev(y), 1e-2, 1.0, alpha, w)
+    torch.cuda.synchronize()
+    h.close()
+    for p in range(2):
+        o = oracle.solve_log(spectra.squared_cost(x), D, y[p], 1e-2, 1.0, alpha, "kl", penalty, w0[p], 2, beta=beta)
+        assert rel_l1(w[p].cpu().numpy(), o["w"]) <= TOL64
