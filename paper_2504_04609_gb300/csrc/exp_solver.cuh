@@ -280,9 +280,9 @@ inline int exa_parts(int batch, int n, int sms) {
 template <int EPI, bool TC, int T>
 static inline cudaError_t launch_ex_cfg(const ExArgs& a, int batch, int parts, cudaStream_t stream) {
   const size_t smem = exa_smem_bytes(a.n, T);
-  if (smem > 48 * 1024) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(ex_apply_kernel<EPI, TC, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > 48 * 1024) {  // the largest size for every call: the limit is the process's, threads would lower it
+    const cudaError_t e = cudaFuncSetAttribute(ex_apply_kernel<EPI, TC, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)exa_smem_bytes(EXA_MAX_N, T));
     if (e != cudaSuccess) return e;
   }
   // CTAs that leave SMs idle are launched late: early ones share SMs beside a running GEMM (one target at

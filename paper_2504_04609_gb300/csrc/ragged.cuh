@@ -533,18 +533,28 @@ constexpr int RAGGED_VARIANTS = 3;
 inline int ragged_nt(int v) { return v == 0 ? 128 : (v == 1 ? 256 : 512); }
 inline int ragged_rmax_log2(int v) { return v == 0 ? 5 : (v == 1 ? 4 : 3); }
 
+// Dynamic shared memory of variant v for n <= n_max, k <= k_max; *fn: its kernel. The kernel's limit is one
+// value for the process and is set to the largest size there is (RAGGED_N_MAX bins, 256 atoms): a limit
+// that followed the call would be lowered by one host thread between another's setting and launch.
+constexpr int RAGGED_N_MAX = 4096, RAGGED_K_MAX = 256;
+template <int NT, int RMAX>
+inline cudaError_t ragged_allow(int n_max, int k_max, size_t* smem, const void** fn) {
+  static_assert(RAGGED_N_MAX <= NT * RMAX, "rows per thread cover the largest problem");
+  *smem = RaggedSmem<NT>::floats(n_max, k_max) * 4;
+  *fn = (const void*)ragged_kernel<NT, RMAX>;
+  return cudaFuncSetAttribute(*fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(RaggedSmem<NT>::floats(RAGGED_N_MAX, RAGGED_K_MAX) * 4));
+}
+inline cudaError_t ragged_allow(int v, int n_max, int k_max, size_t* smem, const void** fn) {
+  if (n_max > RAGGED_N_MAX || k_max > RAGGED_K_MAX) return cudaErrorInvalidValue;
+  if (v == 0) return ragged_allow<128, 32>(n_max, k_max, smem, fn);
+  if (v == 1) return ragged_allow<256, 16>(n_max, k_max, smem, fn);
+  return ragged_allow<512, 8>(n_max, k_max, smem, fn);
+}
 inline cudaError_t ragged_prepare(int v, int n_max, int k_max, int* blocks_per_sm, size_t* smem) {
-  const int nt = ragged_nt(v);
-  size_t bytes = 0;
   const void* fn = nullptr;
-  if (v == 0) { bytes = RaggedSmem<128>::floats(n_max, k_max) * 4; fn = (const void*)ragged_kernel<128, 32>; }
-  else if (v == 1) { bytes = RaggedSmem<256>::floats(n_max, k_max) * 4; fn = (const void*)ragged_kernel<256, 16>; }
-  else { bytes = RaggedSmem<512>::floats(n_max, k_max) * 4; fn = (const void*)ragged_kernel<512, 8>; }
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) return e;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, nt, bytes);
-  *smem = bytes;
-  return e;
+  const cudaError_t e = ragged_allow(v, n_max, k_max, smem, &fn);
+  return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, ragged_nt(v), *smem);
 }
 
 // A small batch sharing grid, dictionary and eps, whole solves in one launch (one CTA per problem).
@@ -553,11 +563,10 @@ inline cudaError_t ragged_prepare(int v, int n_max, int k_max, int* blocks_per_s
 inline cudaError_t ragged_small(const RaggedArgs& a0, cudaStream_t s) {
   RaggedArgs a = a0;
   const int v = a.n_all <= 512 ? 1 : 2;
-  int bps = 0;
   size_t smem = 0;
-  const cudaError_t e = ragged_prepare(v, a.n_all, a.k_all, &bps, &smem);
+  const void* fn = nullptr;
+  const cudaError_t e = ragged_allow(v, a.n_all, a.k_all, &smem, &fn);
   if (e != cudaSuccess) return e;
-  if (bps < 1) return cudaErrorInvalidConfiguration;
   a.n_max = a.n_all; a.k_max = a.k_all;
   a.tot_n = (long long)a.batch * a.n_all; a.tot_D = (long long)a.n_all * a.k_all; a.tot_k = (long long)a.batch * a.k_all;
   a.smem_floats = (int)(smem / 4);
