@@ -6,9 +6,9 @@
 
 namespace otlm {
 
-// b = bins per block (a multiple of 32), nb = blocks; nb = 0: the grid does not qualify (not sorted,
-// too coarse or too long) and rows are summed term by term.  q: centres are multiples of q (a power
-// of two at least 2^-18 of the largest |xt|), so that differences of centres are exact.
+// b = bins per block (a multiple of 8, at least 32), nb = blocks; nb = 0: the grid does not qualify (not
+// sorted, too coarse or too long) and runs elsewhere.  q: centres are multiples of q (a power of two at
+// least 2^-18 of the largest |xt|), so that differences of centres are exact.
 struct ExPlan {
   int b, nb;
   float q;
@@ -52,8 +52,9 @@ struct MMBArgs {
 
 // Launches (the first error of the launch): the block plan of a grid on the device, one apply over
 // the active problems (tc: the tensor-core handle's variant), the log ratios of a later MM step, and
-// the batched MM and source step.
-cudaError_t ex_plan(const float* xt, int n, ExPlan* plan, cudaStream_t stream);
+// the batched MM and source step.  with_plan, without (may be null): the numbers of active problems of
+// the expansion kernels and of the log-domain kernels, batch and 0 or 0 and batch by the plan.
+cudaError_t ex_plan(const float* xt, int n, ExPlan* plan, int batch, int* with_plan, int* without, cudaStream_t stream);
 cudaError_t ex_apply_source(const ExArgs& a, int batch, bool tc, int sms, cudaStream_t stream);
 cudaError_t ex_apply_target(const ExArgs& a, int batch, bool tc, int sms, cudaStream_t stream);
 cudaError_t ex_ratio(const ExArgs& a, int batch, cudaStream_t stream);

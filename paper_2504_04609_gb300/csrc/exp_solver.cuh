@@ -11,8 +11,8 @@
 // The row is staged in shared memory (n <= EXA_MAX_N).  Small batches split a problem's row blocks
 // over `parts` CTAs (grid.y), each forming the moments of its own row blocks from the whole row; the
 // last CTA of a problem to finish adds the violation's partial sums in a fixed order and decides.
-// A grid that does not qualify for expansions (ExPlan.nb = 0, known on the device only) is summed
-// term by term here too.
+// A grid without a plan (ExPlan.nb = 0) never gets here: the host chooses other kernels, or the device
+// counts no active problem for these.
 #pragma once
 
 #include "expansion.cuh"
@@ -24,75 +24,16 @@ inline size_t exa_smem_bytes(int n, int warps) {
   return 4 * ((size_t)(n + 3) / 4 * 4 + ex_scratch_floats(warps));
 }
 
-static __global__ void __launch_bounds__(1024) ex_plan_kernel(const float* xt, int n, ExPlan* plan) {
+static __global__ void __launch_bounds__(1024) ex_plan_kernel(const float* xt, int n, ExPlan* plan, int batch,
+                                                              int* with_plan, int* without) {
   const bool sorted = ex_sorted(xt, n);
   if (threadIdx.x < 32) {
     const ExPlan pl = ex_plan_warp(xt, n, sorted);
-    if (threadIdx.x == 0) *plan = pl;
-  }
-}
-
-// Rows [i0, i1) term by term, four rows per warp at a time, lanes over the columns.  Shift: the
-// previous sum `old` where there is one; rows whose sum leaves [2^-60, 2^60] are redone around their
-// largest term.  row(...) as in ex_apply, with the shift in place of the integer base.
-template <int T, class Load, class Row>
-__device__ __forceinline__ void ex_direct(const float* in_s, const float* xt, int n, int i0, int i1, const float* old,
-                                          Load load, Row row) {
-  using P = Prec<float>;
-  constexpr int Q = 4;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int r0 = i0 + warp * Q; r0 < i1; r0 += T * Q) {
-    float xi[Q], m[Q], sum[Q];
-    bool ok = old != nullptr;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const int i = min(r0 + q, i1 - 1);
-      xi[q] = xt[i];
-      m[q] = old ? old[i] : 0.f;
-      ok &= isfinite(m[q]);
+    if (threadIdx.x == 0) {
+      *plan = pl;
+      if (with_plan) *with_plan = pl.nb > 0 ? batch : 0;
+      if (without) *without = pl.nb > 0 ? 0 : batch;
     }
-    auto sweep = [&] {
-#pragma unroll
-      for (int q = 0; q < Q; ++q) sum[q] = 0.f;
-#pragma unroll 4
-      for (int j = lane; j < n; j += 32) {
-        const float v = in_s[j], xj = xt[j];
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-          const float d = xi[q] - xj;
-          sum[q] += P::exp2(fmaf(-d, d, v - m[q]));
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < Q; ++q)
-        for (int o = 16; o > 0; o >>= 1) sum[q] += __shfl_xor_sync(0xffffffffu, sum[q], o);
-    };
-    if (ok) {
-      sweep();
-#pragma unroll
-      for (int q = 0; q < Q; ++q) ok &= sum[q] >= 0x1p-60f && sum[q] <= 0x1p60f;
-    }
-    if (!ok) {  // the totals, and so this branch, are the same in every lane
-#pragma unroll
-      for (int q = 0; q < Q; ++q) m[q] = -CUDART_INF_F;
-      for (int j = lane; j < n; j += 32) {
-        const float v = in_s[j], xj = xt[j];
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-          const float d = xi[q] - xj;
-          m[q] = fmaxf(m[q], fmaf(-d, d, v));
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        for (int o = 16; o > 0; o >>= 1) m[q] = fmaxf(m[q], __shfl_xor_sync(0xffffffffu, m[q], o));
-        if (!(m[q] > -CUDART_INF_F)) m[q] = 0.f;  // every term vanishes
-      }
-      sweep();
-    }
-#pragma unroll
-    for (int q = 0; q < Q; ++q)
-      if (lane == q && r0 + q < i1) row(r0 + q, load(r0 + q), m[q], sum[q], 0.f);
   }
 }
 
@@ -149,17 +90,19 @@ __global__ void __launch_bounds__(32 * T, T == 4 ? EXA_MINB : 1) ex_apply_kernel
   const int p = A.active[slot], n = A.n, tid = threadIdx.x;
   if (A.done[p]) return;
   const size_t o = (size_t)p * n;
+  const float* yp = A.y + o;  // the problem's rows
+  float *sp = A.S + o, *lap = A.LA2 + o, *lbp = A.LB2 + o, *gp = A.G2 + o;
   float* in_s = smem;
   float* scr = smem + (n + 3) / 4 * 4;
   const ExPlan pl = *A.plan;
   float mass = 0.f;
   if (EPI == EXA_SOURCE) {
 #pragma unroll 8
-    for (int j = tid; j < n; j += NT) in_s[j] = A.G2[o + j];
+    for (int j = tid; j < n; j += NT) in_s[j] = gp[j];
   } else {
 #pragma unroll 8
     for (int j = tid; j < n; j += NT) {
-      const float s = A.S[o + j], la = A.LA2[o + j];
+      const float s = sp[j], la = lap[j];
       in_s[j] = s > 0.f ? P::log2(s) - la : P::ninf();
       mass += s;
     }
@@ -173,13 +116,12 @@ __global__ void __launch_bounds__(32 * T, T == 4 ? EXA_MINB : 1) ex_apply_kernel
   auto load = [&](int i) {
     Pre q{0.f, 0.f};
     if (EPI == EXA_SOURCE) {
-      if (A.check || TC) q.a = A.S[o + i];
-      if (A.check) q.b = A.LA2[o + i];
-    } else q.a = A.y[o + i];
+      if (A.check || TC) q.a = sp[i];
+      if (A.check) q.b = lap[i];
+    } else q.a = yp[i];
     return q;
   };
   auto row = [&](int i, Pre pre, float base, float sum, float di2) {
-    const size_t idx = o + i;
     const float v = sum > 0.f ? base + (P::log2(sum) - di2) : P::ninf();
     if (EPI == EXA_SOURCE) {
       const float s = pre.a;
@@ -191,7 +133,7 @@ __global__ void __launch_bounds__(32 * T, T == 4 ? EXA_MINB : 1) ex_apply_kernel
         else if (dl + P::log2(sum) > 64.f) part += P::exp2(fminf(P::log2(s) + (dl + P::log2(sum)), 120.f));
         else part += s * fabsf(sum * P::exp2(dl) - 1.f);
       }
-      A.LA2[idx] = v;
+      lap[i] = v;
       if (TC) {
         const float r = s > 0.f ? v - P::log2(s) : 0.f, hi = exa_tf32(r);
         const size_t ro = (size_t)slot * A.ld + i;
@@ -199,18 +141,15 @@ __global__ void __launch_bounds__(32 * T, T == 4 ? EXA_MINB : 1) ex_apply_kernel
         A.Rlo[ro] = exa_tf32(r - hi);
       }
     } else {
-      A.LB2[idx] = v;
-      A.G2[idx] = exa_datafit<TC>(A, v, pre.a);
+      lbp[i] = v;
+      gp[i] = exa_datafit<TC>(A, v, pre.a);
     }
   };
-  if (pl.nb > 0) {
+  if constexpr (T == 4) {  // one CTA per problem
+    ex_apply<T>(in_s, A.xt, n, pl, 0, pl.nb, scr, load, row);
+  } else {
     const int I0 = pl.nb * prt / parts, I1 = pl.nb * (prt + 1) / parts;
     if (I1 > I0) ex_apply<T>(in_s, A.xt, n, pl, I0, I1, scr, load, row);
-  } else {
-    ex_sync<T>();
-    const float* old = A.it > 0 ? (EPI == EXA_SOURCE ? A.LA2 : A.LB2) + o : nullptr;
-    const int i0 = (int)((long long)n * prt / parts), i1 = (int)((long long)n * (prt + 1) / parts);
-    ex_direct<T>(in_s, A.xt, n, i0, i1, old, load, row);
   }
   if (EPI == EXA_TARGET || !A.check) return;
 
@@ -278,8 +217,11 @@ inline int exa_parts(int batch, int n, int sms) {
 }
 
 template <int EPI, bool TC, int T>
-static inline cudaError_t launch_ex_cfg(const ExArgs& a, int batch, int parts, cudaStream_t stream) {
-  const size_t smem = exa_smem_bytes(a.n, T);
+static inline cudaError_t launch_ex_cfg(const ExArgs& a, int batch, int parts, int sms, cudaStream_t stream) {
+  size_t smem = exa_smem_bytes(a.n, T);
+  // CTAs that leave SMs idle get an SM each: more than half its shared memory (one target at n = 16384, 20
+  // iterations: 2.33 ms where two may share an SM, 2.22 with one; four: 2.38, 2.21)
+  if (parts > 1 && (long long)batch * parts <= sms && smem < 116 * 1024) smem = 116 * 1024;
   if (smem > 48 * 1024) {  // the largest size for every call: the limit is the process's, threads would lower it
     const cudaError_t e = cudaFuncSetAttribute(ex_apply_kernel<EPI, TC, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)exa_smem_bytes(EXA_MAX_N, T));
@@ -294,8 +236,8 @@ static inline cudaError_t launch_ex_cfg(const ExArgs& a, int batch, int parts, c
 #endif
 template <int EPI, bool TC>
 static inline cudaError_t launch_ex_apply(const ExArgs& a, int batch, int sms, cudaStream_t stream) {
-  if (batch >= 4 * sms && a.n <= 8192) return launch_ex_cfg<EPI, TC, EXA_T1>(a, batch, 1, stream);
-  return launch_ex_cfg<EPI, TC, 8>(a, batch, exa_parts(batch, a.n, sms), stream);
+  if (batch >= 4 * sms && a.n <= 8192) return launch_ex_cfg<EPI, TC, EXA_T1>(a, batch, 1, sms, stream);
+  return launch_ex_cfg<EPI, TC, 8>(a, batch, exa_parts(batch, a.n, sms), sms, stream);
 }
 
 // ---- MM step and source step of a batch sharing the dictionary (FP32) ---------------------------

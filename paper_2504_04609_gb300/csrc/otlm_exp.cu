@@ -3,8 +3,8 @@
 
 namespace otlm {
 
-cudaError_t ex_plan(const float* xt, int n, ExPlan* plan, cudaStream_t stream) {
-  ex_plan_kernel<<<1, 1024, 0, stream>>>(xt, n, plan);
+cudaError_t ex_plan(const float* xt, int n, ExPlan* plan, int batch, int* with_plan, int* without, cudaStream_t stream) {
+  ex_plan_kernel<<<1, 1024, 0, stream>>>(xt, n, plan, batch, with_plan, without);
   return cudaGetLastError();
 }
 cudaError_t ex_apply_source(const ExArgs& a, int batch, bool tc, int sms, cudaStream_t stream) {

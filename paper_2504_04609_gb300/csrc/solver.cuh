@@ -295,6 +295,8 @@ void objective_eval(const Launch& L, const Workspace<T>& ws, const ObjWorkspace<
 // after the active count, a small batch's partial violations in F2 (the expansion path forms F2 on
 // the fly) and the per-problem CTA counts in err_acc (zeroed by prep_kernel, left at zero).
 inline ExPlan* ex_plan_of(const Workspace<float>& ws) { return reinterpret_cast<ExPlan*>(ws.n_active + 4); }
+// The expansion kernels' own number of active problems, where the device chooses the kernels by the plan.
+inline int* ex_count_of(const Workspace<float>& ws) { return ws.n_active + 8; }
 inline ExArgs ex_args(const Workspace<float>& ws, const SolveParams& sp, const float* y) {
   const double eps_ln2 = sp.eps * kLn2;
   ExArgs a{};
@@ -315,19 +317,24 @@ inline bool ex_serves(const SolveParams& sp, bool dense, bool checks) {
 }
 
 // The number of blocks of a grid's plan on the host (0: the grid does not qualify), read while the
-// kernels queued in between run. A stream under capture cannot be read: `known` stays false and the
-// kernels follow the plan on the device.
+// kernels queued in between run. A solve that makes no convergence poll must not wait for the stream, and a
+// stream under capture cannot be read: `known` stays false, and the two counts of active problems, the
+// expansion kernels' and the log-domain kernels', follow the plan on the device.
 struct ExPlanRead {
   cudaEvent_t ev = nullptr;
   bool known = false;
   int nb = 0;
-  cudaError_t begin(const Launch& L, const Workspace<float>& ws, int n) {
-    L.begin(KIND_OTHER);
-    cudaError_t e = ex_plan(ws.xt, n, ex_plan_of(ws), L.stream);
-    L.end();
+  cudaError_t begin(const Launch& L, const Workspace<float>& ws, int batch, int n, bool wait, bool on_device) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (e == cudaSuccess) e = cudaStreamIsCapturing(L.stream, &cap);
-    if (e != cudaSuccess || !L.host_flag || cap != cudaStreamCaptureStatusNone) return e;
+    cudaError_t e = cudaStreamIsCapturing(L.stream, &cap);
+    if (e != cudaSuccess) return e;
+    wait = wait && L.host_flag && cap == cudaStreamCaptureStatusNone;
+    L.begin(KIND_OTHER);
+    on_device = on_device && !wait;
+    e = ex_plan(ws.xt, n, ex_plan_of(ws), batch, on_device ? ex_count_of(ws) : nullptr, on_device ? ws.n_active : nullptr,
+                L.stream);
+    L.end();
+    if (e != cudaSuccess || !wait) return e;
     e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(L.host_flag, &ex_plan_of(ws)->nb, sizeof(int), cudaMemcpyDeviceToHost, L.stream);
@@ -347,13 +354,14 @@ struct ExPlanRead {
 };
 
 // The iteration loop of solve_device with expansion applies (three launches beside the compaction);
-// the plan is on the device.
+// the plan is on the device, and so is the number of active problems.
 inline cudaError_t ex_iterate(const Launch& L, const Workspace<float>& ws, const SolveParams& sp, const float* D,
-                              const float* y) {
+                              const float* y, int* n_active) {
   const int batch = sp.batch, sms = sm_count();
   cudaError_t e = cudaSuccess;
   ExArgs a = ex_args(ws, sp, y);
-  MMBArgs mm{ws.active, ws.n_active, sp.n, sp.k, D, ws.Dt, ws.xcol, ws.LA2, ws.S, ws.W, ws.mass, ws.dw, ws.done,
+  a.n_active = n_active;
+  MMBArgs mm{ws.active, n_active, sp.n, sp.k, D, ws.Dt, ws.xcol, ws.LA2, ws.S, ws.W, ws.mass, ws.dw, ws.done,
              sp.penalty, sp.mm_steps, float(sp.eps), float(sp.alpha), float(sp.beta)};
   for (int it = 0;; ++it) {
     a.it = it;
@@ -370,7 +378,7 @@ inline cudaError_t ex_iterate(const Launch& L, const Workspace<float>& ws, const
     const bool poll = (it + 1) % sp.poll_every == 0;
     if (poll && it > 0) {  // finished problems are skipped by their flag in between
       L.begin(KIND_COMPACT);
-      (void)launch_pdl(true, compact_kernel, dim3(1), dim3(1024), 0, L.stream, ws.active, ws.n_active, ws.done);
+      (void)launch_pdl(true, compact_kernel, dim3(1), dim3(1024), 0, L.stream, ws.active, n_active, ws.done);
       L.end();
     }
     L.begin(KIND_APPLY);
@@ -378,7 +386,7 @@ inline cudaError_t ex_iterate(const Launch& L, const Workspace<float>& ws, const
     L.end();
     if (e != cudaSuccess) return e;
     if (poll) {
-      e = cudaMemcpyAsync(L.host_flag, ws.n_active, sizeof(int), cudaMemcpyDeviceToHost, L.stream);
+      e = cudaMemcpyAsync(L.host_flag, n_active, sizeof(int), cudaMemcpyDeviceToHost, L.stream);
       if (e == cudaSuccess) e = cudaStreamSynchronize(L.stream);
       if (e == cudaSuccess && L.timer && L.timer->on) e = L.timer->harvest();
       if (e != cudaSuccess) return e;
@@ -441,7 +449,7 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
   ExPlanRead plan;
   if constexpr (sizeof(T) == 4) {
     if (serves) {
-      const cudaError_t e = plan.begin(L, ws, n);
+      const cudaError_t e = plan.begin(L, ws, batch, n, sp.poll_every <= sp.max_iter, true);
       if (e != cudaSuccess) return e;
     }
   }
@@ -481,19 +489,19 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
   mm.dw = ws.dw; mm.dw_tol = T(sp.dw_tol); mm.gap_on = checks && sp.gap_tol > 0;
   mm.gap_ok = checks ? ow->gap_ok : nullptr;
 
-  bool by_expansion = false;
+  bool tiles = true;  // the tiled log-domain applies
   if constexpr (sizeof(T) == 4) {
     // a grid without a plan keeps the tiled log-domain applies (1024 x 1024, 20 iterations: 8.9 ms, rows summed
-    // one by one 17.8)
+    // one by one 17.8). Where the host does not know, both loops are queued and one finds no active problem:
+    // 3 us a launch (20 iterations of 1024 x 1024 with a plan 1.75 -> 1.96 ms, without 8.80 -> 8.85; 4 x 3000,
+    // whose one launch needs the plan: 1.16 -> 1.64 and 9.85 -> 9.99)
     if (serves) {
-      const cudaError_t e = plan.end(L);
+      cudaError_t e = plan.end(L);
+      if (e == cudaSuccess && plan.known && plan.nb > 0 && prefers) return small();
+      if (e == cudaSuccess && (!plan.known || plan.nb > 0))
+        e = ex_iterate(L, ws, sp, D, y, plan.known ? ws.n_active : ex_count_of(ws));
       if (e != cudaSuccess) return e;
-    }
-    by_expansion = serves && (!plan.known || plan.nb > 0);
-    if (by_expansion && prefers) return small();
-    if (by_expansion) {
-      const cudaError_t e = ex_iterate(L, ws, sp, D, y);
-      if (e != cudaSuccess) return e;
+      tiles = !plan.known || plan.nb == 0;
     }
   }
   bool linear = false;
@@ -541,7 +549,7 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
       }
     }
   }
-  for (int it = 0; !by_expansion && !linear; ++it) {
+  for (int it = 0; tiles && !linear; ++it) {
     src.check = it > 0;
     launch_apply<T, EPI_SOURCE>(L, src, it == 0, batch, n, sp.cost);
     // a check: the state (w, g) whose a = K u1 was just computed is the one this iteration returns

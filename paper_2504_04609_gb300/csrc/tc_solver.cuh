@@ -848,7 +848,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
   ExPlanRead plan;
   const bool by_plan = serves && (small || tc_prefers_expansion(batch, n, 0));
   if (by_plan) {
-    const cudaError_t e = plan.begin(L, ws, n);
+    const cudaError_t e = plan.begin(L, ws, batch, n, true, false);  // (such solves end in a wait)
     if (e != cudaSuccess) return e;
   }
   L.begin(KIND_OTHER);
