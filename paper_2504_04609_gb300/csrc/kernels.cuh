@@ -492,10 +492,6 @@ struct MMArgs {
   int gap_on;       // gap_tol > 0: the gap is a stopping criterion
   int penalty;
   int mm_steps = 1;  // MM steps with the same LA2 (a = K u1)
-  // f64_mm_kernel: the first step's log ratios, 1 / a, and u2 = S / a out
-  const T* R = nullptr;
-  const T* IA = nullptr;
-  T* U2 = nullptr;
   T eps, alpha, beta;
 };
 

@@ -516,16 +516,16 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
       f64_scale_kernel<<<1184, 256, 0, L.stream>>>(ws.G2, f64.U1, y, f64.LY, (size_t)batch * n);
       L.end();
       src.G2 = ws.G2;
-      mm.R = ws.F2; mm.IA = f64.IA; mm.U2 = f64.U2;
+      MMArgsF64 fm{mm, ws.F2, f64.IA, f64.U2};
       for (int it = 0;; ++it) {
         src.check = it > 0;
         L.begin(KIND_APPLY);
         cudaError_t e = launch_f64_apply<EPI_SOURCE>(src, f64, ws.LA2, ws.F2, ws.done, batch, abs_cost, 1, sm_count(), L.stream);
         L.end();
         if (e != cudaSuccess) return e;
-        mm.it = it;
+        fm.it = it;
         L.begin(KIND_MM);
-        e = launch_f64_mm(mm, batch, L.stream);
+        e = launch_f64_mm(fm, batch, L.stream);
         L.end();
         if (e != cudaSuccess) return e;
         if (it >= sp.max_iter) break;
