@@ -23,6 +23,7 @@ struct ExArgs {
   const ExPlan* plan;
   const float* xt;
   int n, k, it, max_iter, check, datafit;
+  int early;                // launch applies that split a problem over CTAs early, too
   const float* y;
   float *G2, *LA2, *LB2, *S, *mass;
   // stopping decision

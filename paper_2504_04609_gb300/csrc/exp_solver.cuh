@@ -229,7 +229,7 @@ static inline cudaError_t launch_ex_cfg(const ExArgs& a, int batch, int parts, i
   }
   // CTAs that leave SMs idle are launched late: early ones share SMs beside a running GEMM (one target at
   // n = 16384, 20 iterations: 2.43 ms early, 2.23 late)
-  return launch_pdl(parts == 1, ex_apply_kernel<EPI, TC, T>, dim3(batch, parts), dim3(32 * T), smem, stream, a);
+  return launch_pdl(parts == 1 || a.early, ex_apply_kernel<EPI, TC, T>, dim3(batch, parts), dim3(32 * T), smem, stream, a);
 }
 #ifndef EXA_T1
 #define EXA_T1 4

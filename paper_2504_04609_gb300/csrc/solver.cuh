@@ -361,6 +361,7 @@ inline cudaError_t ex_iterate(const Launch& L, const Workspace<float>& ws, const
   cudaError_t e = cudaSuccess;
   ExArgs a = ex_args(ws, sp, y);
   a.n_active = n_active;
+  a.early = n_active != ws.n_active;  // launches that may find no problem: 0.9 us each, 2.2 in turn
   MMBArgs mm{ws.active, n_active, sp.n, sp.k, D, ws.Dt, ws.xcol, ws.LA2, ws.S, ws.W, ws.mass, ws.dw, ws.done,
              sp.penalty, sp.mm_steps, float(sp.eps), float(sp.alpha), float(sp.beta)};
   for (int it = 0;; ++it) {
@@ -493,8 +494,8 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
   if constexpr (sizeof(T) == 4) {
     // a grid without a plan keeps the tiled log-domain applies (1024 x 1024, 20 iterations: 8.9 ms, rows summed
     // one by one 17.8). Where the host does not know, both loops are queued and one finds no active problem:
-    // 3 us a launch (20 iterations of 1024 x 1024 with a plan 1.75 -> 1.96 ms, without 8.80 -> 8.85; 4 x 3000,
-    // whose one launch needs the plan: 1.16 -> 1.64 and 9.85 -> 9.99)
+    // one to three us a launch (20 iterations of 1024 x 1024 with a plan 1.75 -> 1.99 ms, without 8.82 -> 8.89;
+    // 4 x 3000, whose one launch needs the plan: 1.16 -> 1.58 and 9.72 -> 9.72)
     if (serves) {
       cudaError_t e = plan.end(L);
       if (e == cudaSuccess && plan.known && plan.nb > 0 && prefers) return small();
