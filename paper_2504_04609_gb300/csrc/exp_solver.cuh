@@ -146,10 +146,10 @@ __global__ void __launch_bounds__(32 * T, T == 4 ? EXA_MINB : 1) ex_apply_kernel
     }
   };
   if constexpr (T == 4) {  // one CTA per problem
-    ex_apply<T>(in_s, A.xt, n, pl, 0, pl.nb, scr, load, row);
+    ex_apply<T>(in_s, A.xt, n, pl, 0, pl.nb, scr, T, load, row);
   } else {
     const int I0 = pl.nb * prt / parts, I1 = pl.nb * (prt + 1) / parts;
-    if (I1 > I0) ex_apply<T>(in_s, A.xt, n, pl, I0, I1, scr, load, row);
+    if (I1 > I0) ex_apply<T>(in_s, A.xt, n, pl, I0, I1, scr, T, load, row);
   }
   if (EPI == EXA_TARGET || !A.check) return;
 

@@ -44,6 +44,10 @@ constexpr int EX_HEAD = 4 * EX_NB;
 __host__ __device__ constexpr int ex_scratch_floats(int warps) {
   return EX_HEAD + EX_M * EX_NB * (4 * warps < EX_NB ? 4 * warps : EX_NB);
 }
+// Groups of (up to) four row blocks a round may take with `floats` of scratch.
+__device__ __forceinline__ int ex_round_groups(int warps, int nb, int floats) {
+  return min(warps, (floats - EX_HEAD) / (EX_M * 4 * nb));
+}
 
 __device__ __forceinline__ float ex_quantum(float x0, float x1) {
   const int e = (__float_as_int(fmaxf(fabsf(x0), fabsf(x1))) >> 23) & 255;
@@ -199,8 +203,8 @@ __device__ __forceinline__ void ex_rows(const float* xt, int i0, int i1, float c
 }
 
 // The apply for row blocks [I0, I1) by the T warps of a CTA: in_s [n] in shared memory (written
-// before the call; the first barrier is here), xt [n] (shared or global), scr = shared scratch of
-// ex_scratch_floats(T) floats, 16-byte aligned.  row(i, pre, base, sum, di2) is called once per row by
+// before the call; the first barrier is here), xt [n] (shared or global), scr = shared scratch, 16-byte
+// aligned, of ex_scratch_floats(T) floats for gr = T or less for gr = ex_round_groups(T, ...).  row(i, pre, base, sum, di2) is called once per row by
 // one thread, with out_i = base + (log2(sum) - di2), base an integer and sum = 0 for an empty (or
 // non-finite) input; pre = load(i) was called before the row's sums, so that what the row's epilogue
 // reads arrives meanwhile.
@@ -214,7 +218,7 @@ __device__ __forceinline__ void ex_sync() {
 }
 template <int T, class Load, class Row>
 __device__ __forceinline__ void ex_apply(const float* in_s, const float* xt, int n, const ExPlan& pl, int I0, int I1,
-                                         float* scr, Load load, Row row) {
+                                         float* scr, int gr, Load load, Row row) {
   using P = Prec<float>;
   // coefficients of the polynomial for 2^(2 t) = e^(2 ln2 t), |2 ln2 t| <= 0.75: (2 ln2)^m a_m with
   // a_m the degree-7 polynomial of smallest relative error for e^t on [-0.75, 0.75] (Remez exchange)
@@ -261,12 +265,12 @@ __device__ __forceinline__ void ex_apply(const float* in_s, const float* xt, int
     if (lane == 0) mask_s[I] = mk;
   }
   ex_sync<T>();
-  // row blocks go in groups of three or four (equal shares), a round takes up to T groups
+  // row blocks go in groups of three or four (equal shares), a round takes up to gr <= T groups
   const int ng = (I1 - I0 + 3) / 4, cpb = (b + 127) / 128, per = ((b + 31) / 32 + cpb - 1) / cpb;
   const bool narrow = b < 256;  // 8 lanes per column block (four at a time) for short blocks
   const int nr = narrow ? (nb + 3) / 4 : nb;
-  for (int g0 = 0; g0 < ng; g0 += T) {
-    const int gn = min(T, ng - g0);
+  for (int g0 = 0; g0 < ng; g0 += gr) {
+    const int gn = min(gr, ng - g0);
     const int Ia = I0 + (I1 - I0) * g0 / ng, Ib = I0 + (I1 - I0) * (g0 + gn) / ng;
     // moments: items of one group and one (or four) column blocks
     for (int t = warp; t < gn * nr; t += T) {

@@ -64,15 +64,17 @@ struct RaggedArgs {
 constexpr int RAGGED_BUCKETS = 16;
 __host__ __device__ inline int ragged_bucket(int n) { return n <= 256 ? 0 : (n - 1) / 256 < 15 ? (n - 1) / 256 : 15; }
 
+// Dynamic shared memory (floats) of a problem of n_max bins, k_max atoms: its state, then a part that the
+// warps' sums of D^T r and the expansion's scratch take in turn. `full` is the scratch of one round; the
+// least one serves in rounds of two groups and more (up to 16 blocks still one round of 8 warps), so that
+// what the scratch adds does not cost a CTA its place on the SM (ragged_prepare).
 template <int NT>
 struct RaggedSmem {
-  // offsets (floats) into dynamic shared memory for a problem of n_max bins, k_max atoms
-  static __host__ __device__ size_t floats(int n_max, int k_max) {
-    return state(n_max, k_max) + ex_scratch_floats(NT / 32);
-  }
-  // everything but the expansion's scratch, rounded up to 16 bytes
-  static __host__ __device__ size_t state(int n_max, int k_max) {
-    return (6 * (size_t)n_max + 3 * (size_t)k_max + (NT / 32) * (size_t)k_max + 64 + 3) / 4 * 4;
+  static constexpr int LEAST = EX_HEAD + EX_M * EX_NB * 8;
+  static __host__ __device__ size_t state(int n_max, int k_max) { return (6 * (size_t)n_max + 3 * (size_t)k_max + 64 + 3) / 4 * 4; }
+  static __host__ __device__ size_t floats(int n_max, int k_max, bool full) {
+    const size_t sums = (NT / 32) * (size_t)k_max, scr = full ? ex_scratch_floats(NT / 32) : LEAST;
+    return state(n_max, k_max) + (sums > scr ? sums : scr);
   }
 };
 
@@ -198,9 +200,9 @@ __device__ __forceinline__ float block_sum_f(float v, float* red) { return block
 // serves the source and target applies of every rows-per-thread variant.
 template <int NT>
 __device__ __noinline__ void ragged_apply_ex(const float* xt, const float* in, float* out, int n, ExPlan pl, float* scr,
-                                             float* ratio) {
+                                             int gr, float* ratio) {
   using P = Prec<float>;
-  ex_apply<NT / 32>(in, xt, n, pl, 0, pl.nb, scr, [](int) { return 0; }, [&](int i, int, float base, float sum, float di2) {
+  ex_apply<NT / 32>(in, xt, n, pl, 0, pl.nb, scr, gr, [](int) { return 0; }, [&](int i, int, float base, float sum, float di2) {
     if (ratio) ratio[i] = sum > 0.f ? sum * P::exp2((base - out[i]) - di2) : 0.f;
     out[i] = sum > 0.f ? base + (P::log2(sum) - di2) : P::ninf();
   });
@@ -328,7 +330,7 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
   const bool valid = n >= 2 && n <= A.n_max && k >= 1 && k <= A.k_max && (n + NT - 1) / NT <= R && on >= 0 &&
                      on + n <= A.tot_n && oD >= 0 && oD + (long long)n * k <= A.tot_D && ok >= 0 &&
                      ok + k <= A.tot_k &&
-                     (long long)RaggedSmem<NT>::floats(A.n_max, A.k_max) <= A.smem_floats;
+                     (long long)RaggedSmem<NT>::floats(A.n_max, A.k_max, false) <= A.smem_floats;
   if (!__syncthreads_and(valid)) {
     if (threadIdx.x == 0) {
       A.iters[p] = 0;
@@ -347,9 +349,9 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
   float* W = S + A.n_max;
   float* xcol = W + A.k_max;
   float* Wp = xcol + A.k_max;     // weights before the last update
-  float* red_k = Wp + A.k_max;    // [NT/32][k_max]
-  float* red = red_k + (NT / 32) * A.k_max;  // 32 floats + scalars
+  float* red = Wp + A.k_max;      // 32 floats + scalars
   float* scr = sm + RaggedSmem<NT>::state(A.n_max, A.k_max);  // the expansion's scratch
+  float* red_k = scr;             // [NT/32][k_max], between the applies
   __shared__ ExPlan plan_s;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int NW = NT / 32;
@@ -370,6 +372,7 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
   for (int i = tid; i < n; i += NT) F2[i] = 1.f;
   __syncthreads();
   const ExPlan plan = plan_s;
+  const int gr = plan.nb ? ex_round_groups(NW, plan.nb, A.smem_floats - (int)(scr - sm)) : 1;
   ragged_dtr_any<NT>(D, F2, n, k, A.k_max, red_k);
   __syncthreads();
   for (int j = tid; j < k; j += NT) {
@@ -392,7 +395,7 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
   int st = ST_MAX_ITER;
   for (;; ++it) {
     // source apply; F2 doubles as the ratio buffer a_new / a_old
-    if (plan.nb) ragged_apply_ex<NT>(xt, G2, LA2, n, plan, scr, it > 0 ? F2 : nullptr);
+    if (plan.nb) ragged_apply_ex<NT>(xt, G2, LA2, n, plan, scr, gr, it > 0 ? F2 : nullptr);
     else ragged_apply<NT, R>(xt, G2, LA2, n, it > 0, F2);
     if (it > 0) {
       float part = 0.f;
@@ -434,7 +437,7 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
       if (m + 1 == A.mm_steps) mass = m_mass;
     }
     // target apply and the datafit step (Table 1) in log2 units
-    if (plan.nb) ragged_apply_ex<NT>(xt, F2, LB2, n, plan, scr, nullptr);
+    if (plan.nb) ragged_apply_ex<NT>(xt, F2, LB2, n, plan, scr, gr, nullptr);
     else ragged_apply<NT, R>(xt, F2, LB2, n, it > 0, nullptr);
     const float kl_coef = A.lam / (eps + A.lam), tv_bound = A.lam / eps_ln2, loe = A.lam / eps;
     const float lloe = logf(A.lam / eps);
@@ -538,23 +541,36 @@ inline int ragged_rmax_log2(int v) { return v == 0 ? 5 : (v == 1 ? 4 : 3); }
 // that followed the call would be lowered by one host thread between another's setting and launch.
 constexpr int RAGGED_N_MAX = 4096, RAGGED_K_MAX = 256;
 template <int NT, int RMAX>
-inline cudaError_t ragged_allow(int n_max, int k_max, size_t* smem, const void** fn) {
+inline cudaError_t ragged_allow(int n_max, int k_max, bool full, size_t* smem, const void** fn) {
   static_assert(RAGGED_N_MAX <= NT * RMAX, "rows per thread cover the largest problem");
-  *smem = RaggedSmem<NT>::floats(n_max, k_max) * 4;
+  *smem = RaggedSmem<NT>::floats(n_max, k_max, full) * 4;
   *fn = (const void*)ragged_kernel<NT, RMAX>;
   return cudaFuncSetAttribute(*fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(RaggedSmem<NT>::floats(RAGGED_N_MAX, RAGGED_K_MAX) * 4));
+                              (int)(RaggedSmem<NT>::floats(RAGGED_N_MAX, RAGGED_K_MAX, true) * 4));
 }
-inline cudaError_t ragged_allow(int v, int n_max, int k_max, size_t* smem, const void** fn) {
+inline cudaError_t ragged_allow(int v, int n_max, int k_max, bool full, size_t* smem, const void** fn) {
   if (n_max > RAGGED_N_MAX || k_max > RAGGED_K_MAX) return cudaErrorInvalidValue;
-  if (v == 0) return ragged_allow<128, 32>(n_max, k_max, smem, fn);
-  if (v == 1) return ragged_allow<256, 16>(n_max, k_max, smem, fn);
-  return ragged_allow<512, 8>(n_max, k_max, smem, fn);
+  if (v == 0) return ragged_allow<128, 32>(n_max, k_max, full, smem, fn);
+  if (v == 1) return ragged_allow<256, 16>(n_max, k_max, full, smem, fn);
+  return ragged_allow<512, 8>(n_max, k_max, full, smem, fn);
 }
+// The full scratch unless the least one lets more CTAs share an SM.  456 unsorted problems of 3300 to 4096
+// bins, k = 128, 6 iterations, 256 threads: one CTA per SM 24.0 ms, two 19.4; sorted ones 4.32 and 3.28.
 inline cudaError_t ragged_prepare(int v, int n_max, int k_max, int* blocks_per_sm, size_t* smem) {
-  const void* fn = nullptr;
-  const cudaError_t e = ragged_allow(v, n_max, k_max, smem, &fn);
-  return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, ragged_nt(v), *smem);
+  *blocks_per_sm = 0;
+  for (const bool full : {true, false}) {
+    size_t bytes = 0;
+    const void* fn = nullptr;
+    int blocks = 0;
+    cudaError_t e = ragged_allow(v, n_max, k_max, full, &bytes, &fn);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fn, ragged_nt(v), bytes);
+    if (e != cudaSuccess) return e;
+    if (blocks > *blocks_per_sm) {
+      *blocks_per_sm = blocks;
+      *smem = bytes;
+    }
+  }
+  return cudaSuccess;
 }
 
 // A small batch sharing grid, dictionary and eps, whole solves in one launch (one CTA per problem).
@@ -565,7 +581,7 @@ inline cudaError_t ragged_small(const RaggedArgs& a0, cudaStream_t s) {
   const int v = a.n_all <= 512 ? 1 : 2;
   size_t smem = 0;
   const void* fn = nullptr;
-  const cudaError_t e = ragged_allow(v, a.n_all, a.k_all, &smem, &fn);
+  const cudaError_t e = ragged_allow(v, a.n_all, a.k_all, true, &smem, &fn);
   if (e != cudaSuccess) return e;
   a.n_max = a.n_all; a.k_max = a.k_all;
   a.tot_n = (long long)a.batch * a.n_all; a.tot_D = (long long)a.n_all * a.k_all; a.tot_k = (long long)a.batch * a.k_all;
