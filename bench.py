@@ -430,13 +430,27 @@ def tc_apply_roofline(workload, n, iters, apply_timing, peaks, iters_hilo=None, 
     return r
 
 
-# Tensor-core handles run grid solves without the precision schedule as block expansions where their
-# GEMMs do not fill the SM pairs.
-EXPANSION_BATCH, EXPANSION_BINS = 64, 5 << 18
+# What a solve ran, by the route its handle reports: compute type, path and kernel of the applies.
+ROUTE_LABELS = {
+    "expansion": ("f32", "FP32 block expansions", "ex_apply_kernel (FP32 block expansions)"),
+    "one launch": ("f32", "whole solves in one launch (FP32 block expansions where the grid has a block plan)",
+                   "ragged_kernel (one problem per CTA, the whole solve)"),
+    "log": ("f32", "FP32 log-domain applies", "apply_kernel (FP32, one exp2 per kernel entry)"),
+    "tensor": ("bf16x3 tensor (hi/lo split) + f32", "tensor-core applies (tcgen05, BF16 hi/lo, FP32 accumulate)", None),
+}
 
 
-def tc_runs_expansions(batch, n, single_until):
-    return single_until == 0.0 and (batch <= EXPANSION_BATCH or batch * n <= EXPANSION_BINS)
+def simt_roofline(route, terms, bins, timing, peaks):
+    """Roofline of a solve whose applies are not GEMMs: the exponent unit for the plain sums (one exp2 per
+    kernel entry), the state's bytes for block expansions."""
+    kernel = ROUTE_LABELS[route][2]
+    if route != "log":
+        return expansion_apply_roofline(terms, bins, timing, peaks, kernel)
+    ms, cnt = timing
+    peak, achieved = SMS * EX2_PER_SM_CLK * MAX_SM_MHZ * 1e6 / 1e9, terms / (ms / 1e3) / 1e9
+    return {"bound": "exp2", "kernel": kernel, "achieved": achieved, "peak": peak, "unit": "Gexp2/s", "frac": achieved / peak,
+            "traffic": None, "launch_ms_avg": ms / max(cnt, 1),
+            "peak_basis": "%d SMs x %g ex2/clk x %.0f MHz (derived)" % (SMS, EX2_PER_SM_CLK, MAX_SM_MHZ)}
 
 
 def expansion_apply_roofline(terms, bins, apply_timing, peaks, kernel):
@@ -513,7 +527,7 @@ def run_ours(args, rank, world, local_rank, pool=None):
         timing = h.get_timing()
         h.set_timing(False)
         return dict(ms=e0.elapsed_time(e1), launches=launches, timing=timing, iters=iters.cpu().numpy(),
-                    status=status.cpu().numpy(), clocks=clk.summary(), handle=h, w=w, t=t)
+                    status=status.cpu().numpy(), clocks=clk.summary(), handle=h, w=w, t=t, route=h.route)
 
     sched = SINGLE_UNTIL.get(args.workload, 0.0)
     tc = measure("bf16tc", args.steps, args.warmup, sched)
@@ -560,23 +574,23 @@ def run_ours(args, rank, world, local_rank, pool=None):
 
     it_tc = tc["iters"].astype(np.float64)
     applies = float(np.sum(2 * it_tc + 1))
-    expansions = tc_runs_expansions(B, n, sched)
-    if expansions:
-        roofline = expansion_apply_roofline(applies * n * n, applies * n, tc["timing"]["apply"], peaks,
-                                            "ex_apply_kernel (FP32 block expansions)")
+    dtype, path, _ = ROUTE_LABELS[tc["route"]]
+    if tc["route"] != "tensor":
+        roofline = simt_roofline(tc["route"], applies * n * n, applies * n, tc["timing"]["apply"], peaks)
     else:
+        dtype += ", bf16x1 until a violation <= %g" % sched if sched else ""
         roofline = tc_apply_roofline(args.workload, n, tc["iters"], tc["timing"]["apply"], peaks,
                                      tc3["iters"] if tc3 is not None else None,
                                      tc3["timing"]["apply"] if tc3 is not None else None)
 
-    # plain FP32 path: block expansions of the log-domain sums
+    # plain FP32 path
     it_fp = fp["iters"].astype(np.float64)
     fp_applies = float(np.sum(2 * it_fp + 1))
     plain = {"value": fp_value, "unit": "problems/s", "ms_per_step": fp_ms / fp_steps, "steps": fp_steps,
              "mean_iters": float(it_fp.mean()), "converged": int(np.sum(fp["status"] == 0)),
              "kernel_ms_per_step": {kk: v[0] for kk, v in fp["timing"].items()},
-             "roofline": expansion_apply_roofline(fp_applies * n * n, fp_applies * n, fp["timing"]["apply"], peaks,
-                                                  "ex_apply_kernel (FP32 block expansions)"),
+             "path": ROUTE_LABELS[fp["route"]][1],
+             "roofline": simt_roofline(fp["route"], fp_applies * n * n, fp_applies * n, fp["timing"]["apply"], peaks),
              "clocks": fp["clocks"]}
     out = {
         "metric": workload_metric(args.workload),
@@ -589,12 +603,11 @@ def run_ours(args, rank, world, local_rank, pool=None):
         "higher_is_better": True,
         "scaling": "weak",
         "vs_baseline": None,
-        "dtype": "f32" if expansions else "bf16x3 tensor (hi/lo split) + f32" + (", bf16x1 until a violation <= %g" % sched if sched else ""),
+        "dtype": dtype,
         "data": "synthetic (seeded Gaussian-peak spectra, no dataset)",
         "config": {"workload": args.workload, "B_per_gpu": B, "n": n, "k": k, "eps": c["eps"],
                    "datafit": c["datafit"], "lam": c["lam"], "penalty": c["penalty"], "alpha": c["alpha"],
-                   "tol": c["tol"], "path": ("FP32 block expansions (GEMMs would not fill the SM pairs)" if expansions else
-                                             "tensor-core applies (tcgen05, BF16 hi/lo, FP32 accumulate)"),
+                   "tol": c["tol"], "path": path,
                    "bf16_single_until": sched,
                    "parallelism": f"replicas x{world}",
                    "l2": "inputs larger than L2 (4096 x 4096 FP32 state arrays, 64 MiB each, several per step)",
@@ -645,7 +658,7 @@ def run_ours(args, rank, world, local_rank, pool=None):
         pick = np.unique(np.linspace(0, B - 1, 16).astype(np.int64))
         out["err_vs_fp64"] = oracle_errors(pool, args.workload, pick, it_tc[pick], tc["w"][pick].cpu().numpy(),
                                            tc["t"][pick].cpu().numpy())
-        out["err_vs_fp64"]["path"] = "tensor-core (BF16 hi/lo applies, TF32 hi/lo contractions)"
+        out["err_vs_fp64"]["path"] = path
         nb = min(B, 64)
         out["cpu_baseline"] = cpu_baseline(args.workload, range(nb), 1, it_tc[:nb], pool=pool,
                                            one_core=16 if n >= 4096 else nb)
@@ -982,6 +995,7 @@ def run_single_hbm(args, rank, world, local_rank):
     torch.cuda.synchronize()
     timing = h.get_timing()
     h.set_timing(False)
+    route = h.route
     it = int(iters.cpu().numpy()[0])
     st = int(status.cpu().numpy()[0])
 
@@ -1014,10 +1028,9 @@ def run_single_hbm(args, rank, world, local_rank):
         "data": "synthetic (seeded Gaussian-peak spectra, no dataset)",
         "config": {"workload": args.workload, "B_per_gpu": B, "n": n, "k": k, "eps": c["eps"], "datafit": c["datafit"],
                    "penalty": c["penalty"], "tol": c["tol"], "iters": it, "status": st,
-                   "path": "FP32 block expansions (small batch; no kernel matrix is stored)",
+                   "path": ROUTE_LABELS[route][1],
                    "l2": "the state and the dictionary (9 MB) stay in L2", "parallelism": f"replicas x{world}"},
-        "roofline": expansion_apply_roofline((2.0 * it + 1) * n * n, (2.0 * it + 1) * n, timing["apply"], _peaks(),
-                                             "ex_apply_kernel (FP32 block expansions, one target over the chip)"),
+        "roofline": simt_roofline(route, (2.0 * it + 1) * n * n, (2.0 * it + 1) * n, timing["apply"], _peaks()),
         "kernel_ms_per_step": {kk: v[0] for kk, v in timing.items()},
         "e2e": {"value": whole_job_rate(B, world, max(1, args.steps), e2e_s), "unit": "problems/s",
                 "h2d_bytes_per_step": (hx.numel() + hD.numel() + hy.numel() + hw.numel()) * 4,

@@ -379,6 +379,19 @@ int otlm_objective(otlm_handle h, int batch, int n, int k,
  * has no counterpart).  NULL handle: -1. */
 long long otlm_launch_count(otlm_handle h);
 
+/* Which kernels the last otlm_solve, otlm_solve_cost or otlm_solve_host on the handle ran (-1 for a
+ * NULL handle). */
+typedef enum {
+  OTLM_ROUTE_NONE       = 0,  /* no solve yet                                                      */
+  OTLM_ROUTE_LOG        = 1,  /* tiled log-domain applies                                          */
+  OTLM_ROUTE_EXPANSION  = 2,  /* FP32 block expansions                                             */
+  OTLM_ROUTE_ONE_LAUNCH = 3,  /* whole solves in one launch, FP32                                  */
+  OTLM_ROUTE_STORED     = 4,  /* FP64 applies of a stored kernel                                   */
+  OTLM_ROUTE_TENSOR     = 5,  /* tensor-core applies                                               */
+  OTLM_ROUTE_DEVICE     = 6   /* block expansions or log-domain applies, as the device found the grid */
+} otlm_route;
+int otlm_solve_route(otlm_handle h);
+
 /* Device-time instrumentation (the paper has no counterpart).  When enabled, every launch a
  * solve or objective call queues is bracketed by two CUDA events on the handle's stream, and
  * the elapsed device time is accumulated per kernel kind: [0] kernel apply (a = K u1 and

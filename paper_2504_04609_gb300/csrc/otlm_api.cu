@@ -31,6 +31,7 @@ struct otlm_ctx {
   void* f64 = nullptr;       // FP64 handles up to n_max = F64_MAX_N: stored kernel and scalings (f64.cuh)
   int* host_flag = nullptr;  // pinned
   long long launches = 0;
+  int route = 0;             // otlm_route of the last solve
   size_t elem = 4;
   otlm::Timer timer;
   bool timer_ready = false;
@@ -120,7 +121,7 @@ int run_solve(otlm_ctx* h, const SolveParams& sp, const void* x, const void* C, 
   otlm::carve_workspace<T>(base, c.n_max, c.k_max, c.batch_max, &ws);
   otlm::ObjWorkspace<T> ow;
   if (lay.obj) otlm::carve_obj_workspace<T>(base + lay.base + lay.tc + lay.mm, c.n_max, c.batch_max, &ow);
-  Launch L{h->stream, &h->launches, h->host_flag, &h->timer};
+  Launch L{h->stream, &h->launches, h->host_flag, &h->timer, &h->route};
   cudaError_t e;
   if (c.precision == OTLM_PREC_BF16_TC) {
     otlm::TcWorkspace tw;
@@ -660,6 +661,11 @@ int otlm_solve_stats(otlm_handle h, int batch, void* dw_out, double* primal_out,
 }
 
 long long otlm_launch_count(otlm_handle h) { return h ? h->launches : -1; }
+static_assert(OTLM_ROUTE_LOG == otlm::ROUTE_LOG && OTLM_ROUTE_EXPANSION == otlm::ROUTE_EXPANSION &&
+                  OTLM_ROUTE_ONE_LAUNCH == otlm::ROUTE_ONE_LAUNCH && OTLM_ROUTE_STORED == otlm::ROUTE_STORED &&
+                  OTLM_ROUTE_TENSOR == otlm::ROUTE_TENSOR && OTLM_ROUTE_DEVICE == otlm::ROUTE_DEVICE,
+              "otlm_route");
+int otlm_solve_route(otlm_handle h) { return h ? h->route : -1; }
 
 int otlm_set_timing(otlm_handle h, int enable) {
   if (!h) return OTLM_EINVAL;

@@ -52,12 +52,18 @@ struct Timer {
   }
 };
 
+enum { ROUTE_NONE = 0, ROUTE_LOG, ROUTE_EXPANSION, ROUTE_ONE_LAUNCH, ROUTE_STORED, ROUTE_TENSOR, ROUTE_DEVICE };
+
 struct Launch {
   cudaStream_t stream;
   long long* counter;
   int* host_flag;  // pinned int used for the convergence polls
   Timer* timer;    // may be null
+  int* route = nullptr;  // the solve's otlm_route (ROUTE_*)
 
+  void took(int r) const {
+    if (route) *route = r;
+  }
   // Bracket one launch: call begin(kind) before and end() after it.
   void begin(int k) const {
     if (timer && timer->on) {
@@ -424,6 +430,7 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
     if constexpr (sizeof(T) == 4) {
       const SmallSolve c{batch, n, k, sp.datafit, sp.penalty, sp.max_iter, sp.mm_steps, sp.eps, sp.lam, sp.alpha, sp.beta,
                          sp.tol, x, D, y, w, g, t_out, iters_out, err_out, status_out, ws.dw};
+      L.took(ROUTE_ONE_LAUNCH);
       L.begin(KIND_APPLY);
       cudaError_t e = small_solve(c, L.stream);
       L.end();
@@ -435,6 +442,7 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
   const bool serves = sizeof(T) == 4 && ex_serves(sp, C != nullptr, checks), prefers = serves && small_prefers(sp, sm_count());
   if (prefers && n <= SMALL_ANY_N) return small();
 
+  L.took(ROUTE_LOG);
   PrepArgs<T> pa;
   pa.x = x; pa.D = D; pa.w_in = w; pa.g_in = g; pa.y = y;
   pa.xt = ws.xt; pa.Dt = ws.Dt; pa.xcol = ws.xcol; pa.W = ws.W; pa.G2 = ws.G2;
@@ -503,12 +511,14 @@ cudaError_t solve_device(const Launch& L, const Workspace<T>& ws, const ObjWorks
         e = ex_iterate(L, ws, sp, D, y, plan.known ? ws.n_active : ex_count_of(ws));
       if (e != cudaSuccess) return e;
       tiles = !plan.known || plan.nb == 0;
+      L.took(!plan.known ? ROUTE_DEVICE : tiles ? ROUTE_LOG : ROUTE_EXPANSION);
     }
   }
   bool linear = false;
   if constexpr (sizeof(T) == 8) {
     linear = f64 && !C && !checks;
     if (linear) {
+      L.took(ROUTE_STORED);
       const int abs_cost = sp.cost == COST_ABS;
       L.begin(KIND_OTHER);
       f64_build_kernel<<<1184, 256, 0, L.stream>>>(ws.xt, n, f64.K, abs_cost);

@@ -865,6 +865,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
     if (e != cudaSuccess) return e;
     by_expansion = plan.nb > 0 && tc_prefers_expansion(batch, n, plan.nb);
     if (plan.nb > 0 && small) {
+      L.took(ROUTE_ONE_LAUNCH);
       const SmallSolve sc{batch, n, k, sp.datafit, sp.penalty, sp.max_iter, sp.mm_steps, sp.eps, sp.lam, sp.alpha, sp.beta,
                           sp.tol, x, D, y, w, g, t_out, iters_out, err_out, status_out, ws.dw};
       L.begin(KIND_APPLY);
@@ -875,6 +876,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
       return e;
     }
   }
+  L.took(by_expansion ? ROUTE_EXPANSION : ROUTE_TENSOR);
   if (!by_expansion) {
   L.begin(KIND_OTHER);
   if (C)

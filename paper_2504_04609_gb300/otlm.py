@@ -26,8 +26,9 @@ EXPORTS = ("otlm_create", "otlm_destroy", "otlm_solve", "otlm_solve_cost", "otlm
            "otlm_tune_ragged", "otlm_ws_create", "otlm_ws_destroy", "otlm_ws_num_params", "otlm_ws_set_normalization",
            "otlm_ws_get_params", "otlm_ws_set_params", "otlm_ws_gradients", "otlm_ws_train_step", "otlm_ws_predict",
            "otlm_ws_make_targets", "otlm_ws_fit_normalization", "otlm_initial_weights", "otlm_solve_stats",
-           "otlm_check_wait_expiry", "otlm_strerror")
+           "otlm_check_wait_expiry", "otlm_solve_route", "otlm_strerror")
 TIMING_KINDS = ("apply", "mm_source", "compact", "other")
+ROUTES = ("none", "log", "expansion", "one launch", "stored", "tensor", "device")  # otlm_route
 COST = {"sq": 0, "abs": 1}  # grid cost (x_i - x_j)^2 or |x_i - x_j| (otlm_cost_kind)
 
 
@@ -69,6 +70,8 @@ def lib() -> ctypes.CDLL:
         L.otlm_objective.restype = i
         L.otlm_launch_count.argtypes = [vp]
         L.otlm_launch_count.restype = ctypes.c_longlong
+        L.otlm_solve_route.argtypes = [vp]
+        L.otlm_solve_route.restype = i
         L.otlm_set_timing.argtypes = [vp, i]
         L.otlm_set_timing.restype = i
         L.otlm_get_timing.argtypes = [vp, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_longlong)]
@@ -179,6 +182,11 @@ class Handle:
     @property
     def launches(self) -> int:
         return lib().otlm_launch_count(self._h)
+
+    @property
+    def route(self) -> str:
+        """otlm_solve_route: which kernels the last shared-grid or dense-cost solve ran (ROUTES)."""
+        return ROUTES[lib().otlm_solve_route(self._h)]
 
     def set_timing(self, enable: bool):
         _check(lib().otlm_set_timing(self._h, int(bool(enable))), "otlm_set_timing")
