@@ -63,22 +63,8 @@ __device__ __forceinline__ float exa_tf32(float x) {
   return __uint_as_float(r);
 }
 
-#ifndef EXA_MINB
-#define EXA_MINB 7
-#endif
-// Sum over the CTA's T warps, the same in every thread.
-template <int T>
-__device__ __forceinline__ float exa_sum(float v, float* red) {
-  if constexpr (T == 1) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-  } else {
-    return block_sum(v, red);
-  }
-}
-
 template <int EPI, bool TC, int T>
-__global__ void __launch_bounds__(32 * T, T == 4 ? EXA_MINB : 1) ex_apply_kernel(ExArgs A) {
+__global__ void __launch_bounds__(32 * T, T == 4 ? 7 : 1) ex_apply_kernel(ExArgs A) {
   using P = Prec<float>;
   constexpr int NT = 32 * T;
   extern __shared__ __align__(16) float smem[];
@@ -107,7 +93,7 @@ __global__ void __launch_bounds__(32 * T, T == 4 ? EXA_MINB : 1) ex_apply_kernel
       mass += s;
     }
     if (TC) {
-      mass = exa_sum<T>(mass, red);
+      mass = block_sum(mass, red);
       if (tid == 0 && prt == 0) A.mass[p] = mass;
     }
   }
@@ -154,7 +140,7 @@ __global__ void __launch_bounds__(32 * T, T == 4 ? EXA_MINB : 1) ex_apply_kernel
   if (EPI == EXA_TARGET || !A.check) return;
 
   // ---- violation of the previous iteration's plan and the stopping decision --------------------
-  part = exa_sum<T>(part, red);
+  part = block_sum(part, red);
   if (parts > 1) {
     if (tid == 0) {
       A.part[o + prt] = part;
@@ -178,8 +164,8 @@ __global__ void __launch_bounds__(32 * T, T == 4 ? EXA_MINB : 1) ex_apply_kernel
       num += fabsf(wv - A.Wprev[(size_t)p * A.k + j]);
       den += fabsf(wv);
     }
-    num = exa_sum<T>(num, red);
-    den = exa_sum<T>(den, red);
+    num = block_sum(num, red);
+    den = block_sum(den, red);
     dw = num / den;
   }
   if (tid == 0) {
@@ -231,12 +217,11 @@ static inline cudaError_t launch_ex_cfg(const ExArgs& a, int batch, int parts, i
   // n = 16384, 20 iterations: 2.43 ms early, 2.23 late)
   return launch_pdl(parts == 1 || a.early, ex_apply_kernel<EPI, TC, T>, dim3(batch, parts), dim3(32 * T), smem, stream, a);
 }
-#ifndef EXA_T1
-#define EXA_T1 4
-#endif
+// Four warps per problem where there are at least four problems per SM (1024 x 1024, in the
+// first version: two, four, eight warps 35, 32, 74 us an apply), else eight and several CTAs per problem.
 template <int EPI, bool TC>
 static inline cudaError_t launch_ex_apply(const ExArgs& a, int batch, int sms, cudaStream_t stream) {
-  if (batch >= 4 * sms && a.n <= 8192) return launch_ex_cfg<EPI, TC, EXA_T1>(a, batch, 1, sms, stream);
+  if (batch >= 4 * sms && a.n <= 8192) return launch_ex_cfg<EPI, TC, 4>(a, batch, 1, sms, stream);
   return launch_ex_cfg<EPI, TC, 8>(a, batch, exa_parts(batch, a.n, sms), sms, stream);
 }
 
@@ -344,8 +329,7 @@ __global__ void __launch_bounds__(MMB_NT) mm_batch_kernel(MMBArgs A) {
               r2[h] = f2_pack(v.x, v.y);
               r2[h + 1] = f2_pack(v.z, v.w);
             }
-          } else if constexpr (PB == 2) r2[0] = f2_pack(rr[0], rr[1]);
-          else r2[0] = f2_pack(rr[0], 0.f);
+          } else r2[0] = f2_pack(rr[0], 0.f);
 #pragma unroll
           for (int q = 0; q < KQ; ++q) {
             const uint64_t d2 = f2_pack(cur[u][q], cur[u][q]);
@@ -424,8 +408,7 @@ __global__ void __launch_bounds__(MMB_NT) mm_batch_kernel(MMBArgs A) {
               w2[h] = f2_pack(v.x, v.y);
               w2[h + 1] = f2_pack(v.z, v.w);
             }
-          } else if constexpr (PB == 2) w2[0] = f2_pack(ww[0], ww[1]);
-          else w2[0] = f2_pack(ww[0], 0.f);
+          } else w2[0] = f2_pack(ww[0], 0.f);
 #pragma unroll
           for (int t = 0; t < IPT; ++t) {
             const uint64_t d2 = f2_pack(d[jj][t], d[jj][t]);
@@ -493,8 +476,11 @@ static inline cudaError_t launch_mmb_pb(const MMBArgs& a, int batch, cudaStream_
   if (a.k <= 128) return launch_mmb_cfg<PB, 4>(a, batch, s);
   return launch_mmb_cfg<PB, 8>(a, batch, s);
 }
-// Problems per CTA: one while the batch does not fill the SMs, then as many as leave two CTAs per SM
-// (latency of the loads of D) and, for the largest batches, eight (traffic of D).
+// Problems per CTA: one up to a problem per SM; then four, which D's reads from L2 serve at once (1024
+// problems, 50 iterations of the FP32 batch: 4.34 ms with eight and 128 CTAs, 4.11 with four and 256), and
+// eight (half the reads of D) once four would leave more than four CTAs per SM.  Lines not measured
+// between: 20 iterations at n = 1024, k = 64 take 1.03 ms for 200 problems, 1.48 for 305, 1.72 for 400, 1.92 for
+// 800, 2.59 for 1600 and 5.28 for 4000.
 static inline cudaError_t launch_mm_batch(const MMBArgs& a, int batch, int sms, cudaStream_t s) {
   if (batch <= sms) return launch_mmb_pb<1>(a, batch, s);
   if (batch <= 16 * sms) return launch_mmb_pb<4>(a, batch, s);

@@ -204,18 +204,11 @@ __device__ __forceinline__ void ex_rows(const float* xt, int i0, int i1, float c
 
 // The apply for row blocks [I0, I1) by the T warps of a CTA: in_s [n] in shared memory (written
 // before the call; the first barrier is here), xt [n] (shared or global), scr = shared scratch, 16-byte
-// aligned, of ex_scratch_floats(T) floats for gr = T or less for gr = ex_round_groups(T, ...).  row(i, pre, base, sum, di2) is called once per row by
-// one thread, with out_i = base + (log2(sum) - di2), base an integer and sum = 0 for an empty (or
-// non-finite) input; pre = load(i) was called before the row's sums, so that what the row's epilogue
-// reads arrives meanwhile.
-//   T = 1 runs a problem in one warp without any block barrier, which is what fills the SMs when
-// there are several problems per SM (the phases of a CTA of eight warps are short against their
-// barriers: 1024 problems of 1024 bins took 74 us that way, see exp_solver.cuh).
-template <int T>
-__device__ __forceinline__ void ex_sync() {
-  if constexpr (T == 1) __syncwarp();
-  else __syncthreads();
-}
+// aligned, of ex_scratch_floats(T) floats for gr = T or less for gr = ex_round_groups(T, ...).
+// row(i, pre, base, sum, di2) is called once per row by one thread, with
+// out_i = base + (log2(sum) - di2), base an integer and sum = 0 for an empty (or non-finite) input;
+// pre = load(i) was called before the row's sums, so that what the row's epilogue reads arrives
+// meanwhile.
 template <int T, class Load, class Row>
 __device__ __forceinline__ void ex_apply(const float* in_s, const float* xt, int n, const ExPlan& pl, int I0, int I1,
                                          float* scr, int gr, Load load, Row row) {
@@ -229,9 +222,9 @@ __device__ __forceinline__ void ex_apply(const float* in_s, const float* xt, int
   float* ref = scr + 2 * EX_NB;
   unsigned* mask_s = reinterpret_cast<unsigned*>(scr + 3 * EX_NB);
   float* cf = scr + EX_HEAD;
-  const int tid = threadIdx.x, lane = tid & 31, warp = T == 1 ? 0 : tid >> 5, nb = pl.nb, b = pl.b;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nb = pl.nb, b = pl.b;
   if (tid < nb) cent[tid] = ex_center(xt, tid, b, n, pl.q);
-  ex_sync<T>();
+  __syncthreads();
   // block maxima of in_j - dj^2, rounded up
   bool bad = false;
   for (int J = warp; J < nb; J += T) {
@@ -247,12 +240,7 @@ __device__ __forceinline__ void ex_apply(const float* in_s, const float* xt, int
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if (lane == 0) amax[J] = ceilf(mx);
   }
-  if constexpr (T == 1) {
-    bad = __any_sync(0xffffffffu, bad);
-    __syncwarp();
-  } else {
-    bad = __syncthreads_or(bad);
-  }
+  bad = __syncthreads_or(bad);
   // which column blocks matter to each row block (bounds over the block pair)
   const float aJ = lane < nb ? amax[lane] : -CUDART_INF_F, cJl = lane < nb ? cent[lane] : 0.f;
   for (int I = I0 + warp; I < I1; I += T) {
@@ -264,7 +252,7 @@ __device__ __forceinline__ void ex_apply(const float* in_s, const float* xt, int
     const unsigned mk = __ballot_sync(0xffffffffu, !bad && lane < nb && aJ > -CUDART_INF_F && top >= low - EX_SKIP);
     if (lane == 0) mask_s[I] = mk;
   }
-  ex_sync<T>();
+  __syncthreads();
   // row blocks go in groups of three or four (equal shares), a round takes up to gr <= T groups
   const int ng = (I1 - I0 + 3) / 4, cpb = (b + 127) / 128, per = ((b + 31) / 32 + cpb - 1) / cpb;
   const bool narrow = b < 256;  // 8 lanes per column block (four at a time) for short blocks
@@ -297,7 +285,7 @@ __device__ __forceinline__ void ex_apply(const float* in_s, const float* xt, int
         else ex_moments<3, 32>(in_s, xt, j0, j1, cJ, a, e2, c, nb, J, G);
       }
     }
-    ex_sync<T>();
+    __syncthreads();
     // coefficients: moments times c_m and the pair's scale relative to the row block's reference
     for (int I = Ia + warp; I < Ib; I += T) {
       const unsigned mk = mask_s[I];
@@ -326,7 +314,7 @@ __device__ __forceinline__ void ex_apply(const float* in_s, const float* xt, int
       }
       if (lane == 0) ref[I] = live ? e : 0.f;
     }
-    ex_sync<T>();
+    __syncthreads();
     // rows: items of up to 128 rows of one block
     for (int t = warp; t < (Ib - Ia) * cpb; t += T) {
       const int I = Ia + t / cpb, r0 = I * b + (t % cpb) * per * 32, i1 = min(n, (I + 1) * b);
@@ -353,7 +341,7 @@ __device__ __forceinline__ void ex_apply(const float* in_s, const float* xt, int
       else if (groups == 2) go(std::integral_constant<int, 2>{});
       else if (groups == 1) go(std::integral_constant<int, 1>{});
     }
-    ex_sync<T>();  // the round's coefficients have been read
+    __syncthreads();  // the round's coefficients have been read
   }
 }
 
