@@ -20,8 +20,8 @@
  *    stream); results are valid once that stream has been synchronised.  The host blocks only
  *    for the short convergence polls that solves make every poll_every iterations; a polling solve
  *    on a squared-distance grid may block once more, before its first iteration, until the kernels
- *    that look the grid over have run.  FP32 solves with poll_every > max_iter never block and can
- *    be captured into a graph.  Tensor-core solves block until they end.
+ *    that look the grid over have run.  FP32 and FP64 solves with poll_every > max_iter never block,
+ *    and FP32 ones can be captured into a graph.  Tensor-core solves block until they end.
  *  - Return value: OTLM_OK (0) or a negative OTLM_E* code; otlm_strerror() names it.  No C++
  *    exception crosses the ABI.  Arguments are validated before any work is queued.
  *  - Potentials: g = eps log u1 (target side), f = eps log u2 (source side).

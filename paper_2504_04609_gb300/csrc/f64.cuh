@@ -13,8 +13,8 @@
 //     most 2^-1074, which a scaling of 2^1000 (transport beyond sqrt(1022 eps ln2)) makes visible; n times
 //     that times the largest scaling is then below 2^-62 of the sum (n <= 4096).
 //   one target, n = 200, k = 10, 500 iterations: 765 ms with log-sum-exp tiles of 4 problems x 128
-//   rows (2 CTAs on 2 SMs), 17 ms now, three launches of 8 to 12 us per iteration whose serial FP64
-//   logarithms are what is left; objective of 16 problems, n = 512: 3.2 ms -> 149 us.
+//   rows (2 CTAs on 2 SMs), 14.2 ms now, three launches of 8 to 12 us per iteration whose serial FP64
+//   logarithms are what is left; objective of 16 problems, n = 512: 3.2 ms -> 144 us.
 #pragma once
 
 #include "kernels.cuh"

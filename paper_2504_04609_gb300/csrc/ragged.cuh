@@ -16,7 +16,7 @@
 // iteration), or an exact max pass when any sum leaves [2^-60, 2^60].
 //
 // 800 problems, n 256..4096, k 8..128, eps 2e-3..5e-2, 20 iterations: 45.4 ms with every apply term by
-// term and row-at-a-time dictionary passes (exponent unit and load latency), 6.6 ms with expansions
+// term and row-at-a-time dictionary passes (exponent unit and load latency), 6.8 ms with expansions
 // and passes that keep 16 loads of D in flight per warp.  What is left is D: 0.6 MB per problem, read
 // twice per iteration, mostly from DRAM.
 #pragma once
