@@ -72,6 +72,7 @@ struct SmallSolve {
   float* err;
   int* status;
   float* dw;
+  int empty_t0 = 0;  // tensor-core handles: t = 0 where the target sum is empty, whatever g is there
 };
 cudaError_t small_solve(const SmallSolve& c, cudaStream_t stream);
 

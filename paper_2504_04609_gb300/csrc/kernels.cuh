@@ -748,6 +748,7 @@ struct FinArgs {
   T* w_out; T* g_out; T* t_out; int* iters_out; int* status_out; T* err_out;
   int batch, n, k;
   T gscale_inv;  // eps ln2
+  int empty_t0 = 0;  // tensor-core handles: t = 0 where the target sum is empty, whatever g is there
 };
 
 // Copy the solver state out: w, g = eps ln2 G2, t = Q^T 1 = 2^(G2 + LB2), per-problem stats.
@@ -781,7 +782,7 @@ __global__ void finalize_kernel(FinArgs<T> A) {
   for (size_t e = tid; e < bk; e += stride) A.w_out[e] = A.W[e];
   for (size_t e = tid; e < bn; e += stride) {
     if (A.g_out) A.g_out[e] = A.G2[e] * A.gscale_inv;
-    if (A.t_out) A.t_out[e] = P::exp2(A.G2[e] + A.LB2[e]);
+    if (A.t_out) A.t_out[e] = A.empty_t0 && !(A.LB2[e] > P::ninf()) ? T(0) : P::exp2(A.G2[e] + A.LB2[e]);
   }
   for (size_t e = tid; e < (size_t)A.batch; e += stride) {
     if (A.iters_out) A.iters_out[e] = A.iters[e];

@@ -289,6 +289,7 @@ cudaError_t small_solve(const SmallSolve& c, cudaStream_t stream) {
   a.datafit = c.datafit; a.penalty = c.penalty; a.max_iter = c.max_iter;
   a.lam = (float)c.lam; a.alpha = (float)c.alpha; a.tol = (float)c.tol; a.beta = (float)c.beta; a.mm_steps = c.mm_steps;
   a.n_all = c.n; a.k_all = c.k; a.eps_all = (float)c.eps; a.xs_all = (float)(1.0 / std::sqrt(c.eps * kLn2));
+  a.empty_t0 = c.empty_t0;
   return ragged_small(a, stream);
 }
 }  // namespace otlm

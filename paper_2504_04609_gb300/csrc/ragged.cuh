@@ -56,6 +56,7 @@ struct RaggedArgs {
   int n_all, k_all;
   float eps_all, xs_all;          // xs_all = 1 / sqrt(eps ln2)
   float* dw;                      // [batch] weight change of the last update, or null
+  int empty_t0;                   // t = 0 where the target sum is empty, whatever g is there
   // rows per thread by size bucket (n in (256 b, 256 (b + 1)]), as log2 R; raised to the fewest
   // that cover n with this CTA size (0: always the fewest)
   unsigned char rows_log2[16];
@@ -468,7 +469,7 @@ __device__ void ragged_solve_one(const RaggedArgs& A, int p, float* sm) {
   for (int j = tid; j < k; j += NT) A.w[ok + j] = W[j];
   for (int i = tid; i < n; i += NT) {
     if (A.g_out) A.g_out[on + i] = G2[i] * eps_ln2;
-    if (A.t_out) A.t_out[on + i] = it > 0 ? P::exp2(G2[i] + LB2[i]) : 0.f;
+    if (A.t_out) A.t_out[on + i] = it > 0 && !(A.empty_t0 && !(LB2[i] > P::ninf())) ? P::exp2(G2[i] + LB2[i]) : 0.f;
   }
   if (A.dw) {  // ||w - w_before||_1 / ||w||_1 of the last update
     float num = 0.f, den = 0.f;

@@ -867,7 +867,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
     if (plan.nb > 0 && small) {
       L.took(ROUTE_ONE_LAUNCH);
       const SmallSolve sc{batch, n, k, sp.datafit, sp.penalty, sp.max_iter, sp.mm_steps, sp.eps, sp.lam, sp.alpha, sp.beta,
-                          sp.tol, x, D, y, w, g, t_out, iters_out, err_out, status_out, ws.dw};
+                          sp.tol, x, D, y, w, g, t_out, iters_out, err_out, status_out, ws.dw, 1};
       L.begin(KIND_APPLY);
       e = small_solve(sc, L.stream);
       L.end();
@@ -1150,6 +1150,7 @@ inline cudaError_t solve_device_tc(const Launch& L, const Workspace<float>& ws, 
   fa.W = ws.W; fa.G2 = ws.G2; fa.LB2 = ws.LB2; fa.iters = ws.iters; fa.status = ws.status; fa.err = ws.err;
   fa.w_out = w; fa.g_out = g; fa.t_out = t_out; fa.iters_out = iters_out; fa.status_out = status_out;
   fa.err_out = err_out; fa.batch = batch; fa.n = n; fa.k = k; fa.gscale_inv = float(eps_ln2);
+  fa.empty_t0 = 1;
   L.begin(KIND_OTHER);
   if (by_expansion) finalize_kernel<float><<<1184, 256, 0, L.stream>>>(fa);
   else tc_finalize_kernel<<<1184, 256, 0, L.stream>>>(fa, ta);
